@@ -13,7 +13,10 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "liblrdmc.so")
 LIB_BOUNDS = os.path.join(HERE, "liblrdmc_bounds.so")
-SOURCES = ["lrdmc_kernels.cu", "lrdmc_api.cu", "lrdmc_neural.cu"]
+# translation units: source and its extra flags (the kernel file's parts
+# compile its variants in parallel)
+SOURCES = [("lrdmc_kernels.cu", [f"-DLRDMC_PART={part}"]) for part in (1, 2, 3, 4, 5, 6, 0)] + \
+    [("lrdmc_api.cu", []), ("lrdmc_neural.cu", [])]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
@@ -49,9 +52,11 @@ def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> s
     if bounds:
         extra.append("-DLRDMC_BOUNDS")
 
-    def compile_one(src):
-        obj = os.path.join(build_dir, os.path.splitext(src)[0] + ".o")
-        cmd = [nvcc, *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit):
+        src, flags = unit
+        tag = "".join(f.rsplit("=", 1)[-1] for f in flags)
+        obj = os.path.join(build_dir, os.path.splitext(src)[0] + tag + ".o")
+        cmd = [nvcc, *ARCH, *FLAGS, *extra, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")

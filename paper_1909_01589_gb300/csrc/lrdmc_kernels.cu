@@ -34,6 +34,13 @@
 #include "lrdmc_internal.h"
 #include "mixed_arith.cuh"
 
+// This file is compiled several times, so that the kernel variants build in
+// parallel: part 0 holds the kernels without variants and every host entry,
+// parts 1.. instantiate the variants listed at the end of the file.
+#ifndef LRDMC_PART
+#define LRDMC_PART 0
+#endif
+
 namespace lrdmc {
 
 #define FULL_MASK 0xffffffffu
@@ -122,7 +129,7 @@ __device__ __forceinline__ uint64_t shfl_u64(uint64_t v, int src)
 }
 
 // Uniformly random rotation (Shoemake's unit quaternion from three uniforms).
-__device__ void rotation_matrix(double u1, double u2, double u3, double* R)
+static __device__ void rotation_matrix(double u1, double u2, double u3, double* R)
 {
   double s1 = sqrt(1.0 - u1), s2 = sqrt(u1);
   double sa, ca, sb, cb;
@@ -247,7 +254,7 @@ __device__ __forceinline__ double warp_sum(double v)
 // Returns the total (identical in every lane). When pick != nullptr, *pick
 // receives the smallest c with target < C_c (or -1), and *last the largest c
 // with T_c > 0 (or -1).
-__device__ double warp_scan(const double* T, int P, int lane, double target, int* pick, int* last)
+static __device__ double warp_scan(const double* T, int P, int lane, double target, int* pick, int* last)
 {
   double carry = 0.0;
   int p = -1, lp = -1;
@@ -346,7 +353,7 @@ __device__ __forceinline__ int solid(int l, const double d[3], double S[5], doub
 
 // Sum_mu v[mu] chi_mu(p): the determinant ratio when v is the projected
 // inverse column of the moving electron.
-__device__ double ao_dot(const SysDev& S, const double* v, double px, double py, double pz)
+static __device__ double ao_dot(const SysDev& S, const double* v, double px, double py, double pz)
 {
   double acc = 0.0;
   int prev_c = -1;
@@ -372,7 +379,7 @@ __device__ double ao_dot(const SysDev& S, const double* v, double px, double py,
 }
 
 // Sum_mu v[mu] chi_mu, grad chi_mu, lap chi_mu at p.
-__device__ void ao_dot_der(const SysDev& S, const double* v, const double* p, double& val,
+static __device__ void ao_dot_der(const SysDev& S, const double* v, const double* p, double& val,
                            double g[3], double& lap)
 {
   val = 0.0; g[0] = g[1] = g[2] = 0.0; lap = 0.0;
@@ -403,7 +410,7 @@ __device__ void ao_dot_der(const SysDev& S, const double* v, const double* p, do
 }
 
 // chi_mu(p) for all AOs into out[n_ao].
-__device__ void ao_values(const SysDev& S, const double* p, double* out)
+static __device__ void ao_values(const SysDev& S, const double* p, double* out)
 {
   int prev_c = -1;
   double d[3] = {0, 0, 0}, r = 0.0, e = 0.0;
@@ -585,7 +592,7 @@ __device__ __forceinline__ BlockMem block_mem(const SysDev& S, double* smem)
 // delta_lq| over the block, where A is the Slater matrix at the current
 // positions; *resid becomes the larger of itself and that residual (the
 // same value in every lane).
-__device__ LRDMC_COLD bool warp_inverse(const SysDev& S, const double* sC, const double* sx, int spin,
+static __device__ LRDMC_COLD bool warp_inverse(const SysDev& S, const double* sC, const double* sx, int spin,
                              double* Ainv, double* scr, int lane, double* resid = nullptr)
 {
   const int n = spin == 0 ? S.n_up : S.n_dn;
@@ -1591,7 +1598,7 @@ __device__ __forceinline__ void warp_eval_any(const SysDev& S, const double* sC,
 // ----------------------------------------------------------------------------
 // chi_mu(p) for all AOs in double-float, one lane per shell, written back
 // as doubles.
-__device__ void ao_values_df_lanes(const SysDev& S, const double* p, double* out, int lane, const BlockMem& bm)
+static __device__ void ao_values_df_lanes(const SysDev& S, const double* p, double* out, int lane, const BlockMem& bm)
 {
   typedef Ar<df> A;
   df pd[3] = {df_from_double(p[0]), df_from_double(p[1]), df_from_double(p[2])};
@@ -1616,7 +1623,7 @@ __device__ void ao_values_df_lanes(const SysDev& S, const double* p, double* out
 }
 
 // chi_mu(p) for all AOs in double-float into out (df), one lane per shell.
-__device__ void ao_values_df_out(const SysDev& S, const df* pd, df* out, int lane, const BlockMem& bm)
+static __device__ void ao_values_df_out(const SysDev& S, const df* pd, df* out, int lane, const BlockMem& bm)
 {
   typedef Ar<df> A;
   // one shell per lane (at most 32 shells), each with its own centre
@@ -1643,7 +1650,7 @@ __device__ void ao_values_df_out(const SysDev& S, const df* pd, df* out, int lan
 // orbitals at the new position, y = phi A^-1, ratio = y_l, and
 // the rank-one update, with the spin block read from and written back to
 // its IEEE-double copy. pd: the new position as a double-float.
-__device__ LRDMC_JUMP bool warp_sm_update_df(const SysDev& S, const BlockMem& bm, const WarpMem& wm, int i, const df* pd,
+static __device__ LRDMC_JUMP bool warp_sm_update_df(const SysDev& S, const BlockMem& bm, const WarpMem& wm, int i, const df* pd,
                                   int lane)
 {
   const int nu = S.n_up;
@@ -1762,6 +1769,7 @@ __device__ __forceinline__ void stage_coefficients(const SysDev& S, double* sC)
 // ----------------------------------------------------------------------------
 // Kernels.
 // ----------------------------------------------------------------------------
+#if LRDMC_PART == 0
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 k_init(const __grid_constant__ SysDev S, const Layout Lo, const PopDev P, const double* x0)
 {
@@ -1787,6 +1795,8 @@ k_init(const __grid_constant__ SysDev S, const Layout Lo, const PopDev P, const 
   }
   store_record(Lo, P.rec_src + (size_t)s * Lo.rec, wm, lane, NAN, NAN);
 }
+
+#endif  // LRDMC_PART == 0
 
 template <int PREC>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
@@ -1969,7 +1979,7 @@ __device__ __forceinline__ int team_wait_publication(TeamSlot* t, int kidx, int 
   return g;
 }
 
-__shared__ TeamSlot g_team[kMaxIntervalWarps];
+static __shared__ TeamSlot g_team[kMaxIntervalWarps];
 
 // Per-warp state of the interval loop that the move code does not need: it
 // lives in shared memory (written by lane 0, read by the whole warp after a
@@ -1982,7 +1992,7 @@ struct WarpState {
   int s, jumps, finish;
   int owner, kidx, last;
 };
-__shared__ WarpState g_ws[kMaxIntervalWarps];
+static __shared__ WarpState g_ws[kMaxIntervalWarps];
 
 // The interval loop of the FP32-pipe evaluations (double-float and FP32):
 // each warp is an owner while it runs a walker (the same steps, draws and
@@ -2358,6 +2368,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
   if (threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+#if LRDMC_PART == 0
 // Reconfiguration at the end of interval k, spread over G blocks of
 // kCombThreads threads; block g owns the R = ceil(W/G) slots from g R. Its
 // FP64 work (running sums, comb targets and comparisons) used to run on one
@@ -2661,6 +2672,7 @@ __global__ void __launch_bounds__(kCombThreads) k_comb_parents(const PopDev P, c
     }
   }
 }
+#endif  // LRDMC_PART == 0
 
 // Stateless evaluation of configuration c (one warp): inverses from x, then
 // one evaluation of every lattice move and of the local energy. Returns
@@ -2717,6 +2729,7 @@ k_evaluate(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, in
 // ----------------------------------------------------------------------------
 // Host launchers.
 // ----------------------------------------------------------------------------
+#if LRDMC_PART == 0
 static df split_ld(long double x)
 {
   float h = (float)x;
@@ -2810,12 +2823,15 @@ Layout make_layout(const SysDev& S, bool caches)
   return Lo;
 }
 
+#endif  // LRDMC_PART == 0
+
 static cudaError_t set_smem(const void* fn, int bytes)
 {
   if (bytes > 48 * 1024) return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return cudaSuccess;
 }
 
+#if LRDMC_PART == 0
 cudaError_t launch_init(const SysDev& S, const Layout& Lo, const PopDev& P, const double* x0,
                         cudaStream_t st)
 {
@@ -2825,6 +2841,8 @@ cudaError_t launch_init(const SysDev& S, const Layout& Lo, const PopDev& P, cons
   k_init<<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, P, x0);
   return cudaGetLastError();
 }
+
+#endif  // LRDMC_PART == 0
 
 // Kernel variant of a system: the arithmetic in bits 0-1 of the template
 // argument, bit 2 for a double-float system whose layout has no evaluation
@@ -2852,7 +2870,7 @@ constexpr int kNjBit = 8;
   } while (0)
 
 template <int PREC>
-static cudaError_t launch_eval_all_t(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
+cudaError_t launch_eval_all_t(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
                                      cudaStream_t st)
 {
   cudaError_t e = set_smem((const void*)k_eval_all<PREC>, Lo.smem_block_bytes);
@@ -2860,13 +2878,6 @@ static cudaError_t launch_eval_all_t(const SysDev& S, const Layout& Lo, const La
   int blocks = (P.W + kWarpsPerBlock - 1) / kWarpsPerBlock;
   k_eval_all<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, P);
   return cudaGetLastError();
-}
-
-cudaError_t launch_eval_all(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
-                            cudaStream_t st)
-{
-  LRDMC_DISPATCH(S, Lo, return launch_eval_all_t<V>(S, Lo, L, P, st));
-  return cudaErrorInvalidValue;
 }
 
 static int sm_count_current()
@@ -2878,27 +2889,13 @@ static int sm_count_current()
   return n;
 }
 
-// Warps per block of the interval kernel: 16 (so that the warps of an SM,
-// one block, can help one another at the end of an interval), halved while
-// the population cannot give every warp of every SM a walker or the block's
-// shared memory does not fit; at least the other kernels' four.
-int interval_warps(const Layout& Lo, int W)
-{
-  const int sms = sm_count_current();
-  int w = kMaxIntervalWarps;
-  while (w > kWarpsPerBlock &&
-         ((int)sizeof(double) * (Lo.head + w * Lo.smem_warp) > kMaxSmemBlock || W < sms * w))
-    w >>= 1;
-  return w;
-}
-
 static int interval_smem(const Layout& Lo, int w) { return (int)sizeof(double) * (Lo.head + w * Lo.smem_warp); }
 
 // Persistent grid of the interval kernel: as many blocks as fit on the GPU
 // at once (occupancy for this system's shared memory), at most one warp per
 // walker.
 template <int PREC>
-static cudaError_t interval_occupancy(const Layout& Lo, int w, int* blocks)
+cudaError_t interval_occupancy(const Layout& Lo, int w, int* blocks)
 {
   int per_sm = 0;
   cudaError_t e = set_smem((const void*)k_interval<PREC>, interval_smem(Lo, w));
@@ -2908,16 +2905,8 @@ static cudaError_t interval_occupancy(const Layout& Lo, int w, int* blocks)
   return e;
 }
 
-int interval_default_blocks(const SysDev& S, const Layout& Lo, int W)
-{
-  int b = 0;
-  const int w = interval_warps(Lo, W);
-  LRDMC_DISPATCH(S, Lo, interval_occupancy<V>(Lo, w, &b));
-  return b;
-}
-
 template <int PREC>
-static cudaError_t launch_interval_t(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
+cudaError_t launch_interval_t(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
                                      int blocks, int carveout, bool pdl, cudaStream_t st)
 {
   static int cached_blocks = -1, cached_smem = -1;
@@ -2964,6 +2953,120 @@ static cudaError_t launch_interval_t(const SysDev& S, const Layout& Lo, const La
   cfg.attrs = attr;
   cfg.numAttrs = na;
   return cudaLaunchKernelEx(&cfg, k_interval<PREC>, S, Lo, L, P);
+}
+
+template <int PREC>
+cudaError_t launch_evaluate_t(const SysDev& S, const Layout& Lo, const LatDev& L, int n, const double* x,
+                                     const double* rot, double* ratio, double* T, double* b, double* el, int* err,
+                                     cudaStream_t st)
+{
+  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
+  cudaError_t e = set_smem((const void*)k_evaluate<PREC>, Lo.smem_block_bytes);
+  if (e != cudaSuccess) return e;
+  k_evaluate<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio, T, b, el,
+                                                                            err);
+  return cudaGetLastError();
+}
+
+template <int PREC>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+k_evaluate_static(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n,
+                  const double* x, const double* rot, double* ratio, double* T, double* b_out,
+                  double* el_out, int* scratch)
+{
+  extern __shared__ double smem[];
+  double* sC = smem;
+  stage_coefficients(S, sC);
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int c = blockIdx.x * kWarpsPerBlock + wib;
+  if (c >= n) return;
+  // word 64 + c: status of configuration c; word 0: OR of all statuses
+  if (!evaluate_config<PREC>(S, Lo, L, sC, c, lane, wib, x, rot, ratio, T, b_out, el_out) && lane == 0) {
+    scratch[64 + c] = kErrSingular;
+    atomicOr(&scratch[0], kErrSingular);
+  }
+}
+
+template <int PREC>
+cudaError_t launch_evaluate_static_t(const SysDev& S, const Layout& Lo, const LatDev& L, int n, const double* x,
+                                     const double* rot, double* ratio, double* T, double* b, double* el,
+                                     int* scratch, cudaStream_t st)
+{
+  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
+  cudaError_t e = set_smem((const void*)k_evaluate_static<PREC>, Lo.smem_block_bytes);
+  if (e != cudaSuccess) return e;
+  if (blocks > 0)
+    k_evaluate_static<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio, T,
+                                                                                     b, el, scratch);
+  return cudaGetLastError();
+}
+
+// The variants and the part that compiles each.
+#define LRDMC_VARIANT(KEYWORD, V)                                                                                  \
+  KEYWORD template cudaError_t launch_eval_all_t<V>(const SysDev&, const Layout&, const LatDev&, const PopDev&,    \
+                                                    cudaStream_t);                                                 \
+  KEYWORD template cudaError_t interval_occupancy<V>(const Layout&, int, int*);                                    \
+  KEYWORD template cudaError_t launch_interval_t<V>(const SysDev&, const Layout&, const LatDev&, const PopDev&,    \
+                                                    int, int, bool, cudaStream_t);                                 \
+  KEYWORD template cudaError_t launch_evaluate_t<V>(const SysDev&, const Layout&, const LatDev&, int,              \
+                                                    const double*, const double*, double*, double*, double*,       \
+                                                    double*, int*, cudaStream_t);                                  \
+  KEYWORD template cudaError_t launch_evaluate_static_t<V>(const SysDev&, const Layout&, const LatDev&, int,       \
+                                                           const double*, const double*, double*, double*,         \
+                                                           double*, double*, int*, cudaStream_t);
+#if LRDMC_PART == 0
+LRDMC_VARIANT(extern, LRDMC_PRECISION_DF64)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_DF64 | kNjBit)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_DF64 | kNoCacheBit)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_DF64 | kNoCacheBit | kNjBit)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_FP32)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_FP32 | kNjBit)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_FP64)
+LRDMC_VARIANT(extern, LRDMC_PRECISION_FP64 | kNjBit)
+#elif LRDMC_PART == 1
+LRDMC_VARIANT(, LRDMC_PRECISION_DF64)
+#elif LRDMC_PART == 2
+LRDMC_VARIANT(, LRDMC_PRECISION_DF64 | kNjBit)
+#elif LRDMC_PART == 3
+LRDMC_VARIANT(, LRDMC_PRECISION_DF64 | kNoCacheBit)
+#elif LRDMC_PART == 4
+LRDMC_VARIANT(, LRDMC_PRECISION_DF64 | kNoCacheBit | kNjBit)
+#elif LRDMC_PART == 5
+LRDMC_VARIANT(, LRDMC_PRECISION_FP32)
+LRDMC_VARIANT(, LRDMC_PRECISION_FP32 | kNjBit)
+#elif LRDMC_PART == 6
+LRDMC_VARIANT(, LRDMC_PRECISION_FP64)
+LRDMC_VARIANT(, LRDMC_PRECISION_FP64 | kNjBit)
+#endif
+
+#if LRDMC_PART == 0
+cudaError_t launch_eval_all(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
+                            cudaStream_t st)
+{
+  LRDMC_DISPATCH(S, Lo, return launch_eval_all_t<V>(S, Lo, L, P, st));
+  return cudaErrorInvalidValue;
+}
+
+// Warps per block of the interval kernel: 16 (so that the warps of an SM,
+// one block, can help one another at the end of an interval), halved while
+// the population cannot give every warp of every SM a walker or the block's
+// shared memory does not fit; at least the other kernels' four.
+int interval_warps(const Layout& Lo, int W)
+{
+  const int sms = sm_count_current();
+  int w = kMaxIntervalWarps;
+  while (w > kWarpsPerBlock &&
+         ((int)sizeof(double) * (Lo.head + w * Lo.smem_warp) > kMaxSmemBlock || W < sms * w))
+    w >>= 1;
+  return w;
+}
+
+int interval_default_blocks(const SysDev& S, const Layout& Lo, int W)
+{
+  int b = 0;
+  const int w = interval_warps(Lo, W);
+  LRDMC_DISPATCH(S, Lo, interval_occupancy<V>(Lo, w, &b));
+  return b;
 }
 
 cudaError_t launch_interval(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P, int blocks,
@@ -3048,19 +3151,6 @@ cudaError_t launch_base_terms(const SysDev& S, const Layout& Lo, int n, const do
   if (e != cudaSuccess) return e;
   const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
   k_base_terms<<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, n, x, grad, e_out, err);
-  return cudaGetLastError();
-}
-
-template <int PREC>
-static cudaError_t launch_evaluate_t(const SysDev& S, const Layout& Lo, const LatDev& L, int n, const double* x,
-                                     const double* rot, double* ratio, double* T, double* b, double* el, int* err,
-                                     cudaStream_t st)
-{
-  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  cudaError_t e = set_smem((const void*)k_evaluate<PREC>, Lo.smem_block_bytes);
-  if (e != cudaSuccess) return e;
-  k_evaluate<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio, T, b, el,
-                                                                            err);
   return cudaGetLastError();
 }
 
@@ -3455,25 +3545,6 @@ cudaError_t launch_evaluate_tc(const SysDev& S, const Layout& Lo, const LatDev& 
 // ----------------------------------------------------------------------------
 static __device__ __align__(256) int g_eval_scratch[64 + LRDMC_STATIC_EVAL_MAX];
 
-template <int PREC>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-k_evaluate_static(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n,
-                  const double* x, const double* rot, double* ratio, double* T, double* b_out,
-                  double* el_out, int* scratch)
-{
-  extern __shared__ double smem[];
-  double* sC = smem;
-  stage_coefficients(S, sC);
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int c = blockIdx.x * kWarpsPerBlock + wib;
-  if (c >= n) return;
-  // word 64 + c: status of configuration c; word 0: OR of all statuses
-  if (!evaluate_config<PREC>(S, Lo, L, sC, c, lane, wib, x, rot, ratio, T, b_out, el_out) && lane == 0) {
-    scratch[64 + c] = kErrSingular;
-    atomicOr(&scratch[0], kErrSingular);
-  }
-}
-
 // Device address of g_eval_scratch, looked up once per device with that
 // device current (host code must not pass the symbol itself: in host code
 // it names a host-side stand-in, not device memory).
@@ -3509,15 +3580,7 @@ cudaError_t launch_evaluate_static(const SysDev& S, const Layout& Lo, const LatD
   // the summary word and the statuses of this call start at zero
   e = cudaMemsetAsync(scratch, 0, sizeof(int) * (64 + (size_t)n), st);
   if (e != cudaSuccess) return e;
-  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  LRDMC_DISPATCH(S, Lo, {
-    e = set_smem((const void*)k_evaluate_static<V>, Lo.smem_block_bytes);
-    if (e != cudaSuccess) return e;
-    if (blocks > 0)
-      k_evaluate_static<V><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio,
-                                                                                    T, b, el, scratch);
-  });
-  e = cudaGetLastError();
+  LRDMC_DISPATCH(S, Lo, e = launch_evaluate_static_t<V>(S, Lo, L, n, x, rot, ratio, T, b, el, scratch, st));
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(summary, scratch, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -3538,5 +3601,7 @@ cudaError_t launch_evaluate_static(const SysDev& S, const Layout& Lo, const LatD
   }
   return cudaSuccess;
 }
+
+#endif  // LRDMC_PART == 0
 
 }  // namespace lrdmc
