@@ -192,6 +192,12 @@ struct ExpConsts {
   float pad;
 };
 
+// The same for a table of 2^(j/1024) (lean64.cuh): ln2/1024 in two floats
+// and its reciprocal.
+struct LeanExp {
+  float c_hi, c_lo, inv;
+};
+
 // Table of 2^(j/64), j = 0..63, as double-floats (x = hi, y = lo).
 struct ExpTable {
   ExpConsts K;

@@ -382,6 +382,8 @@ lrdmc_status lrdmc_create_system(int n_nuc, const double* nuc_xyz, const double*
       sh.alpha[p] = in.alpha[p];
       sh.coef[p] = in.coef[p];
     }
+    sh.prim_begin = S.n_prim;
+    S.n_prim += sh.n_prim;
     const lrdmc_shell* prev = qs > 0 ? &shells[order[qs - 1]] : nullptr;
     sh.same_exp = (prev && in.kind == 0 && prev->kind == 0 && prev->center == in.center && prev->zeta == in.zeta)
                       ? 1 : 0;
@@ -399,6 +401,27 @@ lrdmc_status lrdmc_create_system(int n_nuc, const double* nuc_xyz, const double*
   for (int qs = 0; qs < n_shells; ++qs)
     if (n_shells <= el_parts || !(S.sh[qs].kind == 0 && S.sh[qs].same_exp)) S.grp_first[S.n_grp++] = qs;
   S.grp_first[S.n_grp] = n_shells;
+  // the double-float mode: one pass over the electrons up to N = 16 (32 / N
+  // lanes each); beyond, as many passes as make the most of the lanes, the
+  // work of a pass being 1 / el_L of an electron's plus a fixed part
+  // (combining the lanes' sums) of about 0.15
+  double best_cost = 1e300;
+  for (int passes = 1; passes <= S.N; ++passes) {
+    const int E = (S.N + passes - 1) / passes;
+    if (E > 32) continue;
+    const double cost = passes * (1.0 / (32 / E) + 0.15);
+    if (cost < best_cost) {
+      best_cost = cost;
+      S.el_E = E;
+      S.el_L = 32 / E;
+    }
+  }
+  S.el_top = 1;
+  while (2 * S.el_top < S.el_L) S.el_top *= 2;
+  S.n_grp64 = 0;
+  for (int qs = 0; qs < n_shells; ++qs)
+    if (n_shells <= S.el_L || !(S.sh[qs].kind == 0 && S.sh[qs].same_exp)) S.grp64_first[S.n_grp64++] = qs;
+  S.grp64_first[S.n_grp64] = n_shells;
   for (int qs = 0; qs < n_shells; ++qs) {
     const int q = order[qs];
     for (int f = 0; f < 2 * shells[q].l + 1; ++f)
@@ -412,10 +435,10 @@ lrdmc_status lrdmc_create_system(int n_nuc, const double* nuc_xyz, const double*
   // that does not fit even then is rejected
   s->Lo = make_layout(S, true);
   if (s->Lo.smem_block_bytes > kMaxSmemBlock) s->Lo = make_layout(S, false);
-  if (s->Lo.smem_block_bytes > kMaxSmemBlock) {
+  if (accept_smem_bytes(S, false) > kMaxSmemBlock || s->Lo.smem_block_bytes > kMaxSmemBlock) {
     static std::string msg;
     msg = "create_system: " + std::to_string(S.N) + " electrons with " + std::to_string(n_ao) +
-          " AOs need " + std::to_string(s->Lo.smem_block_bytes / 1024) + " KB of shared memory per block of " +
+          " AOs need " + std::to_string(accept_smem_bytes(S, false) / 1024) + " KB of shared memory per block of " +
           std::to_string(kWarpsPerBlock) + " walkers (at most " + std::to_string(kMaxSmemBlock / 1024) + " KB)";
     g_static_error = msg.c_str();
     delete s;

@@ -67,7 +67,7 @@ struct ShellDev {
   int ao_offset;
   int m_int;       // Slater power r^m as an integer (>= 0), or -1 for pow()
   int same_exp;    // 1: same centre and Slater exponent as the previous shell
-  int pad;
+  int prim_begin;  // first primitive among those of all Gaussian shells
   double m;        // n_eff - 1 - l
   double zeta;
   double alpha[kMaxPrim];
@@ -90,6 +90,11 @@ struct DfSys {
   ExpTable exp;
   df inv_fact[18];  // 1/k!, k = 0..17 (series of sin and cos)
   df half_pi;
+  LeanExp lexp;
+  // e-e part of the double-float evaluation: its lengths are scaled by
+  // ee_scale = |b| (1 for b = 0); ee_factor turns the sums it compares into
+  // the Jastrow exponent (-1/b in the reciprocal form, 1/scale in the other)
+  df ee_scale, ee_scale2, ee_iscale, ee_factor;
 };
 
 // Trial function and Hamiltonian constants, passed by value as a kernel
@@ -113,6 +118,14 @@ struct SysDev {
   // (a shell with same_exp joins the group of the shell before it)
   int n_grp;
   int grp_first[kMaxShell + 1];
+  // the same for the double-float mode, which takes el_E electrons at a time
+  // with el_L lanes each (el_top: the largest power of two below el_L)
+  int el_E, el_L, el_top;
+  int n_grp64;
+  int grp64_first[kMaxShell + 1];
+  int n_prim;       // primitives of all Gaussian shells
+  int ee_recip;     // 1: the e-e Pade sum in the reciprocal form (b >= 1/4)
+  float ee_sign;    // sign of b (0 for b = 0)
   double C[kMaxAO * kMaxMO];  // [n_ao][n_mo]
   int precision;  // LRDMC_PRECISION_FP64 or LRDMC_PRECISION_DF64
   // neural pair term of the Jastrow factor, tabulated: channel c, cell k
@@ -149,14 +162,27 @@ struct Layout {
   int head;       // doubles of shared memory per block before the warp regions
   int smem_warp;  // doubles of shared memory per warp
   int smem_block_bytes;
-  int n_pc;       // electron pairs with a cached distance and projections (0: no cache)
-  int pcw;        // double-floats per cached pair: 4 (distance, projections) or 8 (+ Jastrow pair terms)
+  int n_scr;      // doubles of scratch per warp (shared with the evaluation's state)
+  int n_pc;       // electron pairs with a cached distance (0: no cache)
   int enc;        // 1: the electron-nucleus cache (and the pair cache, if any) is in the layout
 };
 
 // Shared-memory layout of a system; caches = false leaves out the
 // evaluation caches (for systems that would not fit otherwise).
 Layout make_layout(const SysDev& S, bool caches);
+// Shared memory that decides what a system is accepted for: four walkers'
+// state, evaluation buffers (with or without caches) and scratch side by
+// side. The layout in use overlays them and needs less.
+int accept_smem_bytes(const SysDev& S, bool caches);
+// Entries of the double-float exponential's table, and the offset (doubles)
+// of the double-float evaluation's tables in a block's shared memory.
+constexpr int kExpBits = 10;
+constexpr int kExpEntries = 1 << kExpBits;
+__host__ __device__ inline int lean_offset(const SysDev& S)
+{
+  const int nc = S.n_ao * S.n_mo;
+  return (2 * nc + (nc + 1) / 2 + 64 + 1) & ~1;
+}
 // Largest dynamic shared memory of one block on sm_100-class GPUs (227 KB),
 // less 2 KB for the kernels' static shared memory (the interval kernel's
 // per-warp loop state and tail-helper slots, 1.7 KB).

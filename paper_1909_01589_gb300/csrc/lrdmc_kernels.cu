@@ -145,8 +145,8 @@ static __device__ void rotation_matrix(double u1, double u2, double u3, double* 
 // spread over the warp: lanes 0-3 evaluate sqrt(1-u1), sqrt(u1),
 // sincospi(2 u2) and sincospi(2 u3), lanes 0-8 then form one entry of R
 // each. FP64 mode: IEEE double (the same operations as rotation_matrix).
-// DF64 mode: double-float (the FP32 pipe), accurate to ~1e-15. FP32 mode:
-// single precision. All lanes must call it; R (double) goes to shared memory.
+// FP32 mode: single precision. (The double-float mode: rotation64.) All
+// lanes must call it; R (double) goes to shared memory.
 template <int PREC>
 __device__ LRDMC_JUMP_INLINE void rotation_matrix_warp(const uint64_t* bits, double* R, int lane, const SysDev& S)
 {
@@ -175,40 +175,6 @@ __device__ LRDMC_JUMP_INLINE void rotation_matrix_warp(const uint64_t* bits, dou
       default: break;
     }
     if (lane < 9) R[lane] = (double)v;
-    return;
-  }
-  if (PREC == LRDMC_PRECISION_DF64) {
-    // lanes 0 and 1: sqrt(1 - u1) and sqrt(u1); lanes 2 and 3: sincospi of
-    // 2 u2 and 2 u3 - one pass each, the operand chosen per lane
-    df a = df_make(0.0f, 0.0f), c = df_make(0.0f, 0.0f);
-    if (lane < 2) {
-      const df u = df_u01(bits[0]);
-      a = df_sqrt(lane == 0 ? df_add_f(df_neg(u), 1.0f) : u);
-    } else if (lane < 4) {
-      df_sincospi(df_mul_f(df_u01(bits[lane - 1]), 2.0f), S.D.inv_fact, S.D.half_pi, &a, &c);
-    }
-    typedef Ar<df> A;
-    df s1 = A::shfl(a, 0), s2 = A::shfl(a, 1), sa = A::shfl(a, 2), ca = A::shfl(c, 2);
-    df sb = A::shfl(a, 3), cb = A::shfl(c, 3);
-    const df q[4] = {df_mul(s1, sa), df_mul(s1, ca), df_mul(s2, sb), df_mul(s2, cb)};  // x, y, z, w
-    // entry (row, col) = lane: delta + 2 (s1 q[a] q[b] + s2 q[c] q[d]); the
-    // operand indices and signs of the nine entries, packed per lane
-    //   R00 = 1 - 2(yy + zz)  R01 = 2(xy - zw)  R02 = 2(xz + yw)
-    //   R10 = 2(xy + zw)  R11 = 1 - 2(xx + zz)  R12 = 2(yz - xw)
-    //   R20 = 2(xz - yw)  R21 = 2(yz + xw)  R22 = 1 - 2(xx + yy)
-    const int L = lane < 9 ? lane : 0;
-    const unsigned long long ka = 0x10100001ull, kb = 0x22201211ull;
-    const unsigned long long kc = 0x101022122ull, kd = 0x133323332ull;
-    const unsigned ia = (ka >> (4 * L)) & 0xF, ib = (kb >> (4 * L)) & 0xF;
-    const unsigned ic = (kc >> (4 * L)) & 0xF, id = (kd >> (4 * L)) & 0xF;
-    const bool diag = L == 0 || L == 4 || L == 8;
-    const bool minus2 = L == 1 || L == 5 || L == 6;
-    auto pick = [&](unsigned k) { return k == 0 ? q[0] : k == 1 ? q[1] : k == 2 ? q[2] : q[3]; };
-    df t1 = df_mul(pick(ia), pick(ib)), t2 = df_mul(pick(ic), pick(id));
-    df v;
-    if (diag) v = df_add_f(df_mul_f(df_add(t1, t2), -2.0f), 1.0f);
-    else v = df_mul_f(minus2 ? df_sub(t1, t2) : df_add(t1, t2), 2.0f);
-    if (lane < 9) R[lane] = df_to_double(v);
     return;
   }
   {
@@ -524,18 +490,23 @@ struct WarpMem {
   double* A;    // inverse up [nu][nu] then down [nd][nd]
   double* R;    // [9]
   double* T;    // [P_max]
+  double* sm;   // [4 + n_ao + 3 nu] Sherman-Morrison scratch of the double-float mode
+  // the evaluation's state; scr is scratch over the same storage (the
+  // inverse and the other modes' Sherman-Morrison updates, which run while
+  // no evaluation's state is needed)
   double* v;    // [N][n_ao]
   double* Ssum; // [N]
-  df* xd;       // [N][3]      double-float copies for the DF64 evaluation
+  df* xd;       // [N][3]      double-float copies for the FP32-pipe evaluations
   df* vd;       // [N][n_ao]   (aliases v)
-  df* Sd;       // [N]         (aliases Ssum)
+  df* Sd;       // [N]         (aliases Ssum) Jastrow sums; double-float mode: the e-e sums
+  df* Sn;       // [N]         double-float mode: the e-n sums (and the neural term)
+  df* y;        // [N][3]      double-float mode: positions on the rotated axes, scaled
   df* Rd;       // [12]
-  df* pc;       // [n_pc][pcw] pair cache: |r_a - r_b|^2, e_k . (r_a - r_b) (a < b) and, with
-                //   pcw = 8, the pair's Jastrow terms u, u'/r, u'' + 2u'/r and 1/r
+  df* pfx;      // [32]        double-float mode: running sums of the rates
   df* enc;      // [N][n_nuc][8] electron-nucleus cache: d, |d|^2, e_k . d
-  double* scr;  // scratch
+  df* pc;       // [n_pc] squared distances of the electron pairs, scaled
+  double* scr;
   int n_pc;     // pairs in the cache (0: no cache)
-  int pcw;      // double-floats per cached pair
 };
 
 __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, double* base)
@@ -545,20 +516,23 @@ __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, d
   m.A = m.x + 3 * Lo.N;
   m.R = m.A + Lo.nu * Lo.nu + Lo.nd * Lo.nd;
   m.T = m.R + 12;
-  m.v = m.T + Lo.P_max;
+  m.sm = m.T + Lo.P_max;
+  m.scr = m.sm + 4 + S.n_ao + 3 * Lo.nu;
+  m.v = m.scr;
   m.Ssum = m.v + Lo.N * S.n_ao;
   // the FP64 evaluation uses v and Ssum, the FP32-pipe evaluations their
   // double-float images vd and Sd: one precision runs per launch, so they
   // share the storage
   m.vd = reinterpret_cast<df*>(m.v);
   m.Sd = reinterpret_cast<df*>(m.Ssum);
-  m.xd = reinterpret_cast<df*>(m.Ssum + Lo.N);
-  m.Rd = m.xd + 3 * Lo.N;
-  m.pc = m.Rd + 12;
-  m.enc = m.pc + Lo.pcw * Lo.n_pc;
-  m.scr = reinterpret_cast<double*>(m.enc + (Lo.enc ? 8 * Lo.N * S.n_nuc : 0));
+  m.Sn = m.Sd + Lo.N;
+  m.xd = m.Sn + Lo.N;
+  m.y = m.xd + 3 * Lo.N;
+  m.Rd = m.y + 3 * Lo.N;
+  m.pfx = m.Rd + 12;
+  m.enc = m.pfx + 32;
+  m.pc = m.enc + (Lo.enc ? 8 * Lo.N * S.n_nuc : 0);
   m.n_pc = Lo.n_pc;
-  m.pcw = Lo.pcw;
   return m;
 }
 
@@ -974,117 +948,6 @@ __device__ void nucleus_terms_m(const SysDev& S, const df* v, const NT p[3], con
   }
 }
 
-// The electron-nucleus cache of one evaluation: for electron i and nucleus
-// I, d = r_i - R_I, |d|^2 and e_k . d on the rotated axes (8 double-floats,
-// the last unused). A move r_i -> r_i + h e_k has r' - R_I = d + h e_k,
-// |r' - R_I|^2 = |d|^2 + 2 h (e_k . d) + h^2, and its bond midpoint
-// |d|^2 + h (e_k . d) + h^2/4.
-template <class NT>
-__device__ void fill_en_cache(const SysDev& S, const WarpMem& wm, int lane)
-{
-  typedef Ar<NT> A;
-  const int n = S.N * S.n_nuc;
-  for (int q = lane; q < n; q += 32) {
-    const int i = q / S.n_nuc, I = q - i * S.n_nuc;
-    NT d[3];
-    for (int k = 0; k < 3; ++k) d[k] = A::sub_fast(A::c(wm.xd[3 * i + k]), A::c(S.D.nuc[I][k]));
-    df* e = &wm.enc[8 * q];
-    for (int k = 0; k < 3; ++k) e[k] = A::store(d[k]);
-    e[3] = A::store(dot3<NT>(d[0], d[1], d[2]));
-    for (int k = 0; k < 3; ++k)
-      e[4 + k] = A::store(A::add(A::add(A::mul(A::c(wm.Rd[k]), d[0]), A::mul(A::c(wm.Rd[3 + k]), d[1])),
-                                 A::mul(A::c(wm.Rd[6 + k]), d[2])));
-  }
-}
-
-// All nuclei's parts of a move from the cache, and (double grid) the
-// squared distance of the bond midpoint from the nearest heavy nucleus.
-template <class NT, bool NJ>
-__device__ __forceinline__ void nucleus_terms_cached_m(const SysDev& S, const df* v, const df* en, int k, NT h,
-                                                       const NT he[3], NT h2, const BlockMem& bm, NT& rdet,
-                                                       NT& jen, NT& mid2)
-{
-  typedef Ar<NT> A;
-  rdet = A::zero();
-  jen = A::zero();
-  mid2 = A::inf();
-  const NT h2q = A::mul_f(h2, 0.25f);
-  for (int I = 0; I < S.n_nuc; ++I) {
-    const df* e = &en[8 * I];
-    const NT hp = A::mul(h, A::c(e[4 + k]));
-    const NT D = A::c(e[3]);
-    NT d[3] = {A::add(A::c(e[0]), he[0]), A::add(A::c(e[1]), he[1]), A::add(A::c(e[2]), he[2])};
-    nucleus_term_m<NT, NJ>(S, v, I, d, A::add(A::add(D, A::mul_f(hp, 2.0f)), h2), bm, rdet, jen);
-    if (S.heavy[I]) {
-      NT m2 = A::add(A::add(D, hp), h2q);
-      if (A::lt(m2, mid2)) mid2 = m2;
-    }
-  }
-}
-
-// p from the squared distance to the nearest heavy nucleus: Eq. 3
-// (Gaussian) or Eq. 2 (Pade).
-template <class NT>
-__device__ __forceinline__ NT p_from_d2_m(const SysDev& S, const LatDev& L, NT best, const BlockMem& bm)
-{
-  typedef Ar<NT> A;
-  if (L.pkind == 0) return A::exp(A::neg(A::mul(best, A::c(L.p_coef_df))), S.D.exp.K, bm.tab);
-  return A::rcp(A::add_f(A::mul(A::c(L.p_coef_df), best), 1.0f));
-}
-
-// Index of the electron pair (a, b), a < b, in the pair cache.
-__device__ __forceinline__ int pair_index(int N, int a, int b) { return a * N - a * (a + 1) / 2 + (b - a - 1); }
-
-// The pair cache of one evaluation: for every pair a < b, D = |r_a - r_b|^2
-// and P_k = e_k . (r_a - r_b) on the evaluation's rotated axes. A lattice
-// move r_i -> r_i + h e_k then has |r' - r_j|^2 = D + 2 h s P_k + h^2, with
-// s = +1 for i = a and -1 for i = b.
-template <class NT, bool NJ>
-__device__ void fill_pair_cache(const SysDev& S, const WarpMem& wm, int lane)
-{
-  typedef Ar<NT> A;
-  const int N = S.N;
-  for (int q = lane; q < wm.n_pc; q += 32) {
-    int a = 0, base = 0;
-    while (base + (N - 1 - a) <= q) { base += N - 1 - a; ++a; }
-    const int b = a + 1 + (q - base);
-    NT d[3];
-    for (int k = 0; k < 3; ++k) d[k] = A::sub_fast(A::c(wm.xd[3 * a + k]), A::c(wm.xd[3 * b + k]));
-    df* e = &wm.pc[wm.pcw * q];
-    const NT D = dot3<NT>(d[0], d[1], d[2]);
-    e[0] = A::store(D);
-    for (int k = 0; k < 3; ++k) {
-      NT pk = A::add(A::add(A::mul(A::c(wm.Rd[k]), d[0]), A::mul(A::c(wm.Rd[3 + k]), d[1])),
-                     A::mul(A::c(wm.Rd[6 + k]), d[2]));
-      e[1 + k] = A::store(pk);
-    }
-    if ((wm.pcw == 8 && wm.n_pc > 0 && NJ)) {
-      // with the neural term, the pair's Jastrow terms for the local energy
-      // (Pade plus neural): u, u'/r, u'' + 2 u'/r, and 1/r (with the Pade
-      // factor alone, evaluating them inside the local energy is faster)
-      const NT rr = A::sqrt(D);
-      const NT bb = A::c(S.D.b_ee);
-      const NT c = (spin_of(S, a) == spin_of(S, b)) ? A::c(S.D.c_par) : A::c(S.D.c_anti);
-      const NT inv = A::rcp(A::add_f(A::mul(bb, rr), 1.0f));
-      const NT inv2 = A::sqr(inv);
-      NT u = A::mul(A::mul(c, rr), inv);
-      NT u1 = A::mul(c, inv2);
-      NT u2 = A::mul_f(A::mul(A::mul(bb, c), A::mul(inv2, inv)), -2.0f);
-      if (NJ) {
-        NT g, g1, g2;
-        nj_value3_m<NT>(S, nj_ch_ee(S, a, b), rr, g, g1, g2);
-        u1 = A::add(u1, g1); u2 = A::add(u2, g2); u = A::add(u, g);
-      }
-      const NT irr = A::rcp(rr);
-      const NT u1ir = A::mul(u1, irr);
-      e[4] = A::store(u);
-      e[5] = A::store(u1ir);
-      e[6] = A::store(A::add(u2, A::mul_f(u1ir, 2.0f)));
-      e[7] = A::store(irr);
-    }
-  }
-}
-
 // num and den times the power of two that brings den (positive, normal,
 // below 2^127) into [1, 2): exact, so num/den keeps its value bit for bit.
 __device__ __forceinline__ void pow2_rescale(float& num, float& den)
@@ -1101,42 +964,6 @@ __device__ __forceinline__ void pow2_rescale(df& num, df& den)
   num.lo *= s;
   den.hi *= s;
   den.lo *= s;
-}
-
-// sum_{j != i} u_ee(|r_i + h e_k - r_j|) from the pair cache (h carries
-// the sign of the move, h2 = h^2); the Pade terms as one running fraction.
-template <class NT, bool NJ>
-__device__ NT jastrow_ee_cached_m(const SysDev& S, const df* pc, int pcw, int i, int k, NT h, NT h2)
-{
-  typedef Ar<NT> A;
-  NT num = A::zero(), den = A::one(), nn = A::zero();
-  const int si = spin_of(S, i), N = S.N;
-  const NT b = A::c(S.D.b_ee), cp = A::c(S.D.c_par), ca = A::c(S.D.c_anti);
-  // 2h s for the partners after i (s = +1) and before i (s = -1): scaling by
-  // a power of two is exact
-  const NT h2p = A::mul_f(h, 2.0f), h2m = A::neg(h2p);
-  // pair (j, i), j < i, sits at j N - j (j + 1)/2 + (i - j - 1), which grows by
-  // N - j - 2 from j to j + 1; pair (i, j), j > i, at q0 + (j - i - 1)
-  int q = i - 1;  // pair (0, i)
-  for (int j = 0; j < N; ++j) {
-    if (j == i) {
-      q = pair_index(N, i, i + 1);  // the next partner's pair (unused when i = N - 1)
-      continue;
-    }
-    const df* e = &pc[pcw * q];
-    const NT hp = A::mul(j > i ? h2p : h2m, A::c(e[1 + k]));
-    // |r' - r_j|^2 = D + 2 h s P_k + h^2: the cheap addition suffices (its
-    // error ~2^-44 (D + |2hP| + h^2) is far below what the ratios resolve)
-    NT r = A::sqrt(A::add_fast(A::add_fast(A::c(e[0]), hp), h2));
-    NT c = (spin_of(S, j) == si) ? cp : ca;
-    NT dj = A::add_f(A::mul(b, r), 1.0f);
-    num = A::add_fast(A::mul(num, dj), A::mul(A::mul(c, r), den));
-    den = A::mul(den, dj);
-    if (NJ) nn = A::add(nn, nj_value_m<NT>(S, nj_ch_ee(S, i, j), r));
-    q += (j < i) ? N - j - 2 : 1;
-    if ((j & 15) == 15) pow2_rescale(num, den);  // every 16 partners, as in jastrow_ee_m
-  }
-  return A::add(A::div(num, den), nn);
 }
 
 // sum_{j != i} u_ee(|p - r_j|): the Pade terms c r/(1 + b r) (all of one
@@ -1222,235 +1049,33 @@ __device__ NT warp_scan_m(const df* T, int P, int lane, NT target, int* pick, in
   return carry;
 }
 
-// Partial sums of the local energy of electron i over the shell units, the
-// partners (the t-th electron other than i) and the nuclei whose index is
-// congruent to part modulo L.
-template <class NT>
-struct ElParts {
-  NT gD[3], lD, gJ[3], lJ, S, V;
-};
-
-template <class NT>
-__device__ __forceinline__ void el_zero(ElParts<NT>& o)
-{
-  typedef Ar<NT> A;
-  o.lD = A::zero(); o.lJ = A::zero(); o.S = A::zero(); o.V = A::zero();
-  for (int k = 0; k < 3; ++k) { o.gD[k] = A::zero(); o.gJ[k] = A::zero(); }
-}
-
-template <class NT, bool NJ, bool PC = true>
-__device__ LRDMC_EL void el_parts_m(const SysDev& S, const WarpMem& wm, int i, int part, int L, const BlockMem& bm,
-                           ElParts<NT>& o)
-{
-  typedef Ar<NT> A;
-  const int nao = S.n_ao;
-  const df* v = &wm.vd[i * nao];
-  const NT ri[3] = {A::c(wm.xd[3 * i]), A::c(wm.xd[3 * i + 1]), A::c(wm.xd[3 * i + 2])};
-  el_zero<NT>(o);
-  // basis: gradient and Laplacian contracted with v. The shells' units
-  // (single shells, or groups sharing one Slater exponential) are dealt to
-  // the parts, and each part loops over its own units only, so that the
-  // parts' shells run side by side on their lanes (a loop over all shells
-  // with the others' skipped would run them one after the other).
-  int prev_c = -1;
-  NT d[3] = {A::zero(), A::zero(), A::zero()}, r = A::zero(), r2 = A::zero(), ir = A::zero(), e = A::zero();
-  for (int gi = part; gi < S.n_grp; gi += L)
-  for (int q = S.grp_first[gi]; q < S.grp_first[gi + 1]; ++q) {
-    const ShellDev& sh = S.sh[q];
-    const DfShell& dsh = S.D.sh[q];
-    const bool first = q == S.grp_first[gi];
-    if (sh.center != prev_c) {
-      prev_c = sh.center;
-      d[0] = A::sub_fast(ri[0], A::c(S.D.nuc[prev_c][0]));
-      d[1] = A::sub_fast(ri[1], A::c(S.D.nuc[prev_c][1]));
-      d[2] = A::sub_fast(ri[2], A::c(S.D.nuc[prev_c][2]));
-      r2 = dot3<NT>(d[0], d[1], d[2]);
-      r = A::sqrt(r2);
-      ir = A::rcp(r);
-    }
-    if (sh.kind == 0 && (first || !sh.same_exp)) e = A::exp(A::neg(A::mul(A::c(dsh.zeta), r)), S.D.exp.K, bm.tab);
-    NT Rv, R1, R2;
-    if (sh.kind == 0) {
-      Rv = radial_value_m<NT>(S, sh, dsh, r, r2, e, bm);
-      NT t = A::sub(A::mul(A::c(dsh.m), ir), A::c(dsh.zeta));
-      R1 = A::mul(A::mul(t, Rv), ir);
-      R2 = A::mul(A::sub(A::sqr(t), A::mul(A::c(dsh.m), A::sqr(ir))), Rv);
-    } else {
-      Rv = A::zero(); R1 = A::zero(); R2 = A::zero();
-      for (int p = 0; p < sh.n_prim; ++p) {
-        NT al = A::c(dsh.alpha[p]);
-        NT g = A::mul(A::c(dsh.coef[p]), A::exp(A::neg(A::mul(al, r2)), S.D.exp.K, bm.tab));
-        Rv = A::add(Rv, g);
-        NT m2a = A::mul_f(al, -2.0f);
-        R1 = A::add(R1, A::mul(m2a, g));
-        NT four_a2r2 = A::mul_f(A::mul(A::sqr(al), r2), 4.0f);
-        R2 = A::add(R2, A::mul(A::add(four_a2r2, m2a), g));
-      }
-    }
-    NT Sv[5];
-    int nf = solid_m<NT>(sh.l, d, Sv);
-    NT radlap = A::add(R2, A::mul_f(R1, 2.0f * (sh.l + 1)));
-    for (int f = 0; f < nf; ++f) {
-      NT cc = A::c(v[sh.ao_offset + f]);
-      NT cS = A::mul(cc, Sv[f]);
-      // grad S of the solid harmonics
-      NT gS[3];
-      if (sh.l == 0) { gS[0] = A::zero(); gS[1] = A::zero(); gS[2] = A::zero(); }
-      else if (sh.l == 1) { gS[0] = A::zero(); gS[1] = A::zero(); gS[2] = A::zero(); gS[f] = A::one(); }
-      else {
-        switch (f) {
-          case 0: gS[0] = d[1]; gS[1] = d[0]; gS[2] = A::zero(); break;
-          case 1: gS[0] = A::zero(); gS[1] = d[2]; gS[2] = d[1]; break;
-          case 2: gS[0] = d[2]; gS[1] = A::zero(); gS[2] = d[0]; break;
-          case 3: gS[0] = A::mul_f(d[0], 2.0f); gS[1] = A::mul_f(d[1], -2.0f); gS[2] = A::zero(); break;
-          default: gS[0] = A::mul_f(d[0], -2.0f); gS[1] = A::mul_f(d[1], -2.0f); gS[2] = A::mul_f(d[2], 4.0f); break;
-        }
-      }
-      NT cSR1 = A::mul(cS, R1);
-      NT cR = A::mul(cc, Rv);
-      for (int k = 0; k < 3; ++k) o.gD[k] = A::add(o.gD[k], A::add(A::mul(cR, gS[k]), A::mul(cSR1, d[k])));
-      o.lD = A::add(o.lD, A::mul(cS, radlap));
-    }
-  }
-  // e-e pairs: the N - 1 partners of i (j = t, skipping i) dealt evenly
-  // to the parts
-  const int si = spin_of(S, i);
-  const NT b = A::c(S.D.b_ee);
-  if (PC && sizeof(NT) == sizeof(df) && (wm.pcw == 8 && wm.n_pc > 0 && NJ)) {
-    // every pair's terms come from the pair cache (evaluated once per pair)
-    for (int t = part; t < S.N - 1; t += L) {
-      const int j = t < i ? t : t + 1;
-      const df* e = &wm.pc[8 * pair_index(S.N, min(i, j), max(i, j))];
-      NT d0 = A::sub_fast(ri[0], A::c(wm.xd[3 * j])), d1 = A::sub_fast(ri[1], A::c(wm.xd[3 * j + 1])),
-         d2 = A::sub_fast(ri[2], A::c(wm.xd[3 * j + 2]));
-      const NT u1ir = A::c(e[5]);
-      o.gJ[0] = A::add(o.gJ[0], A::mul(u1ir, d0));
-      o.gJ[1] = A::add(o.gJ[1], A::mul(u1ir, d1));
-      o.gJ[2] = A::add(o.gJ[2], A::mul(u1ir, d2));
-      o.lJ = A::add(o.lJ, A::c(e[6]));
-      o.S = A::add(o.S, A::c(e[4]));
-      if (j > i && S.ee_on) o.V = A::add(o.V, A::c(e[7]));
-    }
-  } else
-  for (int t = part; t < S.N - 1; t += L) {
-    const int j = t < i ? t : t + 1;
-    NT d0 = A::sub_fast(ri[0], A::c(wm.xd[3 * j])), d1 = A::sub_fast(ri[1], A::c(wm.xd[3 * j + 1])),
-       d2 = A::sub_fast(ri[2], A::c(wm.xd[3 * j + 2]));
-    NT rr = A::sqrt(dot3<NT>(d0, d1, d2));
-    NT c = (spin_of(S, j) == si) ? A::c(S.D.c_par) : A::c(S.D.c_anti);
-    NT inv = A::rcp(A::add_f(A::mul(b, rr), 1.0f));
-    NT inv2 = A::sqr(inv);
-    NT u1 = A::mul(c, inv2);
-    NT u2 = A::mul_f(A::mul(A::mul(b, c), A::mul(inv2, inv)), -2.0f);
-    o.S = A::add(o.S, A::mul(A::mul(c, rr), inv));
-    if (NJ) {
-      NT g, g1, g2;
-      nj_value3_m<NT>(S, nj_ch_ee(S, i, j), rr, g, g1, g2);
-      u1 = A::add(u1, g1); u2 = A::add(u2, g2); o.S = A::add(o.S, g);
-    }
-    NT irr = A::rcp(rr);
-    NT u1ir = A::mul(u1, irr);
-    o.gJ[0] = A::add(o.gJ[0], A::mul(u1ir, d0));
-    o.gJ[1] = A::add(o.gJ[1], A::mul(u1ir, d1));
-    o.gJ[2] = A::add(o.gJ[2], A::mul(u1ir, d2));
-    o.lJ = A::add(o.lJ, A::add(u2, A::mul_f(u1ir, 2.0f)));
-    if (j > i && S.ee_on) o.V = A::add(o.V, irr);
-  }
-  // e-n terms
-  for (int I = part; I < S.n_nuc; I += L) {
-    NT d0 = A::sub_fast(ri[0], A::c(S.D.nuc[I][0])), d1 = A::sub_fast(ri[1], A::c(S.D.nuc[I][1])),
-       d2 = A::sub_fast(ri[2], A::c(S.D.nuc[I][2]));
-    NT rr = A::sqrt(dot3<NT>(d0, d1, d2));
-    NT b1 = A::c(S.D.en_b1[I]), b2 = A::c(S.D.en_b2);
-    NT inv = A::rcp(A::add_f(A::mul(b2, rr), 1.0f));
-    NT inv2 = A::sqr(inv);
-    NT u1 = A::neg(A::mul(b1, inv2));
-    NT u2 = A::mul_f(A::mul(A::mul(b2, b1), A::mul(inv2, inv)), 2.0f);
-    o.S = A::sub(o.S, A::mul(A::mul(b1, rr), inv));
-    if (NJ) {
-      NT g, g1, g2;
-      nj_value3_m<NT>(S, 2 + S.nj_species[I], rr, g, g1, g2);
-      u1 = A::add(u1, g1); u2 = A::add(u2, g2); o.S = A::add(o.S, g);
-    }
-    NT irr = A::rcp(rr);
-    NT u1ir = A::mul(u1, irr);
-    o.gJ[0] = A::add(o.gJ[0], A::mul(u1ir, d0));
-    o.gJ[1] = A::add(o.gJ[1], A::mul(u1ir, d1));
-    o.gJ[2] = A::add(o.gJ[2], A::mul(u1ir, d2));
-    o.lJ = A::add(o.lJ, A::add(u2, A::mul_f(u1ir, 2.0f)));
-    o.V = A::sub(o.V, A::mul(A::c(S.D.Z[I]), irr));
-  }
-}
-
-template <class NT>
-__device__ __forceinline__ void el_combine(ElParts<NT>& o, int src, bool take)
-{
-  typedef Ar<NT> A;
-  NT t;
-#define ELC(field)            \
-  t = A::shfl(o.field, src);  \
-  if (take) o.field = A::add(o.field, t);
-  ELC(lD) ELC(lJ) ELC(S) ELC(V)
-  ELC(gD[0]) ELC(gD[1]) ELC(gD[2]) ELC(gJ[0]) ELC(gJ[1]) ELC(gJ[2])
-#undef ELC
-}
-
-template <class NT>
-__device__ __forceinline__ NT el_local(const ElParts<NT>& o)
-{
-  typedef Ar<NT> A;
-  NT dot = A::add(A::add(A::mul(o.gD[0], o.gJ[0]), A::mul(o.gD[1], o.gJ[1])), A::mul(o.gD[2], o.gJ[2]));
-  NT gg = A::add(A::add(A::sqr(o.gJ[0]), A::sqr(o.gJ[1])), A::sqr(o.gJ[2]));
-  NT lap = A::add(A::add(o.lD, A::mul_f(dot, 2.0f)), A::add(o.lJ, gg));
-  return A::add(A::mul_f(lap, -0.5f), o.V);
-}
-
 // One lattice move c of an evaluation (Eq. 1 lattice, fixed-node rate): the
 // determinant and Jastrow ratios at the displaced position, p at the bond
 // midpoint on the double grid, the rate T_c into Td[c]. Reads the
 // evaluation's shared-memory state (projected inverse columns, positions,
-// rotation, caches and the Jastrow sums Sd of its local-energy pass).
-template <class NT, bool NJ, bool NC>
+// rotation and the Jastrow sums Sd of its local-energy pass).
+template <class NT, bool NJ>
 __device__ __forceinline__ void candidate_m(const SysDev& S, const LatDev& L, const WarpMem& wm, const BlockMem& bm,
                                             int c, df* Td, double* ratio_out)
 {
   typedef Ar<NT> A;
   const int nao = S.n_ao;
   const int G = L.G, per_e = 6 * G;
-  constexpr bool kUsePairCache = sizeof(NT) == sizeof(df) && !NC;
   {
     const int i = c / per_e, rem = c - i * per_e, g = rem / 6, k = (rem % 6) >> 1;
     NT h = g ? A::c(L.ap_df) : A::c(L.a_df);
     if (c & 1) h = A::neg(h);
     const NT e0 = A::c(wm.Rd[k]), e1 = A::c(wm.Rd[3 + k]), e2 = A::c(wm.Rd[6 + k]);
     NT rdet, jen, jee, pm = A::one();
-    if (kUsePairCache) {
-      // the caches pay in double-float arithmetic only (single precision
-      // recomputes a distance faster than it reads it back)
-      const NT h2 = A::sqr(h);
-      const NT he[3] = {A::mul(h, e0), A::mul(h, e1), A::mul(h, e2)};
-      NT mid2;
-      nucleus_terms_cached_m<NT, NJ>(S, &wm.vd[i * nao], &wm.enc[8 * i * S.n_nuc], k, h, he, h2, bm, rdet, jen,
-                                 mid2);
-      if (wm.n_pc) {
-        jee = jastrow_ee_cached_m<NT, NJ>(S, wm.pc, wm.pcw, i, k, h, h2);
-      } else {
-        const NT p[3] = {A::add(A::c(wm.xd[3 * i]), he[0]), A::add(A::c(wm.xd[3 * i + 1]), he[1]),
-                         A::add(A::c(wm.xd[3 * i + 2]), he[2])};
-        jee = jastrow_ee_m<NT, NJ>(S, wm.xd, i, p);
-      }
-      if (G == 2) pm = p_from_d2_m<NT>(S, L, mid2, bm);
-    } else {
-      const NT ri[3] = {A::c(wm.xd[3 * i]), A::c(wm.xd[3 * i + 1]), A::c(wm.xd[3 * i + 2])};
-      const NT p[3] = {A::add(ri[0], A::mul(h, e0)), A::add(ri[1], A::mul(h, e1)), A::add(ri[2], A::mul(h, e2))};
-      nucleus_terms_m<NT, NJ>(S, &wm.vd[i * nao], p, bm, rdet, jen);
-      jee = jastrow_ee_m<NT, NJ>(S, wm.xd, i, p);
-      if (G == 2) {
-        const NT hh = A::half(h);
-        const NT mid[3] = {A::add(ri[0], A::mul(hh, e0)), A::add(ri[1], A::mul(hh, e1)),
-                           A::add(ri[2], A::mul(hh, e2))};
-        pm = p_weight_m<NT>(S, L, mid, bm);
-      }
+    const NT ri[3] = {A::c(wm.xd[3 * i]), A::c(wm.xd[3 * i + 1]), A::c(wm.xd[3 * i + 2])};
+    const NT p[3] = {A::add(ri[0], A::mul(h, e0)), A::add(ri[1], A::mul(h, e1)), A::add(ri[2], A::mul(h, e2))};
+    nucleus_terms_m<NT, NJ>(S, &wm.vd[i * nao], p, bm, rdet, jen);
+    jee = jastrow_ee_m<NT, NJ>(S, wm.xd, i, p);
+    if (G == 2) {
+      const NT hh = A::half(h);
+      const NT mid[3] = {A::add(ri[0], A::mul(hh, e0)), A::add(ri[1], A::mul(hh, e1)),
+                         A::add(ri[2], A::mul(hh, e2))};
+      pm = p_weight_m<NT>(S, L, mid, bm);
     }
     NT dJ = A::sub(A::add(jee, jen), A::c(wm.Sd[i]));
     NT rho = A::mul(rdet, A::exp(dJ, S.D.exp.K, bm.tab));
@@ -1463,131 +1088,45 @@ __device__ __forceinline__ void candidate_m(const SysDev& S, const LatDev& L, co
   }
 }
 
-// The first part of an evaluation: projected inverse columns, converted
-// positions and rotation, the caches, then the local energy (into el) and
-// the Jastrow sums Sd of every electron. The moves read all of it.
-// 1: the FP32 mode's local energy in double-float (the lattice moves stay in
-// single precision); 0: all of its evaluation in single precision.
-#ifndef LRDMC_FP32_EL_DF
-#define LRDMC_FP32_EL_DF 1
-#endif
-template <class NT, bool NJ, bool NC>
-__device__ __forceinline__ void eval_prelude_m(const SysDev& S, const double* sC, const LatDev& L, const WarpMem& wm,
-                                               int lane, double& el)
+}  // namespace lrdmc
+#include "eval64.cuh"
+namespace lrdmc {
+
+// The mixed mode's evaluation: projected columns, local energy and Jastrow
+// sums as in the double-float mode, the moves in single precision (they read
+// the double-float values' leading floats).
+template <bool NJ>
+__device__ __forceinline__ double prelude32(const SysDev& S, const double* sC, const WarpMem& wm, const Lean& lt,
+                                            int lane, int moved)
 {
-  typedef Ar<NT> A;
-  const int N = S.N, nao = S.n_ao, nu = S.n_up;
-  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
-  // projected inverse columns (FP64, or FP32 in the mixed mode), then
-  // converted with the positions. The mixed mode converts the inverse
-  // blocks to float once (scratch), not once per use: each conversion from
-  // double runs on the FP64 pipe
-  // The FP32 mode can take its local energy in double-float (LRDMC_FP32_EL_DF,
-  // on by default): the projected columns, positions and rotation are then
-  // formed as in the double-float mode, and only the lattice moves run in
-  // single precision (they read the double-float values' leading floats).
-  constexpr bool kElDf = sizeof(NT) == sizeof(float) && LRDMC_FP32_EL_DF;
-  constexpr bool kFloatProj = sizeof(NT) == sizeof(float) && !kElDf;
-  typedef typename std::conditional<kElDf, df, NT>::type ET;
-  typedef Ar<ET> AE;
-  const float* Af = reinterpret_cast<const float*>(wm.scr);
-  if (kFloatProj) {
-    for (int j = lane; j < nu * nu + S.n_dn * S.n_dn; j += 32) reinterpret_cast<float*>(wm.scr)[j] = (float)wm.A[j];
-    __syncwarp();
-  }
-  for (int idx = lane; idx < N * nao; idx += 32) {
-    int i = idx / nao, mu = idx % nao;
-    int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
-    const double* Am = spin ? wm.A + nu * nu : wm.A;
-    if (kFloatProj) {
-      const float* Amf = spin ? Af + nu * nu : Af;
-      float acc = 0.0f;
-      for (int m = 0; m < n; ++m) acc += bm.Cf[mu * S.n_mo + m] * Amf[m * n + l];
-      wm.vd[idx] = df_make(acc, 0.0f);
-    } else {
-      double acc = 0.0;
-      for (int m = 0; m < n; ++m) acc += sC[mu * S.n_mo + m] * Am[m * n + l];
-      wm.vd[idx] = AE::store(AE::from_double(acc));
-    }
-  }
-  for (int j = lane; j < 3 * N; j += 32) wm.xd[j] = AE::store(AE::from_double(wm.x[j]));
-  if (lane < 9) wm.Rd[lane] = AE::store(AE::from_double(wm.R[lane]));
-  __syncwarp();
-  // the caches pay in double-float arithmetic only, and exist only when
-  // the system's layout has room for them (NC is set otherwise: the
-  // kernels of such systems carry no cached code)
-  constexpr bool kUsePairCache = sizeof(NT) == sizeof(df) && !NC;
-  if (kUsePairCache) {
-    fill_pair_cache<NT, NJ>(S, wm, lane);
-    fill_en_cache<NT>(S, wm, lane);
-    __syncwarp();
-  }
-  // local energy: Lp lanes per electron share its shells, electrons and nuclei
-  constexpr bool kPC = sizeof(NT) == sizeof(df) && !NC;  // the pair cache holds the pairs' terms
-  ET epart = AE::zero();
-  if (N <= 32) {
-    const int Lp = 32 / N;
-    const int i = lane % N, part = lane / N;
-    const bool act = lane < N * Lp;
-    ElParts<ET> o;
-    if (act) el_parts_m<ET, NJ, kPC>(S, wm, i, part, Lp, bm, o);
-    else el_zero<ET>(o);
-    for (int pp = 1; pp < Lp; ++pp) {
-      int src = lane + pp * N;
-      el_combine<ET>(o, src < 32 ? src : lane, part == 0 && src < N * Lp);
-    }
-    if (part == 0 && act) {
-      wm.Sd[i] = AE::store(o.S);
-      epart = el_local<ET>(o);
-    }
-  } else {
-    for (int i = lane; i < N; i += 32) {
-      ElParts<ET> o;
-      el_parts_m<ET, NJ, kPC>(S, wm, i, 0, 1, bm, o);
-      wm.Sd[i] = AE::store(o.S);
-      epart = AE::add(epart, el_local<ET>(o));
-    }
-  }
-  ET etot = warp_sum_m<ET>(epart);
-  el = AE::to_double(etot) + S.V_nn;
-  __syncwarp();
+  const double el = prelude64<NJ, true, false>(S, sC, wm, lt, lane, moved);
+  total_jastrow64(S, wm, lane);
+  return el;
 }
 
-template <class NT, bool NJ, bool NC, bool MOVES = true>
-__device__ void warp_eval_m(const SysDev& S, const double* sC, const LatDev& L, const WarpMem& wm, int lane,
-                            double* ratio_out, double& b, df& bdf, double& el)
+template <bool NJ>
+__device__ void warp_eval32(const SysDev& S, double* sC, const LatDev& L, const WarpMem& wm, int lane,
+                            double* ratio_out, double& b, double& el)
 {
-  typedef Ar<NT> A;
-  const int N = S.N;
-  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
-  eval_prelude_m<NT, NJ, NC>(S, sC, L, wm, lane, el);
-  if (!MOVES) {  // local energy and Jastrow sums only (the caller forms the moves)
-    b = 0.0;
-    bdf = A::store(A::zero());
-    return;
-  }
-  // the P lattice moves
-  const int G = L.G, per_e = 6 * G, P = N * per_e;
-  df* Td = reinterpret_cast<df*>(wm.T);  // rates stay in NT, stored as double-floats
-  for (int c = lane; c < P; c += 32) candidate_m<NT, NJ, NC>(S, L, wm, bm, c, Td, ratio_out);
+  const BlockMem bm = block_mem(S, sC);
+  el = prelude32<NJ>(S, sC, wm, lean_mem(S, sC), lane, -1);
+  const int P = 6 * L.G * S.N;
+  df* Td = reinterpret_cast<df*>(wm.T);  // rates stored as double-floats
+  for (int c = lane; c < P; c += 32) candidate_m<float, NJ>(S, L, wm, bm, c, Td, ratio_out);
   __syncwarp();
-  NT btot = warp_scan_m<NT>(Td, P, lane, A::zero(), nullptr, nullptr);
-  bdf = A::store(btot);
-  b = A::to_double(btot);
+  b = (double)warp_scan_m<float>(Td, P, lane, 0.0f, nullptr, nullptr);
 }
 
 template <int PREC, bool NJ, bool NC>
-__device__ __forceinline__ void warp_eval_any(const SysDev& S, const double* sC, const LatDev& L,
-                                              const WarpMem& wm, int lane, double* ratio_out, double& b,
-                                              df& bdf, double& el)
+__device__ __forceinline__ void warp_eval_any(const SysDev& S, double* sC, const LatDev& L, const WarpMem& wm,
+                                              int lane, double* ratio_out, double& b, double& el)
 {
   if (PREC == LRDMC_PRECISION_DF64) {
-    warp_eval_m<df, NJ, NC>(S, sC, L, wm, lane, ratio_out, b, bdf, el);
+    warp_eval64<NJ, NC>(S, sC, L, wm, lane, ratio_out, b, el);
   } else if (PREC == LRDMC_PRECISION_FP32) {
-    warp_eval_m<float, NJ, true>(S, sC, L, wm, lane, ratio_out, b, bdf, el);
+    warp_eval32<NJ>(S, sC, L, wm, lane, ratio_out, b, el);
   } else {
     warp_eval<NJ>(S, sC, L, wm, lane, ratio_out, b, el);
-    bdf = df_make(0.0f, 0.0f);
   }
 }
 
@@ -1596,100 +1135,9 @@ __device__ __forceinline__ void warp_eval_any(const SysDev& S, const double* sC,
 // y_n = sum_m phi_m(p) Ainv[m][n], ratio = y_l,
 // Ainv[m][n] -= Ainv[m][l] (y_n - delta_nl) / ratio.
 // ----------------------------------------------------------------------------
-// chi_mu(p) for all AOs in double-float, one lane per shell, written back
-// as doubles.
-static __device__ void ao_values_df_lanes(const SysDev& S, const double* p, double* out, int lane, const BlockMem& bm)
-{
-  typedef Ar<df> A;
-  df pd[3] = {df_from_double(p[0]), df_from_double(p[1]), df_from_double(p[2])};
-  // one shell per lane (at most 32 shells), each with its own centre
-  // distance and exponential: all shells side by side
-  for (int q = lane; q < S.n_shell; q += 32) {
-    const ShellDev& sh = S.sh[q];
-    const DfShell& dsh = S.D.sh[q];
-    df d[3];
-    d[0] = df_sub_fast(pd[0], S.D.nuc[sh.center][0]);
-    d[1] = df_sub_fast(pd[1], S.D.nuc[sh.center][1]);
-    d[2] = df_sub_fast(pd[2], S.D.nuc[sh.center][2]);
-    const df r2 = dot3<df>(d[0], d[1], d[2]);
-    const df r = df_sqrt(r2);
-    df e = A::zero();
-    if (sh.kind == 0) e = df_exp(df_neg(df_mul(dsh.zeta, r)), S.D.exp.K, bm.tab);
-    df Rv = radial_value_m<df>(S, sh, dsh, r, r2, e, bm);
-    df Sv[5];
-    int nf = solid_m<df>(sh.l, d, Sv);
-    for (int f = 0; f < nf; ++f) out[sh.ao_offset + f] = df_to_double(df_mul(Sv[f], Rv));
-  }
-}
-
-// chi_mu(p) for all AOs in double-float into out (df), one lane per shell.
-static __device__ void ao_values_df_out(const SysDev& S, const df* pd, df* out, int lane, const BlockMem& bm)
-{
-  typedef Ar<df> A;
-  // one shell per lane (at most 32 shells), each with its own centre
-  // distance and exponential: all shells side by side
-  for (int q = lane; q < S.n_shell; q += 32) {
-    const ShellDev& sh = S.sh[q];
-    const DfShell& dsh = S.D.sh[q];
-    df d[3];
-    d[0] = df_sub_fast(pd[0], S.D.nuc[sh.center][0]);
-    d[1] = df_sub_fast(pd[1], S.D.nuc[sh.center][1]);
-    d[2] = df_sub_fast(pd[2], S.D.nuc[sh.center][2]);
-    const df r2 = dot3<df>(d[0], d[1], d[2]);
-    const df r = df_sqrt(r2);
-    df e = A::zero();
-    if (sh.kind == 0) e = df_exp(df_neg(df_mul(dsh.zeta, r)), S.D.exp.K, bm.tab);
-    df Rv = radial_value_m<df>(S, sh, dsh, r, r2, e, bm);
-    df Sv[5];
-    int nf = solid_m<df>(sh.l, d, Sv);
-    for (int f = 0; f < nf; ++f) out[sh.ao_offset + f] = df_mul(Sv[f], Rv);
-  }
-}
-
-// Sherman-Morrison update in double-float arithmetic (the FP32 mode): the
-// orbitals at the new position, y = phi A^-1, ratio = y_l, and
-// the rank-one update, with the spin block read from and written back to
-// its IEEE-double copy. pd: the new position as a double-float.
-static __device__ LRDMC_JUMP bool warp_sm_update_df(const SysDev& S, const BlockMem& bm, const WarpMem& wm, int i, const df* pd,
-                                  int lane)
-{
-  const int nu = S.n_up;
-  const int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
-  double* A = spin ? wm.A + nu * nu : wm.A;
-  df* chi = reinterpret_cast<df*>(wm.scr);  // [n_ao]
-  df* phi = chi + S.n_ao;                   // [n]
-  df* y = phi + n;                          // [n]
-  df* Ad = y + n;                           // [n][n]
-  ao_values_df_out(S, pd, chi, lane, bm);
-  for (int idx = lane; idx < n * n; idx += 32) Ad[idx] = df_from_double(A[idx]);
-  __syncwarp();
-  for (int m = lane; m < n; m += 32) {
-    df a = df_make(0.0f, 0.0f);
-    for (int mu = 0; mu < S.n_ao; ++mu) a = df_add(a, df_mul(bm.Cd[mu * S.n_mo + m], chi[mu]));
-    phi[m] = a;
-  }
-  __syncwarp();
-  for (int q = lane; q < n; q += 32) {
-    df a = df_make(0.0f, 0.0f);
-    for (int m = 0; m < n; ++m) a = df_add(a, df_mul(phi[m], Ad[m * n + q]));
-    y[q] = a;
-  }
-  __syncwarp();
-  const df ratio = y[l];
-  if (ratio.hi == 0.0f) return false;
-  const df inv = df_rcp(ratio);
-  for (int idx = lane; idx < n * n; idx += 32) {
-    int m = idx / n, q = idx % n;
-    df yq = (q == l) ? df_add_f(y[q], -1.0f) : y[q];
-    A[idx] = df_to_double(df_sub(Ad[idx], df_mul(Ad[m * n + l], df_mul(yq, inv))));
-  }
-  __syncwarp();
-  return true;
-}
-
-template <int PREC>
-__device__ LRDMC_JUMP bool warp_sm_update(const SysDev& S, const double* sC, const WarpMem& wm, int i,
-                               const double* p, int lane)
+// The FP64 mode's update.
+static __device__ LRDMC_JUMP bool warp_sm_update(const SysDev& S, const double* sC, const WarpMem& wm, int i,
+                                                 const double* p, int lane)
 {
   const int nu = S.n_up;
   const int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
@@ -1698,8 +1146,7 @@ __device__ LRDMC_JUMP bool warp_sm_update(const SysDev& S, const double* sC, con
   double* phi = chi + S.n_ao;      // [n]
   double* y = phi + n;             // [n]
   double* col = y + n;             // [n]
-  if (PREC != LRDMC_PRECISION_FP64) ao_values_df_lanes(S, p, chi, lane, block_mem(S, const_cast<double*>(sC)));
-  else if (lane == 0) ao_values(S, p, chi);
+  if (lane == 0) ao_values(S, p, chi);
   __syncwarp();
   for (int m = lane; m < n; m += 32) {
     double a = 0.0;
@@ -1754,8 +1201,10 @@ __device__ __forceinline__ void store_record(const Layout& Lo, double* rec, cons
   }
 }
 
+template <bool LEAN = false>
 __device__ __forceinline__ void stage_coefficients(const SysDev& S, double* sC)
 {
+  if (LEAN) lean_stage(S, sC);
   BlockMem bm = block_mem(S, sC);
   for (int j = threadIdx.x; j < S.n_ao * S.n_mo; j += blockDim.x) {
     sC[j] = S.C[j];
@@ -1773,7 +1222,7 @@ __device__ __forceinline__ void stage_coefficients(const SysDev& S, double* sC)
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 k_init(const __grid_constant__ SysDev S, const Layout Lo, const PopDev P, const double* x0)
 {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
   stage_coefficients(S, sC);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1805,18 +1254,17 @@ k_eval_all(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
   constexpr int PR = PREC & 3;         // the arithmetic (LRDMC_PRECISION_*)
   constexpr bool NJ = (PREC & 8) != 0;  // the neural pair term is set
   constexpr bool NC = (PREC & 4) != 0;  // the layout has no evaluation caches
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
-  stage_coefficients(S, sC);
+  stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int s = blockIdx.x * kWarpsPerBlock + wib;
   if (s >= P.W) return;
   WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
   double* rec = P.rec_src + (size_t)s * Lo.rec;
   double b, el;
-  df bdf;
   load_record(Lo, rec, wm, lane, b, el);
-  warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, bdf, el);
+  warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, el);
   if (!isfinite(el) || !isfinite(b)) {
     if (lane == 0) atomicOr(P.err, kErrNonFinite);
   }
@@ -1879,9 +1327,10 @@ __device__ __forceinline__ int team_publish(TeamSlot* t, int lane)
 
 // The moves of an evaluation in chunks of 32: alone (t == nullptr) in
 // order, or taken in turn from t->next by the owner and its helpers.
+// A unit is one move, in the double-float mode the two moves along one axis.
 template <class NT, bool NJ, bool NC>
 __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, const WarpMem& wm, const BlockMem& bm,
-                                              TeamSlot* t, int P, int lane)
+                                              const Lean& lt, TeamSlot* t, int units, int lane)
 {
   df* Td = reinterpret_cast<df*>(wm.T);
   // chunks of 16 moves in a team (more helpers take part in a small
@@ -1896,8 +1345,11 @@ __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, 
       if (lane == 0) c = atomicAdd(&t->next, cs);
       c0 = __shfl_sync(FULL_MASK, c, 0);
     }
-    if (c0 >= P) break;
-    if (lane < cs && c0 + lane < P) candidate_m<NT, NJ, NC>(S, L, wm, bm, c0 + lane, Td, nullptr);
+    if (c0 >= units) break;
+    if (lane < cs && c0 + lane < units) {
+      if (sizeof(NT) == sizeof(df)) moves64<NJ, NC>(S, L, wm, lt, c0 + lane, Td, nullptr);
+      else candidate_m<float, NJ>(S, L, wm, bm, c0 + lane, Td, nullptr);
+    }
   }
   if (t) __threadfence_block();
   __syncwarp();
@@ -1990,6 +1442,7 @@ struct WarpState {
   unsigned long long m;
   df bdf;
   int s, jumps, finish;
+  int fresh;  // no evaluation of this walker by this warp yet
   int owner, kidx, last;
 };
 static __shared__ WarpState g_ws[kMaxIntervalWarps];
@@ -2002,9 +1455,11 @@ template <class NT, int PR, bool NJ, bool NC>
 __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
                                               double* sC, uint64_t k, bool recompute, int lane, int wib)
 {
-  typedef Ar<NT> A;
   const int P_moves = S.N * 6 * L.G;
+  constexpr bool kDf = PR == LRDMC_PRECISION_DF64;
+  const int units = kDf ? P_moves / 2 : P_moves;
   const BlockMem bm = block_mem(S, sC);
+  const Lean lt = lean_mem(S, sC);
   TeamSlot* mine = &g_team[wib];
   WarpState& st = g_ws[wib];
   enum { kNeed, kOwner, kSearch, kHelper, kDone };
@@ -2033,11 +1488,14 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
           if (!ok && lane == 0) atomicOr(P.err, kErrSingular);
           if (lane == 0 && isfinite(rs)) atomicMax(P.resid, (unsigned long long)__double_as_longlong(rs));
         }
+        // the running sums of the cached rates, for the first heat bath
+        if (kDf) rate_scan64(reinterpret_cast<const df*>(wm.T), P_moves, lane, wm.pfx);
         if (lane == 0) {
           st.s = s;
           st.b = b;
           st.el = el;
-          st.bdf = df_from_double(b);
+          st.bdf = kDf ? dl_from_double(b) : df_from_double(b);
+          st.fresh = 1;
           st.tau_left = P.tau;
           st.logw = 0.0;
           st.jumps = 0;
@@ -2067,8 +1525,9 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
           b0[j] = shfl_u64(cb[j], 0);
           b1[j] = shfl_u64(cb[j], 1);
         }
-        if (PR == LRDMC_PRECISION_DF64)
-          t = b > 0.0 ? df_to_double(df_div(df_neg(df_log(df_u01(b0[0]), S.D.exp.K, bm.tab)), bdf)) : INFINITY;
+        if (kDf)
+          t = b > 0.0 ? df_to_double(dl_mul(dl_neg(dl_log(df_u01(b0[0]), S.D.lexp, lt.tab)), dl_norm(dl_rcp(bdf))))
+                      : INFINITY;
         else
           t = b > 0.0 ? (double)(-logf(f_u01(b0[0])) / bdf.hi) : INFINITY;
         if (t >= tau_left) {
@@ -2080,42 +1539,27 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       if (!over) {
         logw -= t * (el - P.e_trial);
         // heat bath over the cached rates
-        int lastc;
-        if (PR == LRDMC_PRECISION_DF64)
-          warp_scan_m<df>(reinterpret_cast<const df*>(wm.T), P_moves, lane, df_mul(df_u01(b0[1]), bdf), &pick,
-                          &lastc);
-        else
+        if (kDf) {
+          pick = heat_bath64(reinterpret_cast<const df*>(wm.T), P_moves, lane, wm.pfx,
+                             dl_norm(dl_mul(df_u01(b0[1]), bdf)));
+        } else {
+          int lastc;
           warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, f_u01(b0[1]) * bdf.hi, &pick,
                              &lastc);
-        if (pick < 0) pick = lastc;
+          if (pick < 0) pick = lastc;
+        }
         if (pick < 0) {  // no allowed move: cannot happen with b > 0
           if (lane == 0) atomicOr(P.err, kErrNonFinite);
           over = true;
         }
       }
-      double pnew[3];
       if (!over) {
         const int per_e = 6 * L.G;
         i = pick / per_e;
         const int rem = pick - i * per_e, g = rem / 6, kx = (rem % 6) >> 1;
         const double sign = (pick & 1) ? -1.0 : 1.0, h = g ? L.ap : L.a;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) pnew[d] = wm.x[3 * i + d] + sign * h * wm.R[3 * d + kx];
-        bool sm_ok;
-        if (PR != LRDMC_PRECISION_FP32) {
-          // the parity modes keep the update in IEEE double: near a node the
-          // update amplifies rounding by the condition number of the Slater
-          // matrix, and a double-float update (2^-48) parts trajectories
-          // from the FP64 reference in rare walkers
-          sm_ok = warp_sm_update<PR>(S, sC, wm, i, pnew, lane);
-        } else {
-          // the new position as a double-float (the shared-memory
-          // double-float copies of x and R belong to the last evaluation,
-          // which for the first jump of an interval may have been another
-          // walker's)
-          df pd[3] = {df_from_double(pnew[0]), df_from_double(pnew[1]), df_from_double(pnew[2])};
-          sm_ok = warp_sm_update_df(S, bm, wm, i, pd, lane);
-        }
+        // both arithmetics keep the update in IEEE double
+        const bool sm_ok = sm_update64(S, sC, wm, lt, i, sign * h, kx, lane);
         if (!sm_ok) {
           if (lane == 0) atomicOr(P.err, kErrSingular);
           over = true;
@@ -2139,13 +1583,18 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
         st.logw = logw;
         st.tau_left = tau_left - t;
       }
-      if (lane < 3) wm.x[3 * i + lane] = pnew[lane];
+      if (lane < 3) wm.x[3 * i + lane] = wm.sm[lane];
       __syncwarp();
-      rotation_matrix_warp<PR>(b1, wm.R, lane, S);
+      if (kDf) rotation64(b1, wm.R, lane, S);
+      else rotation_matrix_warp<PR>(b1, wm.R, lane, S);
       __syncwarp();
       double eln;
-      eval_prelude_m<NT, NJ, NC>(S, sC, L, wm, lane, eln);
-      if (lane == 0) st.el = eln;
+      if (kDf) eln = prelude64<NJ, NC>(S, sC, wm, lt, lane, st.fresh ? -1 : i);
+      else eln = prelude32<NJ>(S, sC, wm, lt, lane, st.fresh ? -1 : i);
+      if (lane == 0) {
+        st.el = eln;
+        st.fresh = 0;
+      }
       if (P.helpers) nh = team_publish(mine, lane);
     } else {
       if (mode == kSearch) {
@@ -2179,7 +1628,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
     // code for the owner alone, the owner with helpers, and the helpers
     {
       const WarpMem twm = warp_mem(Lo, S, sC + Lo.head + target * Lo.smem_warp);
-      chunked_moves<NT, NJ, NC>(S, L, twm, bm, (mode == kHelper || nh > 0) ? &g_team[target] : nullptr, P_moves,
+      chunked_moves<NT, NJ, NC>(S, L, twm, bm, lt, (mode == kHelper || nh > 0) ? &g_team[target] : nullptr, units,
                                 lane);
     }
     if (mode == kHelper) {
@@ -2188,11 +1637,14 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       continue;
     }
     if (nh > 0) team_wait_helpers(mine, nh, lane, P.err);
-    const NT btot = warp_scan_m<NT>(reinterpret_cast<const df*>(warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp).T),
-                                    P_moves, lane, A::zero(), nullptr, nullptr);
-    const double b = A::to_double(btot);
+    const WarpMem own = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
+    const df* Td = reinterpret_cast<const df*>(own.T);
+    df bnew;
+    if (kDf) bnew = rate_scan64(Td, P_moves, lane, own.pfx);
+    else bnew = df_make(warp_scan_m<float>(Td, P_moves, lane, 0.0f, nullptr, nullptr), 0.0f);
+    const double b = df_to_double(bnew);
     if (lane == 0) {
-      st.bdf = A::store(btot);
+      st.bdf = bnew;
       st.b = b;
       st.jumps = st.jumps + 1;
       int fin = 0;
@@ -2225,7 +1677,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
   constexpr int PR = PREC & 3;         // the arithmetic (LRDMC_PRECISION_*)
   constexpr bool NJ = (PREC & 8) != 0;  // the neural pair term is set
   constexpr bool NC = (PREC & 4) != 0;  // the layout has no evaluation caches
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
   // interval k from the device counter (advanced by k_comb_parents); the inverse
   // Slater matrices are recomputed at the start of every recompute_every-th
@@ -2240,7 +1692,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
     g_team[wib].done = 0;
     g_team[wib].gen = 0;
   }
-  stage_coefficients(S, sC);  // ends with __syncthreads
+  stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);  // ends with __syncthreads
   if constexpr (PR != LRDMC_PRECISION_FP64) {
     if (PR == LRDMC_PRECISION_DF64) interval_team<df, PR, NJ, NC>(S, Lo, L, P, sC, k, recompute, lane, wib);
     else interval_team<float, PR, NJ, true>(S, Lo, L, P, sC, k, recompute, lane, wib);
@@ -2248,7 +1700,6 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
     // the FP64 mode: every warp alone
     WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
     const int P_moves = S.N * 6 * L.G;
-    const BlockMem bm = block_mem(S, sC);
     for (;;) {
       int idx = 0;
       if (lane == 0) idx = atomicAdd(P.counter, 1);
@@ -2264,7 +1715,6 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
       const int src = bounded(P.parent[s], P.W, P.err);
       double b, el;
       load_record(Lo, P.rec_src + (size_t)src * Lo.rec, wm, lane, b, el);
-      df bdf = df_from_double(b);
       if (recompute) {
         double rs = 0.0;
         bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane, &rs);
@@ -2280,18 +1730,12 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
         uint64_t cb[4] = {(uint64_t)s, k, m, (lane & 1) ? kTagRot : kTagTimeHB};
         philox4x64_10(cb, P.seed, 0ull);
         uint64_t b0[4], b1[4];
-  #pragma unroll
+#pragma unroll
         for (int j = 0; j < 4; ++j) {
           b0[j] = shfl_u64(cb[j], 0);
           b1[j] = shfl_u64(cb[j], 1);
         }
-        double t;
-        if (PR == LRDMC_PRECISION_DF64)
-          t = b > 0.0 ? df_to_double(df_div(df_neg(df_log(df_u01(b0[0]), S.D.exp.K, bm.tab)), bdf)) : INFINITY;
-        else if (PR == LRDMC_PRECISION_FP32)
-          t = b > 0.0 ? (double)(-logf(f_u01(b0[0])) / bdf.hi) : INFINITY;
-        else
-          t = b > 0.0 ? -log(to_u01(b0[0])) / b : INFINITY;
+        const double t = b > 0.0 ? -log(to_u01(b0[0])) / b : INFINITY;
         if (t >= tau_left) {
           logw -= tau_left * (el - P.e_trial);
           break;
@@ -2300,12 +1744,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
         tau_left -= t;
         // heat bath over the cached rates
         int pick, last;
-        if (PR == LRDMC_PRECISION_DF64)
-          warp_scan_m<df>(reinterpret_cast<const df*>(wm.T), P_moves, lane, df_mul(df_u01(b0[1]), bdf), &pick, &last);
-        else if (PR == LRDMC_PRECISION_FP32)
-          warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, f_u01(b0[1]) * bdf.hi, &pick, &last);
-        else
-          warp_scan(wm.T, P_moves, lane, to_u01(b0[1]) * b, &pick, &last);
+        warp_scan(wm.T, P_moves, lane, to_u01(b0[1]) * b, &pick, &last);
         if (pick < 0) pick = last;
         if (pick < 0) {  // no allowed move: cannot happen with b > 0
           if (lane == 0) atomicOr(P.err, kErrNonFinite);
@@ -2315,22 +1754,9 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
         const int i = pick / per_e, rem = pick - i * per_e, g = rem / 6, kx = (rem % 6) >> 1;
         const double sign = (pick & 1) ? -1.0 : 1.0, h = g ? L.ap : L.a;
         double pnew[3];
-  #pragma unroll
+#pragma unroll
         for (int d = 0; d < 3; ++d) pnew[d] = wm.x[3 * i + d] + sign * h * wm.R[3 * d + kx];
-        bool sm_ok;
-        if (PR != LRDMC_PRECISION_FP32) {
-          // the parity modes keep the update in IEEE double: near a node the
-          // update amplifies rounding by the condition number of the Slater
-          // matrix, and a double-float update (2^-48) parts trajectories from
-          // the FP64 reference in rare walkers
-          sm_ok = warp_sm_update<PR>(S, sC, wm, i, pnew, lane);
-        } else {
-          // the new position as a double-float (the shared-memory double-float
-          // copies of x and R belong to the last evaluation, which for the
-          // first jump of an interval may have been another walker's)
-          df pd[3] = {df_from_double(pnew[0]), df_from_double(pnew[1]), df_from_double(pnew[2])};
-          sm_ok = warp_sm_update_df(S, bm, wm, i, pd, lane);
-        }
+        const bool sm_ok = warp_sm_update(S, sC, wm, i, pnew, lane);
         if (!sm_ok) {
           if (lane == 0) atomicOr(P.err, kErrSingular);
           break;
@@ -2339,7 +1765,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
         __syncwarp();
         rotation_matrix_warp<PR>(b1, wm.R, lane, S);
         __syncwarp();
-        warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, bdf, el);
+        warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, el);
         ++jumps;
         if (!isfinite(el) || !isfinite(b)) {
           if (lane == 0) atomicOr(P.err, kErrNonFinite);
@@ -2696,8 +2122,7 @@ __device__ __forceinline__ bool evaluate_config(const SysDev& S, const Layout& L
   if (!ok) return false;
   const int P = S.N * 6 * L.G;
   double b, el;
-  df bdf;
-  warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, ratio ? ratio + (size_t)c * P : nullptr, b, bdf, el);
+  warp_eval_any<PR, NJ, NC>(S, const_cast<double*>(sC), L, wm, lane, ratio ? ratio + (size_t)c * P : nullptr, b, el);
   if (T)
     for (int j = lane; j < P; j += 32)
       T[(size_t)c * P + j] = (PR != LRDMC_PRECISION_FP64) ? df_to_double(reinterpret_cast<const df*>(wm.T)[j])
@@ -2716,9 +2141,9 @@ k_evaluate(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, in
            const double* x, const double* rot, double* ratio, double* T, double* b_out,
            double* el_out, int* err)
 {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
-  stage_coefficients(S, sC);
+  stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int c = blockIdx.x * kWarpsPerBlock + wib;
   if (c >= n) return;
@@ -2757,9 +2182,22 @@ void fill_df_constants(SysDev& S)
       D.sh[q].coef[p] = split_ld(S.sh[q].coef[p]);
     }
   }
+  // e-e part: the reciprocal form needs b away from zero (its terms c/b q
+  // would lose log2(c/b) bits) and positive (1 + b r > 0)
+  const double bs = S.b_ee != 0.0 ? fabs(S.b_ee) : 1.0;
+  S.ee_recip = S.b_ee >= 0.25 ? 1 : 0;
+  S.ee_sign = S.b_ee > 0.0 ? 1.0f : (S.b_ee < 0.0 ? -1.0f : 0.0f);
+  D.ee_scale = split_ld(bs);
+  D.ee_scale2 = split_ld((long double)bs * bs);
+  D.ee_iscale = split_ld(1.0L / bs);
+  D.ee_factor = split_ld((S.ee_recip ? -1.0L : 1.0L) / bs);
   // Tang's table: 2^(j/64) and ln2/64, from long double arithmetic
   const long double ln2 = logl(2.0L);
-  df c = split_ld(ln2 / 64.0L);
+  df c = split_ld(ln2 / kExpEntries);
+  D.lexp.c_hi = c.hi;
+  D.lexp.c_lo = c.lo;
+  D.lexp.inv = (float)(kExpEntries / ln2);
+  c = split_ld(ln2 / 64.0L);
   D.exp.K.ln2_64_hi = c.hi;
   D.exp.K.ln2_64_lo = c.lo;
   D.exp.K.inv_ln2_64 = (float)(64.0L / ln2);
@@ -2804,25 +2242,32 @@ Layout make_layout(const SysDev& S, bool caches)
   Lo.off_el = Lo.off_b + 1;
   Lo.rec = (Lo.off_el + 1 + 3) & ~3;
   const int n = S.n_up;
-  int scr = 2 * n * n + n * S.n_ao;          // Gauss-Jordan + orbital rows
-  int scr_sm = S.n_ao + 3 * n + n * n;       // Sherman-Morrison (FP64 or double-float)
-  if (scr_sm > scr) scr = scr_sm;
+  Lo.n_scr = 2 * n * n + n * S.n_ao;                         // Gauss-Jordan + orbital rows
+  Lo.n_scr = std::max(Lo.n_scr, S.n_ao + 3 * n + n * n);     // Sherman-Morrison (FP64 or FP32 mode)
   // The caches of the double-float evaluation (omitted when caches is false):
-  // the electron-nucleus cache (8 df per electron and nucleus), and the pair
-  // cache up to 24 electrons (beyond, its 4 df per pair would cost blocks
-  // per SM), with room for the pair's Jastrow terms up to 12 electrons (used
-  // with the neural term: the local energy then evaluates every pair once)
-  Lo.n_pc = (caches && S.N <= 24) ? S.N * (S.N - 1) / 2 : 0;
-  Lo.pcw = S.N <= 12 ? 8 : 4;
+  // the electron-nucleus cache (8 df per electron and nucleus), and one
+  // squared distance per electron pair up to 40 electrons (beyond, the cache
+  // would cost warps per SM)
+  Lo.n_pc = (caches && S.N <= 40) ? S.N * (S.N - 1) / 2 : 0;
   Lo.enc = caches ? 1 : 0;
-  Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + S.N * S.n_ao + S.N +
-                 (3 * S.N + 12) + Lo.pcw * Lo.n_pc + (Lo.enc ? 8 * S.N * S.n_nuc : 0) + scr;
+  const int state = S.N * S.n_ao + 2 * S.N + 6 * S.N + 12 + 32 + (Lo.enc ? 8 * S.N * S.n_nuc : 0) + Lo.n_pc;
+  Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + 4 + S.n_ao + 3 * n +
+                 std::max(Lo.n_scr, state);
   Lo.smem_warp = (Lo.smem_warp + 1) & ~1;
-  Lo.head = ((2 * S.n_ao * S.n_mo + (S.n_ao * S.n_mo + 1) / 2 + 64) + 1) & ~1;
+  Lo.head = lean_offset(S) + kExpEntries + 2 * S.n_prim + (int)(sizeof(LShell) / sizeof(double)) * S.n_shell;
   Lo.smem_block_bytes = (int)sizeof(double) * (Lo.head + kWarpsPerBlock * Lo.smem_warp);
   return Lo;
 }
 
+int accept_smem_bytes(const SysDev& S, bool caches)
+{
+  const int n = S.n_up;
+  const int scr = std::max(2 * n * n + n * S.n_ao, S.n_ao + 3 * n + n * n);
+  int warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + 12 * S.N + S.N * S.n_ao + S.N + (3 * S.N + 12) + scr;
+  if (caches) warp += (S.N <= 24 ? S.N * (S.N - 1) / 2 * (S.N <= 12 ? 8 : 4) : 0) + 8 * S.N * S.n_nuc;
+  warp = (warp + 1) & ~1;
+  return (int)sizeof(double) * (lean_offset(S) + kWarpsPerBlock * warp);
+}
 #endif  // LRDMC_PART == 0
 
 static cudaError_t set_smem(const void* fn, int bytes)
@@ -2974,9 +2419,9 @@ k_evaluate_static(const __grid_constant__ SysDev S, const Layout Lo, const LatDe
                   const double* x, const double* rot, double* ratio, double* T, double* b_out,
                   double* el_out, int* scratch)
 {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
-  stage_coefficients(S, sC);
+  stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int c = blockIdx.x * kWarpsPerBlock + wib;
   if (c >= n) return;
@@ -3049,15 +2494,14 @@ cudaError_t launch_eval_all(const SysDev& S, const Layout& Lo, const LatDev& L, 
 
 // Warps per block of the interval kernel: 16 (so that the warps of an SM,
 // one block, can help one another at the end of an interval), halved while
-// the population cannot give every warp of every SM a walker or the block's
-// shared memory does not fit; at least the other kernels' four.
+// the population cannot give every warp of every SM a walker, then as many
+// as the shared memory holds; at least the other kernels' four.
 int interval_warps(const Layout& Lo, int W)
 {
   const int sms = sm_count_current();
   int w = kMaxIntervalWarps;
-  while (w > kWarpsPerBlock &&
-         ((int)sizeof(double) * (Lo.head + w * Lo.smem_warp) > kMaxSmemBlock || W < sms * w))
-    w >>= 1;
+  while (w > kWarpsPerBlock && W < sms * w) w >>= 1;
+  while (w > kWarpsPerBlock && (int)sizeof(double) * (Lo.head + w * Lo.smem_warp) > kMaxSmemBlock) --w;
   return w;
 }
 
@@ -3119,7 +2563,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 k_base_terms(const __grid_constant__ SysDev S, const Layout Lo, int n, const double* x, double* grad,
              double* e, int* err)
 {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   double* sC = smem;
   stage_coefficients(S, sC);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -3338,7 +2782,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
 {
   constexpr bool NJ = (PREC & 8) != 0;
   typedef Ar<float> A;
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) double smem[];
   __shared__ __align__(8) uint64_t s_mbar;
   __shared__ uint32_t s_tmem;
   __shared__ int s_bad;
@@ -3350,7 +2794,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
   char* Al = Ah + tileA;
   char* Bh = Al + tileA;
   char* Bl = Bh + tileB;
-  stage_coefficients(S, sC);
+  stage_coefficients<true>(S, sC);
   const BlockMem bm = block_mem(S, sC);
   // B = C^T (orbital m, AO k), split into bfloat16 high and low parts
   for (int idx = tid; idx < kTcN * Kp; idx += blockDim.x) {
@@ -3390,7 +2834,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
     ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane);
     ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane);
     if (!ok && lane == 0) atomicOr(err, kErrSingular);
-    if (ok) warp_eval_m<float, NJ, true, false>(S, sC, L, wm, lane, nullptr, b, bdf, el);
+    if (ok) el = prelude32<NJ>(S, sC, wm, lean_mem(S, sC), lane, -1);
   }
   const int N = S.N, G = L.G, per_e = 6 * G, P = N * per_e;
   const int rounds = (P + 31) / 32;
@@ -3499,10 +2943,15 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
 static int tc_tile_offset(const Layout& Lo) { return (Lo.smem_block_bytes + 127) & ~127; }
 static int tc_smem_bytes(const Layout& Lo, int Kp) { return tc_tile_offset(Lo) + 2 * (kTcRows + kTcN) * Kp * 2; }
 
+// The same beside the acceptance layout (its caches where they fit): what
+// decides whether a system can use the tensor-core evaluation.
 int evaluate_tc_smem_bytes(const SysDev& S, const Layout& Lo)
 {
   const int Kp = (S.n_ao + 15) & ~15;
-  return tc_smem_bytes(Lo, Kp);
+  Layout La = Lo;
+  La.smem_block_bytes = accept_smem_bytes(S, true);
+  if (La.smem_block_bytes > kMaxSmemBlock) La.smem_block_bytes = accept_smem_bytes(S, false);
+  return std::max(tc_smem_bytes(Lo, Kp), tc_smem_bytes(La, Kp));
 }
 
 cudaError_t launch_evaluate_tc(const SysDev& S, const Layout& Lo, const LatDev& L, int n, const double* x,
