@@ -62,8 +62,10 @@ __device__ __forceinline__ void lean_stage(const SysDev& S, double* head)
 {
   const Lean m = lean_mem(S, head);
   float4* tab = reinterpret_cast<float4*>(const_cast<float2*>(m.tab));
+#pragma unroll 1
   for (int j = threadIdx.x; j < kExpEntries / 2; j += blockDim.x)
     tab[j] = __ldg(reinterpret_cast<const float4*>(g_exp_tab) + j);
+#pragma unroll 1
   for (int q = threadIdx.x; q < S.n_shell; q += blockDim.x) {
     LShell* o = const_cast<LShell*>(m.sh) + q;
     const ShellDev& sh = S.sh[q];
@@ -72,6 +74,7 @@ __device__ __forceinline__ void lean_stage(const SysDev& S, double* head)
     o->prim = sh.prim_begin; o->n_prim = sh.n_prim; o->same_exp = sh.same_exp; o->center = sh.center;
     o->zeta_hi = d.zeta.hi; o->zeta_lo = d.zeta.lo; o->m_hi = d.m.hi; o->m_lo = d.m.lo;
     float4* pr = const_cast<float4*>(m.prim) + sh.prim_begin;
+#pragma unroll 1
     for (int p = 0; p < sh.n_prim; ++p)
       pr[p] = make_float4(d.alpha[p].hi, d.alpha[p].lo, d.coef[p].hi, d.coef[p].lo);
   }
@@ -102,16 +105,23 @@ __device__ __forceinline__ int pair_q(const SysDev& S, int i, int j)
   return tu + nd * (nd - 1) / 2 + a * nd + (b - nu);
 }
 
+// r^m = e^(m log r) (out of line: one copy of code that few systems run)
+static __device__ __noinline__ dl real_power(dl m, dl r, const LeanExp K, const float2* tab)
+{
+  return dl_norm(dl_exp(dl_norm(dl_mul(m, dl_log(dl_norm(r), K, tab))), K, tab));
+}
+
 // r^m for a Slater shell: a small whole power, or e^(m log r)
 __device__ __forceinline__ dl slater_power(const LShell& sh, dl r, const SysDev& S, const Lean& t)
 {
   if (sh.m_int == 1) return r;
   if (sh.m_int >= 0) {
     dl p = df_make(1.0f, 0.0f);
+#pragma unroll 1
     for (int j = 0; j < sh.m_int; ++j) p = dl_mul(p, r);
     return dl_norm(p);
   }
-  return dl_exp(dl_norm(dl_mul(df_make(sh.m_hi, sh.m_lo), dl_log(dl_norm(r), S.D.lexp, t.tab))), S.D.lexp, t.tab);
+  return real_power(df_make(sh.m_hi, sh.m_lo), r, S.D.lexp, t.tab);
 }
 
 // The five degree-2 solid harmonics of d contracted with v.
@@ -188,6 +198,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
   const dl zero = df_make(0.0f, 0.0f);
   const bool recip = S.ee_recip != 0;
   dl total = zero;
+#pragma unroll 1
   for (int i0 = 0; i0 < N; i0 += E) {
     const int i = i0 + lane - part * E;
     const bool act = part < L && i < N;
@@ -199,7 +210,9 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
       dl lap = zero;
       int pc = -1;
       dl d[3], r2 = zero, r = zero, ir = zero, e = zero;
+#pragma unroll 1
       for (int gi = part; gi < S.n_grp64; gi += L)
+#pragma unroll 1
         for (int q = S.grp64_first[gi]; q < S.grp64_first[gi + 1]; ++q) {
           const LShell sh = lt.sh[q];
           if (sh.center != pc) {
@@ -220,6 +233,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
             R2 = dl_mul_n(dl_sub_n(dl_sqr(t), dl_mul(mir, ir)), R);
           } else {
             dl A0 = zero, A1 = zero, A2 = zero;
+#pragma unroll 1
             for (int p = 0; p < sh.n_prim; ++p) {
               const float4 pr = lt.prim[sh.prim + p];
               const dl al = dl_at(pr, 0);
@@ -263,6 +277,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
       // (b: the scale; sb its sign or 0 in the general form)
       dl lap2 = zero, pot = zero, snj = zero;
       const int si = spin_of(S, i);
+#pragma unroll 1
       for (int t = part; t < N - 1; t += L) {
         const int j = t < i ? t : t + 1;
         dl dd[3], D;
@@ -302,6 +317,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
       for (int k = 0; k < 3; ++k) gJ[k] = dl_mul(dl_norm(gJ[k]), S.D.ee_scale);
       dl lin = S.ee_on ? dl_mul(dl_norm(pot), S.D.ee_scale) : zero;
       // e-n terms
+#pragma unroll 1
       for (int I = part; I < S.n_nuc; I += L) {
         dl dd[3], D;
         en_geometry(S, wm, i, I, dd, D);
@@ -329,6 +345,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
     }
     // combine the parts of each electron (lane part * E + i)
     if (L > 1) {
+#pragma unroll 1
       for (int o = S.el_top; o > 0; o >>= 1) {
         const bool take = part < o && part + o < L;
         const int sh = o * E;
@@ -372,32 +389,35 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
                                             int lane, int moved)
 {
   const int N = S.N, nao = S.n_ao, nu = S.n_up, nd = S.n_dn;
+  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
   int lo = 0, hi = N;
   if (moved >= 0) {
     lo = moved < nu ? 0 : nu;
     hi = moved < nu ? nu : N;
   }
+#pragma unroll 1
   for (int idx = lo * nao + lane; idx < hi * nao; idx += 32) {
     const int i = idx / nao, mu = idx - i * nao;
     const int l = i < nu ? i : i - nu, n = i < nu ? nu : nd;
     const double* Am = i < nu ? wm.A : wm.A + nu * nu;
-    double acc = 0.0;
-    for (int m = 0; m < n; ++m) acc += sC[mu * S.n_mo + m] * Am[m * n + l];
-    wm.vd[idx] = dl_from_double(acc);
+    wm.vd[idx] = dl_from_double(project_ao(S, bm, Am, mu, l, n));
   }
   if (moved < 0) {
+#pragma unroll 1
     for (int j = lane; j < 3 * N; j += 32) wm.xd[j] = dl_from_double(wm.x[j]);
   } else if (lane < 3) {
     wm.xd[3 * moved + lane] = dl_from_double(wm.x[3 * moved + lane]);
   }
   if (lane < 9) wm.Rd[lane] = dl_from_double(wm.R[lane]);
   __syncwarp();
+#pragma unroll 1
   for (int j = lane; MOVES && j < 3 * N; j += 32) {
     const int i = j / 3, k = j - 3 * i;
     const dl x[3] = {wm.xd[3 * i], wm.xd[3 * i + 1], wm.xd[3 * i + 2]};
     wm.y[j] = dl_norm(dl_mul(axis_dot(wm, k, x), S.D.ee_scale));
   }
   if (MOVES && !NC) {
+#pragma unroll 1
     for (int q = lane; q < N * S.n_nuc; q += 32) {
       const int i = q / S.n_nuc, I = q - i * S.n_nuc;
       dl d[3], D;
@@ -414,6 +434,7 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
       dl d[3];
       if (moved < 0) {
         const int tu = nu * (nu - 1) / 2, td = nd * (nd - 1) / 2;
+#pragma unroll 1
         for (int q = lane; q < wm.n_pc; q += 32) {
           int i, j;
           if (q < tu + td) {
@@ -433,6 +454,7 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
           wm.pc[q] = pair_d2(S, wm, i, j, d);
         }
       } else {
+#pragma unroll 1
         for (int t = lane; t < N - 1; t += 32) {
           const int j = t < moved ? t : t + 1;
           wm.pc[pair_q(S, moved, j)] = pair_d2(S, wm, moved, j, d);
@@ -481,6 +503,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
   {
     const dl h2 = dl_sqr(h);
     const dl he[3] = {dl_mul(h, wm.Rd[k]), dl_mul(h, wm.Rd[3 + k]), dl_mul(h, wm.Rd[6 + k])};
+#pragma unroll 1
     for (int I = 0; I < S.n_nuc; ++I) {
       dl d[3], D, hp;
       if (NC) {
@@ -522,6 +545,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
 #pragma unroll
         for (int m = 0; m < 2; ++m) jn[m] = dl_add(jn[m], nj_value64(S, 2 + S.nj_species[I], r[m]));
       }
+#pragma unroll 1
       for (int q = S.nuc_shell_begin[I]; q < S.nuc_shell_begin[I + 1]; ++q) {
         const LShell sh = lt.sh[q];
         dl R[2];
@@ -535,6 +559,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
           for (int m = 0; m < 2; ++m) R[m] = sh.m_int == 0 ? e[m] : dl_mul(slater_power(sh, r[m], S, lt), e[m]);
         } else {
           R[0] = R[1] = zero;
+#pragma unroll 1
           for (int p = 0; p < sh.n_prim; ++p) {
             const float4 pr = lt.prim[sh.prim + p];
             const dl al = df_make(-pr.x, -pr.y), co = df_make(pr.z, pr.w);
@@ -577,6 +602,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
     acc[0] = acc[1] = df_make(start, 0.0f);
     int qq = tri + l * (l - 1) / 2;
     dl dd[3];
+#pragma unroll 1
     for (int t = 0; t < n_same - 1; ++t) {
       const int jl = t < l ? t : t + 1, j = off_same + jl;
       dl D;
@@ -600,6 +626,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
     const int opp = nu * (nu - 1) / 2 + S.n_dn * (S.n_dn - 1) / 2;
     int qo = up ? opp + l * S.n_dn : opp + l;
     const int dq = up ? 1 : S.n_dn;
+#pragma unroll 1
     for (int t = 0; t < n_opp; ++t) {
       const int j = off_opp + t;
       dl D;
@@ -652,6 +679,7 @@ __device__ __forceinline__ dl rate_scan64(const df* T, int P, int lane, df* pfx)
 {
   const int run = (P + 31) >> 5, c0 = lane * run;
   dl v = df_make(0.0f, 0.0f);
+#pragma unroll 1
   for (int q = 0; q < run; ++q)
     if (c0 + q < P) v = dl_add_n(v, T[c0 + q]);
 #pragma unroll
@@ -676,49 +704,68 @@ __device__ __forceinline__ int heat_bath64(const df* T, int P, int lane, const d
   const int L = hit ? __ffs(hit) - 1 : 31;
   const int c0 = L * run, c1 = min(P, c0 + run);
   dl C = L > 0 ? pfx[L - 1] : df_make(0.0f, 0.0f);
+#pragma unroll 1
   for (int c = c0; c < c1; ++c) {
     C = dl_add_n(C, T[c]);
     if (dl_lt(target, C)) return c;
   }
+#pragma unroll 1
   for (int c = c1 - 1; c >= 0; --c)
     if (T[c].hi > 0.0f) return c;
   return -1;
 }
 
-// New rotation from three uniforms: lanes 0-3 form sqrt(1 - u1), sqrt(u1),
-// sincospi(2 u2), sincospi(2 u3), lanes 0-8 one matrix entry each.
-__device__ __forceinline__ void rotation64(const uint64_t* bits, double* R, int lane, const SysDev& S)
+// The random numbers of iterations m0 .. m0 + kDrawAhead - 1 of a walker's
+// interval, one iteration per lane: lanes 0-15 the waiting time's -log u and
+// the heat bath's uniform, lanes 16-31 the rotation (Shoemake's quaternion
+// from three uniforms). Per iteration dr holds R[9], then the two
+// double-floats. A walker makes about ten jumps per interval, so one pass
+// replaces ten in which 30 lanes idled (10 k of 78 k cycles per Ne move).
+__device__ __forceinline__ void draw_ahead64(uint64_t seed, uint64_t slot, uint64_t k, uint64_t m0, double* dr,
+                                             int lane, const SysDev& S, const Lean& lt)
 {
-  dl a = df_make(0.0f, 0.0f), c = a;
-  if (lane < 2) {
-    const dl u = df_u01(bits[0]);
-    a = dl_norm(dl_sqrt_acc(lane == 0 ? dl_norm(dl_add_f(dl_neg(u), 1.0f)) : u));
-  } else if (lane < 4) {
-    dl_sincospi(dl_scale(df_u01(bits[lane - 1]), 2.0f), S.D.inv_fact, S.D.half_pi, &a, &c);
+  static_assert(kDrawAhead == 16, "half a warp per tag");
+  uint64_t c[4] = {slot, k, m0 + (lane & 15), lane < 16 ? kTagTimeHB : kTagRot};
+  philox4x64_10(c, seed, 0ull);
+  double* o = dr + (lane & 15) * kDrawWords;
+  __syncwarp();
+  if (lane < 16) {
+    df* od = reinterpret_cast<df*>(o);
+    od[9] = dl_neg(dl_log(df_u01(c[0]), S.D.lexp, lt.tab));
+    od[10] = df_u01(c[1]);
+  } else {
+    const dl u = df_u01(c[0]);
+    const dl s1 = dl_norm(dl_sqrt_acc(dl_norm(dl_add_f(dl_neg(u), 1.0f)))), s2 = dl_norm(dl_sqrt_acc(u));
+    dl q[4];  // x, y, z, w
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      dl a, b;
+      dl_sincospi(dl_scale(df_u01(h ? c[2] : c[1]), 2.0f), S.D.inv_fact, S.D.half_pi, &a, &b);
+      const dl sh = h ? s2 : s1;
+      a = dl_mul(sh, dl_norm(a));
+      b = dl_mul(sh, dl_norm(b));
+      if (h) { q[2] = a; q[3] = b; }
+      else { q[0] = a; q[1] = b; }
+    }
+    // R00 = 1 - 2(yy + zz)  R01 = 2(xy - zw)  R02 = 2(xz + yw)
+    // R10 = 2(xy + zw)  R11 = 1 - 2(xx + zz)  R12 = 2(yz - xw)
+    // R20 = 2(xz - yw)  R21 = 2(yz + xw)  R22 = 1 - 2(xx + yy)
+    const dl xx = dl_sqr(q[0]), yy = dl_sqr(q[1]), zz = dl_sqr(q[2]);
+    const dl xy = dl_mul(q[0], q[1]), xz = dl_mul(q[0], q[2]), yz = dl_mul(q[1], q[2]);
+    const dl xw = dl_mul(q[0], q[3]), yw = dl_mul(q[1], q[3]), zw = dl_mul(q[2], q[3]);
+    auto off = [](dl a, dl b) { return df_to_double(dl_scale(dl_add_n(a, b), 2.0f)); };
+    auto diag = [](dl a, dl b) { return df_to_double(dl_norm(dl_add_f(dl_scale(dl_add_n(a, b), -2.0f), 1.0f))); };
+    o[0] = diag(yy, zz);
+    o[1] = off(xy, dl_neg(zw));
+    o[2] = off(xz, yw);
+    o[3] = off(xy, zw);
+    o[4] = diag(xx, zz);
+    o[5] = off(yz, dl_neg(xw));
+    o[6] = off(xz, dl_neg(yw));
+    o[7] = off(yz, xw);
+    o[8] = diag(xx, yy);
   }
-  auto get = [](dl v, int src) {
-    return df_make(__shfl_sync(FULL_MASK, v.hi, src), __shfl_sync(FULL_MASK, v.lo, src));
-  };
-  const dl s1 = get(a, 0), s2 = get(a, 1), sa = get(a, 2), ca = get(c, 2), sb = get(a, 3), cb = get(c, 3);
-  const dl q0 = dl_mul(s1, dl_norm(sa)), q1 = dl_mul(s1, dl_norm(ca)), q2 = dl_mul(s2, dl_norm(sb)),
-           q3 = dl_mul(s2, dl_norm(cb));  // x, y, z, w
-  // entry (row, col) = lane: delta + 2 (q_a q_b +- q_c q_d)
-  //   R00 = 1 - 2(yy + zz)  R01 = 2(xy - zw)  R02 = 2(xz + yw)
-  //   R10 = 2(xy + zw)  R11 = 1 - 2(xx + zz)  R12 = 2(yz - xw)
-  //   R20 = 2(xz - yw)  R21 = 2(yz + xw)  R22 = 1 - 2(xx + yy)
-  const int l = lane < 9 ? lane : 0;
-  const unsigned long long ka = 0x10100001ull, kb = 0x22201211ull;
-  const unsigned long long kc = 0x101022122ull, kd = 0x133323332ull;
-  auto pick = [&](unsigned long long key) {
-    const unsigned k = (unsigned)(key >> (4 * l)) & 0xF;
-    const dl x = (k & 1) ? q1 : q0, y = (k & 1) ? q3 : q2;
-    return (k & 2) ? y : x;
-  };
-  const bool diag = l == 0 || l == 4 || l == 8, minus = l == 1 || l == 5 || l == 6;
-  const dl t1 = dl_mul(pick(ka), pick(kb)), t2 = dl_mul(pick(kc), pick(kd));
-  dl v = dl_scale(dl_add_n(t1, minus ? dl_neg(t2) : t2), diag ? -2.0f : 2.0f);
-  if (diag) v = dl_norm(dl_add_f(v, 1.0f));
-  if (lane < 9) R[lane] = df_to_double(v);
+  __syncwarp();
 }
 
 // Sherman-Morrison update for electron i jumping by sign h along axis kx, in
@@ -732,6 +779,7 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
 {
   const int nu = S.n_up, nao = S.n_ao;
   const int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
+  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
   double* A = spin ? wm.A + nu * nu : wm.A;
   double* pn = wm.sm;          // [4]
   double* chi = pn + 4;        // [n_ao] (double-float, then double)
@@ -742,6 +790,7 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
   __syncwarp();
   const dl pd[3] = {dl_from_double(pn[0]), dl_from_double(pn[1]), dl_from_double(pn[2])};
   df* cd = reinterpret_cast<df*>(chi);
+#pragma unroll 1
   for (int q = lane; q < S.n_shell; q += 32) {
     const LShell sh = lt.sh[q];
     dl d[3];
@@ -755,6 +804,7 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
       if (sh.m_int != 0) R = dl_mul(slater_power(sh, r, S, lt), R);
     } else {
       R = df_make(0.0f, 0.0f);
+#pragma unroll 1
       for (int p = 0; p < sh.n_prim; ++p) {
         const float4 pr = lt.prim[sh.prim + p];
         R = dl_add(R, dl_mul(df_make(pr.z, pr.w),
@@ -778,16 +828,18 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
     }
   }
   __syncwarp();
+#pragma unroll 1
   for (int mu = lane; mu < nao; mu += 32) chi[mu] = df_to_double(cd[mu]);
   __syncwarp();
+#pragma unroll 1
   for (int m = lane; m < n; m += 32) {
-    double a = 0.0;
-    for (int mu = 0; mu < nao; ++mu) a += sC[mu * S.n_mo + m] * chi[mu];
-    phi[m] = a;
+    phi[m] = orbital_value(S, bm, chi, m);
   }
   __syncwarp();
+#pragma unroll 1
   for (int q = lane; q < n; q += 32) {
     double a = 0.0;
+#pragma unroll 1
     for (int m = 0; m < n; ++m) a += phi[m] * A[m * n + q];
     y[q] = a;
     col[q] = A[q * n + l];
@@ -797,8 +849,10 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
   if (ratio == 0.0) return false;
   const double inv = 1.0 / ratio;
   __syncwarp();
+#pragma unroll 1
   for (int q = lane; q < n; q += 32) y[q] = (y[q] - (q == l ? 1.0 : 0.0)) * inv;
   __syncwarp();
+#pragma unroll 1
   for (int idx = lane; idx < n * n; idx += 32) {
     const int m = idx / n, q = idx - m * n;
     A[idx] -= col[m] * y[q];
@@ -811,6 +865,7 @@ __device__ __forceinline__ bool sm_update64(const SysDev& S, const double* sC, c
 // single-precision moves compare with), in place of the e-e sums.
 __device__ __forceinline__ void total_jastrow64(const SysDev& S, const WarpMem& wm, int lane)
 {
+#pragma unroll 1
   for (int i = lane; i < S.N; i += 32) {
     const int n_same = (i < S.n_up ? S.n_up : S.n_dn) - 1, n_opp = i < S.n_up ? S.n_dn : S.n_up;
     dl s = wm.Sd[i];
@@ -830,6 +885,7 @@ __device__ void warp_eval64(const SysDev& S, double* sC, const LatDev& L, const 
   el = prelude64<NJ, NC>(S, sC, wm, lt, lane, -1);
   const int units = 3 * L.G * S.N;
   df* Td = reinterpret_cast<df*>(wm.T);
+#pragma unroll 1
   for (int u = lane; u < units; u += 32) moves64<NJ, NC>(S, L, wm, lt, u, Td, ratio_out);
   __syncwarp();
   b = df_to_double(rate_scan64(Td, 2 * units, lane, wm.pfx));

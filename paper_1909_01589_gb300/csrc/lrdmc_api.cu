@@ -30,11 +30,21 @@ struct NvtxRange {
 }  // namespace
 
 
+// Quadrature of Eq. 7 for one Z (core_quadrature).
+constexpr int kPanels = 240, kPanelNodes = 24;
+struct CoreQuadrature {
+  int Z = 0;
+  double edge[kPanels + 1];           // panel limits
+  std::vector<double> r, w, f;        // nodes, weights, density
+  std::vector<double> later;          // largest w f from a panel on
+};
+
 struct lrdmc_system_s {
   SysDev S;
   Layout Lo;
   double Zmax;
   int iZmax;
+  CoreQuadrature core;
   // population
   int W = 0;
   int trace_cap = 0;
@@ -177,29 +187,61 @@ static void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w
 // Eq. 7: N_core(r_c) = int 4 pi r^2 rho_eff(r) exp(-r^2/(2 r_c^2)) dr with
 // rho_eff from Slater's effective orbitals (normalised r^(n*-1) e^(-zeta r)).
 // Composite 24-point Gauss-Legendre on 240 panels clustered towards r = 0.
-static double n_core(int Z, double rc)
+// The density at the nodes depends on Z only, so a system keeps it and each
+// lattice costs the Gaussian factors: 5760 nodes with two to five logarithms
+// and exponentials each took 0.2 to 0.7 ms of every call that names this
+// lattice, as long as a small evaluation takes on the GPU.
+static void core_quadrature(CoreQuadrature& c, int Z)
 {
   auto g = slater_groups(Z);
   double zmin = 1e300;
-  for (auto& q : g) zmin = fmin(zmin, q.zeta);
+  std::vector<double> lognorm;
+  for (auto& q : g) {
+    zmin = fmin(zmin, q.zeta);
+    lognorm.push_back((2.0 * q.nstar + 1.0) * log(2.0 * q.zeta) - lgamma(2.0 * q.nstar + 1.0));
+  }
   std::vector<double> gx, gw;
-  gauss_legendre(24, gx, gw);
+  gauss_legendre(kPanelNodes, gx, gw);
   const double rmax = 90.0 / zmin;
-  const int panels = 240;
-  double total = 0.0;
-  for (int p = 0; p < panels; ++p) {
-    double t0 = (double)p / panels, t1 = (double)(p + 1) / panels;
+  c.r.clear();
+  c.w.clear();
+  c.f.clear();
+  for (int p = 0; p < kPanels; ++p) {
+    double t0 = (double)p / kPanels, t1 = (double)(p + 1) / kPanels;
     double r0 = rmax * t0 * t0, r1 = rmax * t1 * t1;
     double half = 0.5 * (r1 - r0), mid = 0.5 * (r1 + r0);
-    for (int i = 0; i < 24; ++i) {
-      double r = mid + half * gx[i];
+    c.edge[p] = r0;
+    c.edge[p + 1] = r1;
+    for (int i = 0; i < kPanelNodes; ++i) {
+      double r = mid + half * gx[i], lr = log(r);
       double f = 0.0;
-      for (auto& q : g) {
-        double lognorm = (2.0 * q.nstar + 1.0) * log(2.0 * q.zeta) - lgamma(2.0 * q.nstar + 1.0);
-        f += q.occ * exp(lognorm + 2.0 * q.nstar * log(r) - 2.0 * q.zeta * r);
-      }
-      if (rc > 0.0 && isfinite(rc)) f *= exp(-r * r / (2.0 * rc * rc));
-      total += half * gw[i] * f;
+      for (size_t q = 0; q < g.size(); ++q) f += g[q].occ * exp(lognorm[q] + 2.0 * g[q].nstar * lr - 2.0 * g[q].zeta * r);
+      c.r.push_back(r);
+      c.w.push_back(half * gw[i]);
+      c.f.push_back(f);
+    }
+  }
+  c.later.assign(kPanels + 1, 0.0);
+  for (int p = kPanels - 1; p >= 0; --p) {
+    c.later[p] = c.later[p + 1];
+    for (int i = 0; i < kPanelNodes; ++i)
+      c.later[p] = fmax(c.later[p], c.w[p * kPanelNodes + i] * c.f[p * kPanelNodes + i]);
+  }
+  c.Z = Z;
+}
+
+static double n_core(CoreQuadrature& c, int Z, double rc)
+{
+  if (c.Z != Z) core_quadrature(c, Z);
+  const bool gauss = rc > 0.0 && isfinite(rc);
+  double total = 0.0;
+  for (int p = 0; p < kPanels; ++p) {
+    // every later term is below half a unit in the last place of the sum
+    if (gauss && c.later[p] * exp(-c.edge[p] * c.edge[p] / (2.0 * rc * rc)) < 0x1p-55 * total) break;
+    for (int i = p * kPanelNodes; i < (p + 1) * kPanelNodes; ++i) {
+      double f = c.f[i];
+      if (gauss) f *= exp(-c.r[i] * c.r[i] / (2.0 * rc * rc));
+      total += c.w[i] * f;
     }
   }
   return total;
@@ -225,7 +267,7 @@ static lrdmc_status lattice_from(lrdmc_system_t s, double a, const lrdmc_spacing
       if (s->iZmax < 1 || fabs(s->Zmax - s->iZmax) > 1e-12)
         return fail(s, LRDMC_ERR_ARG, "THIS_WORK needs an integer Z_max (Slater's rules)");
       rc = rc_s13(a, s->Zmax, sp->beta, sp->kappa);
-      double nc = n_core(s->iZmax, rc);
+      double nc = n_core(s->core, s->iZmax, rc);
       ratio = sqrt((s->Zmax - nc) / nc);
       L.pkind = 0;
       break;
@@ -428,6 +470,12 @@ lrdmc_status lrdmc_create_system(int n_nuc, const double* nuc_xyz, const double*
       for (int m = 0; m < n_mo; ++m)
         S.C[(S.sh[qs].ao_offset + f) * n_mo + m] = mo_coeff[(user_off[q] + f) * n_mo + m];
   }
+  for (int mu = 0; mu < n_ao; ++mu)
+    for (int m = 0; m < n_mo; ++m)
+      if (S.C[mu * n_mo + m] != 0.0) {
+        S.row_mask[mu] |= 1u << m;
+        S.col_mask[m] |= 1ull << mu;
+      }
   S.precision = LRDMC_PRECISION_DF64;
   fill_df_constants(S);
   // one block holds kWarpsPerBlock walkers in shared memory; without room

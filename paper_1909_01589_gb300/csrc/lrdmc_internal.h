@@ -20,6 +20,10 @@ constexpr int kMaxMO = LRDMC_MAX_SPIN;
 constexpr int kMaxNjCh = LRDMC_NJ_MAX_CH;
 constexpr int kWarpsPerBlock = 4;
 constexpr int kMaxItersPerInterval = 1 << 20;
+// Iterations whose random numbers a warp of the double-float mode draws at
+// once, and the doubles each takes (rotation, waiting time, heat bath).
+constexpr int kDrawAhead = 16;
+constexpr int kDrawWords = 11;
 
 // Error bits of the device error word.
 constexpr int kErrSingular = 1;
@@ -126,6 +130,11 @@ struct SysDev {
   int n_prim;       // primitives of all Gaussian shells
   int ee_recip;     // 1: the e-e Pade sum in the reciprocal form (b >= 1/4)
   float ee_sign;    // sign of b (0 for b = 0)
+  // the non-zero MO coefficients: bit m of row_mask[mu] and bit mu of
+  // col_mask[m] for C[mu][m] != 0 (an atom's orbitals mix basis functions of
+  // one symmetry only)
+  unsigned row_mask[kMaxAO];
+  unsigned long long col_mask[kMaxMO];
   double C[kMaxAO * kMaxMO];  // [n_ao][n_mo]
   int precision;  // LRDMC_PRECISION_FP64 or LRDMC_PRECISION_DF64
   // neural pair term of the Jastrow factor, tabulated: channel c, cell k
@@ -162,6 +171,7 @@ struct Layout {
   int head;       // doubles of shared memory per block before the warp regions
   int smem_warp;  // doubles of shared memory per warp
   int smem_block_bytes;
+  int n_draw;     // doubles per warp of draws made ahead (double-float mode)
   int n_scr;      // doubles of scratch per warp (shared with the evaluation's state)
   int n_pc;       // electron pairs with a cached distance (0: no cache)
   int enc;        // 1: the electron-nucleus cache (and the pair cache, if any) is in the layout
@@ -174,14 +184,19 @@ Layout make_layout(const SysDev& S, bool caches);
 // state, evaluation buffers (with or without caches) and scratch side by
 // side. The layout in use overlays them and needs less.
 int accept_smem_bytes(const SysDev& S, bool caches);
-// Entries of the double-float exponential's table, and the offset (doubles)
-// of the double-float evaluation's tables in a block's shared memory.
+// Entries of the double-float exponential's table.
 constexpr int kExpBits = 10;
 constexpr int kExpEntries = 1 << kExpBits;
-__host__ __device__ inline int lean_offset(const SysDev& S)
+// A block's shared tables: the MO coefficients in the three arithmetics, the
+// 64-entry table, the coefficients' masks; then the double-float ones.
+__host__ __device__ inline int mask_offset(const SysDev& S)
 {
   const int nc = S.n_ao * S.n_mo;
   return (2 * nc + (nc + 1) / 2 + 64 + 1) & ~1;
+}
+__host__ __device__ inline int lean_offset(const SysDev& S)
+{
+  return (mask_offset(S) + S.n_mo + (S.n_ao + 1) / 2 + 1) & ~1;
 }
 // Largest dynamic shared memory of one block on sm_100-class GPUs (227 KB),
 // less 2 KB for the kernels' static shared memory (the interval kernel's

@@ -375,26 +375,17 @@ static __device__ void ao_dot_der(const SysDev& S, const double* v, const double
   }
 }
 
-// chi_mu(p) for all AOs into out[n_ao].
-static __device__ void ao_values(const SysDev& S, const double* p, double* out)
+// chi_mu(p) of shell q into out[n_ao].
+static __device__ void shell_values(const SysDev& S, int q, const double* p, double* out)
 {
-  int prev_c = -1;
-  double d[3] = {0, 0, 0}, r = 0.0, e = 0.0;
-  for (int q = 0; q < S.n_shell; ++q) {
-    const ShellDev& sh = S.sh[q];
-    if (sh.center != prev_c) {
-      prev_c = sh.center;
-      d[0] = p[0] - S.nuc[prev_c][0];
-      d[1] = p[1] - S.nuc[prev_c][1];
-      d[2] = p[2] - S.nuc[prev_c][2];
-      r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    }
-    if (sh.kind == 0 && !sh.same_exp) e = exp(-sh.zeta * r);
-    double R, R1, R2, Sv[5], gS[5][3];
-    radial(sh, r, e, R, R1, R2, false);
-    int nf = solid(sh.l, d, Sv, gS, false);
-    for (int f = 0; f < nf; ++f) out[sh.ao_offset + f] = Sv[f] * R;
-  }
+  const ShellDev& sh = S.sh[q];
+  const double d[3] = {p[0] - S.nuc[sh.center][0], p[1] - S.nuc[sh.center][1], p[2] - S.nuc[sh.center][2]};
+  const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+  const double e = sh.kind == 0 ? exp(-sh.zeta * r) : 0.0;
+  double R, R1, R2, Sv[5], gS[5][3];
+  radial(sh, r, e, R, R1, R2, false);
+  const int nf = solid(sh.l, d, Sv, gS, false);
+  for (int f = 0; f < nf; ++f) out[sh.ao_offset + f] = Sv[f] * R;
 }
 
 // ----------------------------------------------------------------------------
@@ -490,6 +481,7 @@ struct WarpMem {
   double* A;    // inverse up [nu][nu] then down [nd][nd]
   double* R;    // [9]
   double* T;    // [P_max]
+  double* dr;   // [kDrawAhead][kDrawWords] draws made ahead (double-float mode)
   double* sm;   // [4 + n_ao + 3 nu] Sherman-Morrison scratch of the double-float mode
   // the evaluation's state; scr is scratch over the same storage (the
   // inverse and the other modes' Sherman-Morrison updates, which run while
@@ -516,7 +508,8 @@ __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, d
   m.A = m.x + 3 * Lo.N;
   m.R = m.A + Lo.nu * Lo.nu + Lo.nd * Lo.nd;
   m.T = m.R + 12;
-  m.sm = m.T + Lo.P_max;
+  m.dr = m.T + Lo.P_max;
+  m.sm = m.dr + Lo.n_draw;
   m.scr = m.sm + 4 + S.n_ao + 3 * Lo.nu;
   m.v = m.scr;
   m.Ssum = m.v + Lo.N * S.n_ao;
@@ -536,13 +529,15 @@ __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, d
   return m;
 }
 
-// Block-shared tables: MO coefficients (double, then a float copy), then
-// the 2^(j/64) table.
+// Block-shared tables: MO coefficients (double, then double-float and float
+// copies), the 2^(j/64) table, the masks of the non-zero coefficients.
 struct BlockMem {
   double* C;
   df* Cd;
   float* Cf;
   float2* tab;
+  unsigned long long* col;  // [n_mo] non-zero rows of a column of C
+  unsigned* row;            // [n_ao] non-zero columns of a row
 };
 
 __device__ __forceinline__ BlockMem block_mem(const SysDev& S, double* smem)
@@ -553,110 +548,160 @@ __device__ __forceinline__ BlockMem block_mem(const SysDev& S, double* smem)
   b.Cd = reinterpret_cast<df*>(smem + nc);
   b.Cf = reinterpret_cast<float*>(smem + 2 * nc);
   b.tab = reinterpret_cast<float2*>(smem + 2 * nc + (nc + 1) / 2);
+  b.col = reinterpret_cast<unsigned long long*>(smem + mask_offset(S));
+  b.row = reinterpret_cast<unsigned*>(smem + mask_offset(S) + S.n_mo);
   return b;
 }
 
-// ----------------------------------------------------------------------------
-// Inverse Slater matrix of one spin block by Gauss-Jordan elimination with
-// partial pivoting (warp-cooperative). A[l][m] = phi_m(r_l); the inverse is
-// stored as Ainv[m][l]. Returns false for a singular matrix (below).
-// ----------------------------------------------------------------------------
-// With resid (nullable), first the residual of the inverse the block holds
-// (the Sherman-Morrison-updated one): max |sum_m A[l][m] Ainv[m][q] -
-// delta_lq| over the block, where A is the Slater matrix at the current
-// positions; *resid becomes the larger of itself and that residual (the
-// same value in every lane).
-static __device__ LRDMC_COLD bool warp_inverse(const SysDev& S, const double* sC, const double* sx, int spin,
-                             double* Ainv, double* scr, int lane, double* resid = nullptr)
+// sum_m C[mu][m] A[m n + l] and sum_mu C[mu][m] chi[mu] over the non-zero
+// coefficients only, in order (a zero's product would add nothing): an FP64
+// multiply-add holds its sub-partition's pipe for 64 cycles, and an atom's C
+// has few non-zeros (18 of 324 for Kr).
+__device__ __forceinline__ double project_ao(const SysDev& S, const BlockMem& bm, const double* A, int mu, int l, int n)
 {
-  const int n = spin == 0 ? S.n_up : S.n_dn;
-  if (n == 0) return true;
-  const int off = spin == 0 ? 0 : S.n_up;
-  const int w2 = 2 * n;
-  double* M = scr;                 // [n][2n]
-  double* chi = scr + n * w2;      // [n][n_ao]
-  for (int l = lane; l < n; l += 32) {
-    ao_values(S, &sx[3 * (off + l)], &chi[l * S.n_ao]);
-    for (int m = 0; m < n; ++m) {
-      double a = 0.0;
-      for (int mu = 0; mu < S.n_ao; ++mu) a += sC[mu * S.n_mo + m] * chi[l * S.n_ao + mu];
-      M[l * w2 + m] = a;
-      M[l * w2 + n + m] = (m == l) ? 1.0 : 0.0;
-    }
+  double acc = 0.0;
+#pragma unroll 1
+  for (unsigned k = bm.row[mu] & (n < 32 ? (1u << n) - 1u : 0xffffffffu); k; k &= k - 1) {
+    const int m = __ffs(k) - 1;
+    acc += bm.C[mu * S.n_mo + m] * A[m * n + l];
+  }
+  return acc;
+}
+
+__device__ __forceinline__ double orbital_value(const SysDev& S, const BlockMem& bm, const double* chi, int m)
+{
+  double a = 0.0;
+#pragma unroll 1
+  for (unsigned long long k = bm.col[m]; k; k &= k - 1) {
+    const int mu = __ffsll((long long)k) - 1;
+    a += bm.C[mu * S.n_mo + m] * chi[mu];
+  }
+  return a;
+}
+
+// ----------------------------------------------------------------------------
+// Inverse Slater matrices of both spin blocks by Gauss-Jordan elimination
+// with partial pivoting (warp-cooperative), A[l][m] = phi_m(r_l), the inverse
+// stored as Ainv[m][l]; false for a singular matrix (below). With resid
+// (nullable), first the residual of the inverses the blocks hold (the
+// Sherman-Morrison-updated ones): max |sum_m A[l][m] Ainv[m][q] - delta_lq|,
+// where A is the Slater matrix at the current positions; *resid becomes the
+// larger of itself and that residual (the same value in every lane).
+//
+// Bound by the FP64 pipe, which takes 64 cycles per warp instruction whatever
+// its lane count, so the work is dealt to all lanes: basis values by
+// (electron, shell), matrix entries one per lane, and the elimination in
+// place on n x n entries (the identity's columns of the augmented form are
+// produced where its pivot columns vanish, with the same operations). Pivots
+// are compared as integers, off that pipe.
+// ----------------------------------------------------------------------------
+static __device__ LRDMC_COLD bool warp_inverses(const SysDev& S, const double* sC, const double* sx, double* Ainv0,
+                                                double* scr, int lane, double* resid = nullptr)
+{
+  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
+  double* chi = scr;                                    // [N][n_ao]
+  double* M = chi + S.N * S.n_ao;                       // [n][n]
+  double* fc = M + S.n_up * S.n_up;                     // [n] the pivot column
+  int* perm = reinterpret_cast<int*>(fc + S.n_up);      // [n] row of the original matrix
+#pragma unroll 1
+  for (int u = lane; u < S.N * S.n_shell; u += 32) {
+    const int i = u / S.n_shell, q = u - i * S.n_shell;
+    shell_values(S, q, &sx[3 * i], &chi[i * S.n_ao]);
   }
   __syncwarp();
-  if (resid) {
-    double r = 0.0;
-    for (int idx = lane; idx < n * n; idx += 32) {
-      const int l = idx / n, q = idx % n;
-      double a = (l == q) ? -1.0 : 0.0;
-      for (int m = 0; m < n; ++m) a += M[l * w2 + m] * Ainv[m * n + q];
-      r = fmax(r, fabs(a));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(FULL_MASK, r, o));
-    *resid = fmax(*resid, r);
-  }
-  // Singular Slater matrix: two equal-spin electrons on one point (the
-  // determinant vanishes by antisymmetry; elimination would leave a residual
-  // row of rounding size, not an exact zero), or a pivot that is zero or not
-  // finite. No relative pivot threshold is applied: the orbitals of a heavy
-  // atom span many orders of magnitude (a 1s value at a valence electron),
-  // so pivots far below the largest entry of their column are legitimate,
-  // and rounding noise amplified by that scale spread cannot be told apart
-  // from a small genuine pivot.
-  int coincide = 0;
-  for (int pr = lane; pr < n * n; pr += 32) {
-    const int l = pr / n, q = pr % n;
-    if (q <= l) continue;
-    const double* a = &sx[3 * (off + l)];
-    const double* c = &sx[3 * (off + q)];
-    coincide |= (a[0] == c[0] && a[1] == c[1] && a[2] == c[2]);
-  }
-  if (__any_sync(FULL_MASK, coincide)) return false;
   bool ok = true;
-  for (int col = 0; col < n && ok; ++col) {
-    // pivot row: largest |M[r][col]| for r >= col, lowest r on ties
-    double best = -1.0;
-    int br = col;
-    for (int r = col + lane; r < n; r += 32) {
-      double a = fabs(M[r * w2 + col]);
-      if (a > best) { best = a; br = r; }
-    }
+#pragma unroll 1
+  for (int spin = 0; spin < 2 && ok; ++spin) {
+    const int n = spin == 0 ? S.n_up : S.n_dn, off = spin == 0 ? 0 : S.n_up;
+    double* Ainv = spin ? Ainv0 + S.n_up * S.n_up : Ainv0;
+    if (n == 0) break;
+    // entry idx = lane, lane + 32, ... as (row, column): advanced without divisions
+    const int dr = 32 / n, dc = 32 - dr * n, r0 = lane / n, c0 = lane - r0 * n;
+#define LRDMC_ENTRIES(r, c) \
+    for (int idx = lane, r = r0, c = c0; idx < n * n; idx += 32, r += dr, c += dc, c >= n ? (c -= n, ++r) : 0)
+#pragma unroll 1
+    LRDMC_ENTRIES(l, m) M[idx] = orbital_value(S, bm, &chi[(off + l) * S.n_ao], m);
+    if (lane < n) perm[lane] = lane;
+    __syncwarp();
+    if (resid) {
+      double res = 0.0;
+#pragma unroll 1
+      LRDMC_ENTRIES(l, q) {
+        double a = (l == q) ? -1.0 : 0.0;
+#pragma unroll 1
+        for (int m = 0; m < n; ++m) a += M[l * n + m] * Ainv[m * n + q];
+        res = fmax(res, fabs(a));
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      double ob = __shfl_xor_sync(FULL_MASK, best, o);
-      int orr = __shfl_xor_sync(FULL_MASK, br, o);
-      if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
+      for (int o = 16; o > 0; o >>= 1) res = fmax(res, __shfl_xor_sync(FULL_MASK, res, o));
+      *resid = fmax(*resid, res);
     }
-    if (!(best > 0.0) || !isfinite(best)) { ok = false; break; }
-    if (br != col) {
-      for (int j = lane; j < w2; j += 32) {
-        double t = M[col * w2 + j];
-        M[col * w2 + j] = M[br * w2 + j];
-        M[br * w2 + j] = t;
+    // Singular Slater matrix: two equal-spin electrons on one point (the
+    // determinant vanishes by antisymmetry; elimination would leave a residual
+    // row of rounding size, not an exact zero), or a pivot that is zero or not
+    // finite. No relative pivot threshold is applied: the orbitals of a heavy
+    // atom span many orders of magnitude (a 1s value at a valence electron),
+    // so pivots far below the largest entry of their column are legitimate,
+    // and rounding noise amplified by that scale spread cannot be told apart
+    // from a small genuine pivot.
+    int coincide = 0;
+#pragma unroll 1
+    LRDMC_ENTRIES(l, q) {
+      const double* a = &sx[3 * (off + l)];
+      const double* b = &sx[3 * (off + q)];
+      coincide |= l < q && a[0] == b[0] && a[1] == b[1] && a[2] == b[2];
+    }
+    if (__any_sync(FULL_MASK, coincide)) return false;
+#pragma unroll 1
+    for (int col = 0; col < n && ok; ++col) {
+      // pivot row: largest |M[r][col]| for r >= col (n <= 32: one row per
+      // lane), lowest r on ties, NaN passed over; the bits of non-negative
+      // doubles order as the doubles
+      long long best = -1;
+      int br = col;
+      if (lane >= col && lane < n) {
+        const long long a = __double_as_longlong(M[lane * n + col]) & 0x7fffffffffffffffll;
+        if (a <= 0x7ff0000000000000ll) { best = a; br = lane; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long ob = __shfl_xor_sync(FULL_MASK, best, o);
+        const int orr = __shfl_xor_sync(FULL_MASK, br, o);
+        if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
+      }
+      if (best <= 0 || best >= 0x7ff0000000000000ll) { ok = false; break; }
+      if (br != col) {
+        if (lane < n) {
+          const double t = M[col * n + lane];
+          M[col * n + lane] = M[br * n + lane];
+          M[br * n + lane] = t;
+        }
+        if (lane == 0) {
+          const int t = perm[col];
+          perm[col] = perm[br];
+          perm[br] = t;
+        }
+        __syncwarp();
+      }
+      const double inv = 1.0 / M[col * n + col];
+      if (lane < n) fc[lane] = M[lane * n + col];
+      __syncwarp();
+      if (lane < n) M[col * n + lane] = lane == col ? inv : M[col * n + lane] * inv;
+      __syncwarp();
+#pragma unroll 1
+      LRDMC_ENTRIES(r, c) {
+        const double f = fc[r];
+        if (r != col && f != 0.0) M[idx] = fma(-f, M[col * n + c], c == col ? 0.0 : M[idx]);
       }
       __syncwarp();
     }
-    double inv = 1.0 / M[col * w2 + col];
-    __syncwarp();
-    for (int j = lane; j < w2; j += 32) M[col * w2 + j] *= inv;
-    __syncwarp();
-    for (int r = lane; r < n; r += 32) {
-      if (r == col) continue;
-      double f = M[r * w2 + col];
-      if (f != 0.0)
-        for (int j = 0; j < w2; ++j) M[r * w2 + j] -= f * M[col * w2 + j];
+    if (ok) {
+#pragma unroll 1
+      LRDMC_ENTRIES(m, c) Ainv[m * n + perm[c]] = M[idx];
     }
     __syncwarp();
+#undef LRDMC_ENTRIES
   }
-  if (ok) {
-    for (int idx = lane; idx < n * n; idx += 32) {
-      int m = idx / n, l = idx % n;
-      Ainv[m * n + l] = M[m * w2 + n + l];
-    }
-  }
-  __syncwarp();
   return ok;
 }
 
@@ -672,14 +717,13 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
                           bool moves = true)
 {
   const int N = S.N, nao = S.n_ao, nu = S.n_up;
+  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
   // projected inverse columns: v[i][mu] = sum_m C[mu][m] Ainv_sigma[m][l_i]
   for (int idx = lane; idx < N * nao; idx += 32) {
     int i = idx / nao, mu = idx % nao;
     int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
     const double* A = spin ? wm.A + nu * nu : wm.A;
-    double acc = 0.0;
-    for (int m = 0; m < n; ++m) acc += sC[mu * S.n_mo + m] * A[m * n + l];
-    wm.v[idx] = acc;
+    wm.v[idx] = project_ao(S, bm, A, mu, l, n);
   }
   __syncwarp();
   // local energy: lanes over electrons
@@ -1142,16 +1186,16 @@ static __device__ LRDMC_JUMP bool warp_sm_update(const SysDev& S, const double* 
   const int nu = S.n_up;
   const int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
   double* A = spin ? wm.A + nu * nu : wm.A;
+  const BlockMem bm = block_mem(S, const_cast<double*>(sC));
   double* chi = wm.scr;            // [n_ao]
   double* phi = chi + S.n_ao;      // [n]
   double* y = phi + n;             // [n]
   double* col = y + n;             // [n]
-  if (lane == 0) ao_values(S, p, chi);
+#pragma unroll 1
+  for (int q = lane; q < S.n_shell; q += 32) shell_values(S, q, p, chi);
   __syncwarp();
   for (int m = lane; m < n; m += 32) {
-    double a = 0.0;
-    for (int mu = 0; mu < S.n_ao; ++mu) a += sC[mu * S.n_mo + m] * chi[mu];
-    phi[m] = a;
+    phi[m] = orbital_value(S, bm, chi, m);
   }
   __syncwarp();
   for (int q = lane; q < n; q += 32) {
@@ -1212,6 +1256,8 @@ __device__ __forceinline__ void stage_coefficients(const SysDev& S, double* sC)
     bm.Cf[j] = (float)S.C[j];
   }
   for (int j = threadIdx.x; j < 64; j += blockDim.x) bm.tab[j] = S.D.exp.t[j];
+  for (int j = threadIdx.x; j < S.n_mo; j += blockDim.x) bm.col[j] = S.col_mask[j];
+  for (int j = threadIdx.x; j < S.n_ao; j += blockDim.x) bm.row[j] = S.row_mask[j];
   __syncthreads();
 }
 
@@ -1232,8 +1278,7 @@ k_init(const __grid_constant__ SysDev S, const Layout Lo, const PopDev P, const 
   for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x0[(size_t)s * 3 * Lo.N + j];
   for (int j = lane; j < Lo.P_max; j += 32) wm.T[j] = 0.0;
   __syncwarp();
-  bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane);
-  ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane);
+  bool ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane);
   if (!ok && lane == 0) atomicOr(P.err, kErrSingular);
   if (lane == 0) {
     double u[4];
@@ -1339,6 +1384,7 @@ __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, 
 #define LRDMC_TEAM_CHUNK 16
 #endif
   const int cs = t ? LRDMC_TEAM_CHUNK : 32;
+#pragma unroll 1
   for (int c0 = 0;; c0 += 32) {
     if (t) {
       int c = 0;
@@ -1483,8 +1529,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
         load_record(Lo, P.rec_src + (size_t)bounded(P.parent[s], P.W, P.err) * Lo.rec, wm, lane, b, el);
         if (recompute) {
           double rs = 0.0;
-          bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane, &rs);
-          ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane, &rs);
+          bool ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane, &rs);
           if (!ok && lane == 0) atomicOr(P.err, kErrSingular);
           if (lane == 0 && isfinite(rs)) atomicMax(P.resid, (unsigned long long)__double_as_longlong(rs));
         }
@@ -1515,21 +1560,24 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       bool over = st.finish != 0;
       double t = 0.0, logw = st.logw;
       uint64_t b0[4], b1[4];
+      const int it = (int)(st.m % kDrawAhead);
       if (!over) {
-        // both draws of this iteration at once: even lanes compute the
-        // (waiting time, heat bath) block, odd lanes the rotation block
-        uint64_t cb[4] = {(uint64_t)st.s, k, (uint64_t)st.m, (lane & 1) ? kTagRot : kTagTimeHB};
-        philox4x64_10(cb, P.seed, 0ull);
+        if (kDf) {
+          if (it == 0) draw_ahead64(P.seed, (uint64_t)st.s, k, (uint64_t)st.m, wm.dr, lane, S, lt);
+          const df nl = reinterpret_cast<const df*>(wm.dr + it * kDrawWords)[9];
+          t = b > 0.0 ? df_to_double(dl_mul(nl, dl_norm(dl_rcp(bdf)))) : INFINITY;
+        } else {
+          // both draws of this iteration at once: even lanes compute the
+          // (waiting time, heat bath) block, odd lanes the rotation block
+          uint64_t cb[4] = {(uint64_t)st.s, k, (uint64_t)st.m, (lane & 1) ? kTagRot : kTagTimeHB};
+          philox4x64_10(cb, P.seed, 0ull);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          b0[j] = shfl_u64(cb[j], 0);
-          b1[j] = shfl_u64(cb[j], 1);
-        }
-        if (kDf)
-          t = b > 0.0 ? df_to_double(dl_mul(dl_neg(dl_log(df_u01(b0[0]), S.D.lexp, lt.tab)), dl_norm(dl_rcp(bdf))))
-                      : INFINITY;
-        else
+          for (int j = 0; j < 4; ++j) {
+            b0[j] = shfl_u64(cb[j], 0);
+            b1[j] = shfl_u64(cb[j], 1);
+          }
           t = b > 0.0 ? (double)(-logf(f_u01(b0[0])) / bdf.hi) : INFINITY;
+        }
         if (t >= tau_left) {
           logw -= tau_left * (el - P.e_trial);
           over = true;
@@ -1541,7 +1589,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
         // heat bath over the cached rates
         if (kDf) {
           pick = heat_bath64(reinterpret_cast<const df*>(wm.T), P_moves, lane, wm.pfx,
-                             dl_norm(dl_mul(df_u01(b0[1]), bdf)));
+                             dl_norm(dl_mul(reinterpret_cast<const df*>(wm.dr + it * kDrawWords)[10], bdf)));
         } else {
           int lastc;
           warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, f_u01(b0[1]) * bdf.hi, &pick,
@@ -1585,8 +1633,11 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       }
       if (lane < 3) wm.x[3 * i + lane] = wm.sm[lane];
       __syncwarp();
-      if (kDf) rotation64(b1, wm.R, lane, S);
-      else rotation_matrix_warp<PR>(b1, wm.R, lane, S);
+      if (kDf) {
+        if (lane < 9) wm.R[lane] = wm.dr[it * kDrawWords + lane];
+      } else {
+        rotation_matrix_warp<PR>(b1, wm.R, lane, S);
+      }
       __syncwarp();
       double eln;
       if (kDf) eln = prelude64<NJ, NC>(S, sC, wm, lt, lane, st.fresh ? -1 : i);
@@ -1717,8 +1768,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
       load_record(Lo, P.rec_src + (size_t)src * Lo.rec, wm, lane, b, el);
       if (recompute) {
         double rs = 0.0;
-        bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane, &rs);
-        ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane, &rs);
+        bool ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane, &rs);
         if (!ok && lane == 0) atomicOr(P.err, kErrSingular);
         if (lane == 0 && isfinite(rs)) atomicMax(P.resid, (unsigned long long)__double_as_longlong(rs));
       }
@@ -2117,8 +2167,7 @@ __device__ __forceinline__ bool evaluate_config(const SysDev& S, const Layout& L
   for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x[(size_t)c * 3 * Lo.N + j];
   for (int j = lane; j < 9; j += 32) wm.R[j] = rot[(size_t)c * 9 + j];
   __syncwarp();
-  bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane);
-  ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane);
+  bool ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane);
   if (!ok) return false;
   const int P = S.N * 6 * L.G;
   double b, el;
@@ -2242,7 +2291,8 @@ Layout make_layout(const SysDev& S, bool caches)
   Lo.off_el = Lo.off_b + 1;
   Lo.rec = (Lo.off_el + 1 + 3) & ~3;
   const int n = S.n_up;
-  Lo.n_scr = 2 * n * n + n * S.n_ao;                         // Gauss-Jordan + orbital rows
+  Lo.n_draw = kDrawAhead * kDrawWords;
+  Lo.n_scr = n * n + S.N * S.n_ao + n + (n + 1) / 2;         // inverses: basis values, matrix, pivot column, order
   Lo.n_scr = std::max(Lo.n_scr, S.n_ao + 3 * n + n * n);     // Sherman-Morrison (FP64 or FP32 mode)
   // The caches of the double-float evaluation (omitted when caches is false):
   // the electron-nucleus cache (8 df per electron and nucleus), and one
@@ -2251,7 +2301,7 @@ Layout make_layout(const SysDev& S, bool caches)
   Lo.n_pc = (caches && S.N <= 40) ? S.N * (S.N - 1) / 2 : 0;
   Lo.enc = caches ? 1 : 0;
   const int state = S.N * S.n_ao + 2 * S.N + 6 * S.N + 12 + 32 + (Lo.enc ? 8 * S.N * S.n_nuc : 0) + Lo.n_pc;
-  Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + 4 + S.n_ao + 3 * n +
+  Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + Lo.n_draw + 4 + S.n_ao + 3 * n +
                  std::max(Lo.n_scr, state);
   Lo.smem_warp = (Lo.smem_warp + 1) & ~1;
   Lo.head = lean_offset(S) + kExpEntries + 2 * S.n_prim + (int)(sizeof(LShell) / sizeof(double)) * S.n_shell;
@@ -2266,13 +2316,15 @@ int accept_smem_bytes(const SysDev& S, bool caches)
   int warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + 12 * S.N + S.N * S.n_ao + S.N + (3 * S.N + 12) + scr;
   if (caches) warp += (S.N <= 24 ? S.N * (S.N - 1) / 2 * (S.N <= 12 ? 8 : 4) : 0) + 8 * S.N * S.n_nuc;
   warp = (warp + 1) & ~1;
-  return (int)sizeof(double) * (lean_offset(S) + kWarpsPerBlock * warp);
+  return (int)sizeof(double) * (mask_offset(S) + kWarpsPerBlock * warp);
 }
 #endif  // LRDMC_PART == 0
 
+// Without the attribute a block's dynamic and static shared memory together
+// are limited to 48 KB (the interval kernel's static part is below 2 KB).
 static cudaError_t set_smem(const void* fn, int bytes)
 {
-  if (bytes > 48 * 1024) return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (bytes > 44 * 1024) return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return cudaSuccess;
 }
 
@@ -2492,15 +2544,14 @@ cudaError_t launch_eval_all(const SysDev& S, const Layout& Lo, const LatDev& L, 
   return cudaErrorInvalidValue;
 }
 
-// Warps per block of the interval kernel: 16 (so that the warps of an SM,
-// one block, can help one another at the end of an interval), halved while
-// the population cannot give every warp of every SM a walker, then as many
-// as the shared memory holds; at least the other kernels' four.
+// Warps per block of the interval kernel: enough that one block per SM holds
+// the population (so that the warps of an SM can help one another at the end
+// of an interval), at least the other kernels' four, at most 16 and what the
+// shared memory holds.
 int interval_warps(const Layout& Lo, int W)
 {
   const int sms = sm_count_current();
-  int w = kMaxIntervalWarps;
-  while (w > kWarpsPerBlock && W < sms * w) w >>= 1;
+  int w = std::min(kMaxIntervalWarps, std::max(kWarpsPerBlock, (W + sms - 1) / sms));
   while (w > kWarpsPerBlock && (int)sizeof(double) * (Lo.head + w * Lo.smem_warp) > kMaxSmemBlock) --w;
   return w;
 }
@@ -2572,8 +2623,7 @@ k_base_terms(const __grid_constant__ SysDev S, const Layout Lo, int n, const dou
   WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
   for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x[(size_t)s * 3 * Lo.N + j];
   __syncwarp();
-  bool ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane);
-  ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane);
+  bool ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane);
   if (!ok) {
     if (lane == 0) atomicOr(err, kErrSingular);
     for (int j = lane; j < 3 * Lo.N; j += 32) grad[(size_t)s * 3 * Lo.N + j] = NAN;
@@ -2831,8 +2881,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
     for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x[(size_t)c * 3 * Lo.N + j];
     for (int j = lane; j < 9; j += 32) wm.R[j] = rot[(size_t)c * 9 + j];
     __syncwarp();
-    ok = warp_inverse(S, sC, wm.x, 0, wm.A, wm.scr, lane);
-    ok = ok && warp_inverse(S, sC, wm.x, 1, wm.A + Lo.nu * Lo.nu, wm.scr, lane);
+    ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane);
     if (!ok && lane == 0) atomicOr(err, kErrSingular);
     if (ok) el = prelude32<NJ>(S, sC, wm, lean_mem(S, sC), lane, -1);
   }
