@@ -124,14 +124,31 @@ __device__ __forceinline__ dl slater_power(const LShell& sh, dl r, const SysDev&
   return real_power(df_make(sh.m_hi, sh.m_lo), r, S.D.lexp, t.tab);
 }
 
-// The five degree-2 solid harmonics of d contracted with v.
-__device__ __forceinline__ dl solid2_dot(const df* v, const dl d[3])
+// The five degree-2 solid harmonics of two points contracted with v.
+__device__ __forceinline__ dl2 solid2_dot2(const df* v, const dl2 d[3])
 {
-  const dl xx = dl_sqr(d[0]), yy = dl_sqr(d[1]), zz = dl_sqr(d[2]);
-  dl s = dl_add(dl_mul(v[0], dl_mul(d[0], d[1])), dl_mul(v[1], dl_mul(d[1], d[2])));
-  s = dl_add(s, dl_mul(v[2], dl_mul(d[2], d[0])));
-  s = dl_add(s, dl_mul(v[3], dl_norm(dl_sub(xx, yy))));
-  return dl_add_n(s, dl_mul(v[4], dl_norm(dl_sub(dl_add(zz, zz), dl_add(xx, yy)))));
+  const dl2 xx = dl2_sqr(d[0]), yy = dl2_sqr(d[1]), zz = dl2_sqr(d[2]);
+  dl2 s = dl2_add(dl2_mul(dl2_all(v[0]), dl2_mul(d[0], d[1])), dl2_mul(dl2_all(v[1]), dl2_mul(d[1], d[2])));
+  s = dl2_add(s, dl2_mul(dl2_all(v[2]), dl2_mul(d[2], d[0])));
+  s = dl2_add(s, dl2_mul(dl2_all(v[3]), dl2_norm(dl2_sub(xx, yy))));
+  return dl2_add_n(s, dl2_mul(dl2_all(v[4]), dl2_norm(dl2_sub(dl2_add(zz, zz), dl2_add(xx, yy)))));
+}
+
+__device__ __forceinline__ dl2 slater_power2(const LShell& sh, dl2 r, const SysDev& S, const Lean& t)
+{
+  if (sh.m_int == 1) return r;
+  if (sh.m_int >= 0) {
+    dl2 p = dl2_all(df_make(1.0f, 0.0f));
+#pragma unroll 1
+    for (int j = 0; j < sh.m_int; ++j) p = dl2_mul(p, r);
+    return dl2_norm(p);
+  }
+  dl a, b;
+  dl2_split(r, a, b);
+  const dl m = df_make(sh.m_hi, sh.m_lo);
+  a = real_power(m, a, S.D.lexp, t.tab);
+  b = real_power(m, b, S.D.lexp, t.tab);
+  return dl2_pack(a, b);
 }
 
 __device__ __forceinline__ dl dl_dot3(const df* a, const dl b[3])
@@ -430,7 +447,7 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
       }
       e[3] = D;
     }
-    if (wm.n_pc) {
+    {
       dl d[3];
       if (moved < 0) {
         const int tu = nu * (nu - 1) / 2, td = nd * (nd - 1) / 2;
@@ -468,23 +485,29 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
   return el;
 }
 
+// The neural pair term at two distances.
+__device__ __forceinline__ dl2 nj_value64_2(const SysDev& S, int c, dl2 r)
+{
+  dl a, b;
+  dl2_split(r, a, b);
+  return dl2_pack(nj_value64(S, c, a), nj_value64(S, c, b));
+}
+
 // One partner of the e-e sums of the moves +-h e_k: Dh = b^2 (D + h^2), p =
 // 2 b^2 h (y_ik - y_jk)/b; acc receives q (or s q, the general form).
 template <bool NJ>
-__device__ __forceinline__ void ee_partner64(const SysDev& S, dl Dh, dl p, int ch, dl acc[2], dl nj[2])
+__device__ __forceinline__ void ee_partner64(const SysDev& S, dl Dh, dl p, int ch, dl2& acc, dl2& nj)
 {
-#pragma unroll
-  for (int m = 0; m < 2; ++m) {
-    const dl s = dl_sqrt(dl_norm(dl_add_big(Dh, m ? dl_neg(p) : p)));
-    if (S.ee_recip) {
-      // q <= 1 <= acc: the sum starts from one
-      acc[m] = dl_add_big(acc[m], dl_rcp(dl_one_plus(s)));
-    } else {
-      const dl q = dl_rcp(dl_norm(dl_add_f(dl_mul_f(s, S.ee_sign), 1.0f)));
-      acc[m] = dl_add(acc[m], dl_mul(s, q));
-    }
-    if (NJ) nj[m] = dl_add(nj[m], nj_value64(S, ch, dl_mul(s, S.D.ee_iscale)));
+  const dl2 s = dl2_sqrt(dl2_norm(dl2_add_big(dl2_all(Dh), dl2_pm(p))));
+  if (S.ee_recip) {
+    // q <= 1 <= acc: the sum starts from one
+    acc = dl2_add_big(acc, dl2_rcp(dl2_one_plus(s)));
+  } else {
+    const dl2 sg = dl2_make(f2_mul(s.hi, f2_all(S.ee_sign)), f2_mul(s.lo, f2_all(S.ee_sign)));
+    const dl2 q = dl2_rcp(dl2_norm(dl2_add_f(sg, f2_all(1.0f))));
+    acc = dl2_add(acc, dl2_mul(s, q));
   }
+  if (NJ) nj = dl2_add(nj, nj_value64_2(S, ch, dl2_mul(s, dl2_all(S.D.ee_iscale))));
 }
 
 // The two lattice moves +-h e_k of unit u = (electron, grid, axis): rates
@@ -494,11 +517,12 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
                                         df* Td, double* ratio_out)
 {
   const int G = L.G, i = u / (3 * G), rem = u - i * 3 * G, g = rem / 3, k = rem - 3 * g;
-  const int N = S.N, nu = S.n_up;
+  const int nu = S.n_up;
   const df* v = &wm.vd[i * S.n_ao];
   const dl h = g ? L.ap_df : L.a_df;
-  const dl zero = df_make(0.0f, 0.0f);
-  dl rdet[2] = {zero, zero}, jn[2] = {zero, zero}, mid[2];
+  const f2 one = f2_all(1.0f);
+  dl2 rdet = dl2_zero(), jn = dl2_zero();
+  dl mid[2];
   mid[0] = mid[1] = df_make(INFINITY, 0.0f);
   {
     const dl h2 = dl_sqr(h);
@@ -518,95 +542,71 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
       }
       // |d +- h e|^2 = D + h^2 +- 2 h p (D + h^2 >= 2 h |p|); the bond's
       // midpoint D + h^2/4 +- h p
-      const dl Dh = dl_add_n(D, h2), hp2 = dl_scale(hp, 2.0f);
+      const dl Dh = dl_add_n(D, h2);
       if (G == 2 && S.heavy[I]) {
-        const dl Dm = dl_add_n(D, dl_scale(h2, 0.25f));
+        dl t[2];
+        dl2_split(dl2_norm(dl2_add_big(dl2_all(dl_add_n(D, dl_scale(h2, 0.25f))), dl2_pm(hp))), t[0], t[1]);
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          const dl t = dl_norm(dl_add_big(Dm, m ? dl_neg(hp) : hp));
-          if (t.hi < mid[m].hi || (t.hi == mid[m].hi && t.lo < mid[m].lo)) mid[m] = t;
-        }
+        for (int m = 0; m < 2; ++m)
+          if (t[m].hi < mid[m].hi || (t[m].hi == mid[m].hi && t[m].lo < mid[m].lo)) mid[m] = t[m];
       }
-      dl r2[2], r[2], e[2];
-#pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        r2[m] = dl_norm(dl_add_big(Dh, m ? dl_neg(hp2) : hp2));
-        r[m] = dl_norm(dl_sqrt_acc(r2[m]));
-        e[m] = zero;
-      }
+      const dl2 r2 = dl2_norm(dl2_add_big(dl2_all(Dh), dl2_pm(dl_scale(hp, 2.0f))));
+      const dl2 r = dl2_norm(dl2_sqrt_acc(r2));
+      dl2 e = dl2_zero();
       if (S.en_b1[I] != 0.0) {
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-          const dl q = dl_rcp(dl_norm(dl_add_f(dl_mul(S.D.en_b2, r[m]), 1.0f)));
-          jn[m] = dl_sub(jn[m], dl_mul(dl_mul(S.D.en_b1[I], r[m]), q));
-        }
+        const dl2 q = dl2_rcp(dl2_norm(dl2_add_f(dl2_mul(dl2_all(S.D.en_b2), r), one)));
+        jn = dl2_sub(jn, dl2_mul(dl2_mul(dl2_all(S.D.en_b1[I]), r), q));
       }
-      if (NJ) {
-#pragma unroll
-        for (int m = 0; m < 2; ++m) jn[m] = dl_add(jn[m], nj_value64(S, 2 + S.nj_species[I], r[m]));
-      }
+      if (NJ) jn = dl2_add(jn, nj_value64_2(S, 2 + S.nj_species[I], r));
 #pragma unroll 1
       for (int q = S.nuc_shell_begin[I]; q < S.nuc_shell_begin[I + 1]; ++q) {
         const LShell sh = lt.sh[q];
-        dl R[2];
+        dl2 R;
         if (sh.kind == 0) {
-          if (!sh.same_exp) {
-            const dl zeta = df_make(-sh.zeta_hi, -sh.zeta_lo);
-#pragma unroll
-            for (int m = 0; m < 2; ++m) e[m] = dl_exp(dl_norm(dl_mul(zeta, r[m])), S.D.lexp, lt.tab);
-          }
-#pragma unroll
-          for (int m = 0; m < 2; ++m) R[m] = sh.m_int == 0 ? e[m] : dl_mul(slater_power(sh, r[m], S, lt), e[m]);
+          if (!sh.same_exp)
+            e = dl2_exp(dl2_norm(dl2_mul(dl2_all(df_make(-sh.zeta_hi, -sh.zeta_lo)), r)), S.D.lexp, lt.tab);
+          R = sh.m_int == 0 ? e : dl2_mul(slater_power2(sh, r, S, lt), e);
         } else {
-          R[0] = R[1] = zero;
+          R = dl2_zero();
 #pragma unroll 1
           for (int p = 0; p < sh.n_prim; ++p) {
             const float4 pr = lt.prim[sh.prim + p];
-            const dl al = df_make(-pr.x, -pr.y), co = df_make(pr.z, pr.w);
-#pragma unroll
-            for (int m = 0; m < 2; ++m)
-              R[m] = dl_add(R[m], dl_mul(co, dl_exp(dl_norm(dl_mul(al, r2[m])), S.D.lexp, lt.tab)));
+            const dl2 al = dl2_all(df_make(-pr.x, -pr.y)), co = dl2_all(df_make(pr.z, pr.w));
+            R = dl2_add(R, dl2_mul(co, dl2_exp(dl2_norm(dl2_mul(al, r2)), S.D.lexp, lt.tab)));
           }
         }
-        dl P[2];
+        dl2 P;
         if (sh.l == 0) {
-          P[0] = P[1] = v[sh.ao];
+          P = dl2_all(v[sh.ao]);
         } else if (sh.l == 1) {
-          const dl base = dl_dot3(&v[sh.ao], d), w = dl_dot3(&v[sh.ao], he);
-          P[0] = dl_add_n(base, w);
-          P[1] = dl_sub_n(base, w);
+          P = dl2_add_n(dl2_all(dl_dot3(&v[sh.ao], d)), dl2_pm(dl_dot3(&v[sh.ao], he)));
         } else {
+          dl2 dm[3];
 #pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            dl dm[3];
-#pragma unroll
-            for (int t = 0; t < 3; ++t) dm[t] = dl_add_n(d[t], m ? dl_neg(he[t]) : he[t]);
-            P[m] = solid2_dot(&v[sh.ao], dm);
-          }
+          for (int t = 0; t < 3; ++t) dm[t] = dl2_add_n(dl2_all(d[t]), dl2_pm(he[t]));
+          P = solid2_dot2(&v[sh.ao], dm);
         }
-#pragma unroll
-        for (int m = 0; m < 2; ++m) rdet[m] = dl_add(rdet[m], dl_mul(P[m], R[m]));
+        rdet = dl2_add(rdet, dl2_mul(P, R));
       }
     }
   }
   // e-e part: partners of the same spin, then of the other
-  dl jee[2], nj[2] = {zero, zero};
+  dl2 jee, nj = dl2_zero();
   {
     const dl hb = dl_norm(dl_mul(h, S.D.ee_scale)), h2b = dl_norm(dl_sqr(hb)), hb2 = dl_scale(hb, 2.0f);
     const dl yi = wm.y[3 * i + k];
-    const bool up = i < nu, cached = !NC && wm.n_pc;
-    const float start = S.ee_recip ? 1.0f : 0.0f;
+    const bool up = i < nu;
+    const dl2 start = dl2_all(df_make(S.ee_recip ? 1.0f : 0.0f, 0.0f));
     const int n_same = up ? nu : S.n_dn, off_same = up ? 0 : nu, l = i - off_same;
     const int tri = up ? 0 : nu * (nu - 1) / 2;
-    dl acc[2];
-    acc[0] = acc[1] = df_make(start, 0.0f);
+    dl2 acc = start;
     int qq = tri + l * (l - 1) / 2;
     dl dd[3];
 #pragma unroll 1
     for (int t = 0; t < n_same - 1; ++t) {
       const int jl = t < l ? t : t + 1, j = off_same + jl;
       dl D;
-      if (cached) {
+      if (!NC) {
         if (t >= l) qq = tri + jl * (jl - 1) / 2 + l;
         D = wm.pc[qq];
         ++qq;
@@ -616,12 +616,8 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
       const dl p = dl_mul(hb2, dl_sub(yi, wm.y[3 * j + k]));
       ee_partner64<NJ>(S, dl_add(D, h2b), p, 0, acc, nj);
     }
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      acc[m] = dl_add_f(acc[m], -start);
-      jee[m] = dl_mul(S.D.c_par, dl_norm(acc[m]));
-      acc[m] = df_make(start, 0.0f);
-    }
+    jee = dl2_mul(dl2_all(S.D.c_par), dl2_norm(dl2_add_f(acc, f2_neg(start.hi))));
+    acc = start;
     const int n_opp = up ? S.n_dn : nu, off_opp = up ? nu : 0;
     const int opp = nu * (nu - 1) / 2 + S.n_dn * (S.n_dn - 1) / 2;
     int qo = up ? opp + l * S.n_dn : opp + l;
@@ -630,7 +626,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
     for (int t = 0; t < n_opp; ++t) {
       const int j = off_opp + t;
       dl D;
-      if (cached) {
+      if (!NC) {
         D = wm.pc[qo];
         qo += dq;
       } else {
@@ -639,34 +635,32 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
       const dl p = dl_mul(hb2, dl_sub(yi, wm.y[3 * j + k]));
       ee_partner64<NJ>(S, dl_add(D, h2b), p, 1, acc, nj);
     }
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      acc[m] = dl_add_f(acc[m], -start);
-      jee[m] = dl_add(jee[m], dl_mul(S.D.c_anti, dl_norm(acc[m])));
-    }
+    jee = dl2_add(jee, dl2_mul(dl2_all(S.D.c_anti), dl2_norm(dl2_add_f(acc, f2_neg(start.hi)))));
   }
   const int c0 = (i * G + g) * 6 + 2 * k;
+  // e^(Delta J): J = J_ee(-1/b sum c q, or 1/b sum c s q) + J_en (+ neural)
+  dl2 dJ = dl2_mul(dl2_sub_n(jee, dl2_all(wm.Sd[i])), dl2_all(S.D.ee_factor));
+  dl2 jx = dl2_sub(jn, dl2_all(wm.Sn[i]));
+  if (NJ) jx = dl2_add(jx, nj);
+  dJ = dl2_add_n(dJ, jx);
+  const dl2 rho = dl2_norm(dl2_mul(dl2_norm(rdet), dl2_exp(dJ, S.D.lexp, lt.tab)));
+  dl2 T = dl2_mul(rho, dl2_all(g ? L.inv2ap2_df : L.inv2a2_df));
+  if (G == 2) {
+    const dl2 x = dl2_mul(dl2_pack(mid[0], mid[1]), dl2_all(L.p_coef_df));
+    dl2 w = L.pkind == 0 ? dl2_exp(dl2_neg(dl2_norm(x)), S.D.lexp, lt.tab) : dl2_rcp(dl2_norm(dl2_add_f(x, one)));
+    if (g) w = dl2_add_f(dl2_neg(w), one);
+    T = dl2_mul(T, dl2_norm(w));
+  }
+  T = dl2_norm(T);
+  dl t[2], ro[2];
+  dl2_split(T, t[0], t[1]);
+  dl2_split(rho, ro[0], ro[1]);
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
-    // e^(Delta J): J = J_ee(-1/b sum c q, or 1/b sum c s q) + J_en (+ neural)
-    dl dJ = dl_mul(dl_sub_n(jee[m], wm.Sd[i]), S.D.ee_factor);
-    dl jx = dl_sub(jn[m], wm.Sn[i]);
-    if (NJ) jx = dl_add(jx, nj[m]);
-    dJ = dl_add_n(dJ, jx);
-    const dl rho = dl_norm(dl_mul(dl_norm(rdet[m]), dl_exp(dJ, S.D.lexp, lt.tab)));
-    dl T = zero;
-    if (rho.hi > 0.0f) {
-      T = dl_mul(rho, g ? L.inv2ap2_df : L.inv2a2_df);
-      if (G == 2) {
-        dl w = L.pkind == 0 ? dl_exp(dl_neg(dl_norm(dl_mul(mid[m], L.p_coef_df))), S.D.lexp, lt.tab)
-                            : dl_rcp(dl_norm(dl_add_f(dl_mul(mid[m], L.p_coef_df), 1.0f)));
-        if (g) w = dl_add_f(dl_neg(w), 1.0f);
-        T = dl_mul(T, dl_norm(w));
-      }
-      T = dl_norm(T);
-    }
-    Td[c0 + m] = T;
-    if (ratio_out) ratio_out[c0 + m] = df_to_double(rho);
+    // a move across a node is not allowed
+    if (!(ro[m].hi > 0.0f)) t[m] = df_make(0.0f, 0.0f);
+    Td[c0 + m] = t[m];
+    if (ratio_out) ratio_out[c0 + m] = df_to_double(ro[m]);
   }
 }
 

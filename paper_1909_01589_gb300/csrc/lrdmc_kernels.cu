@@ -2296,10 +2296,10 @@ Layout make_layout(const SysDev& S, bool caches)
   Lo.n_scr = std::max(Lo.n_scr, S.n_ao + 3 * n + n * n);     // Sherman-Morrison (FP64 or FP32 mode)
   // The caches of the double-float evaluation (omitted when caches is false):
   // the electron-nucleus cache (8 df per electron and nucleus), and one
-  // squared distance per electron pair up to 40 electrons (beyond, the cache
+  // squared distance per electron pair; up to 40 electrons (beyond, they
   // would cost warps per SM)
   Lo.n_pc = (caches && S.N <= 40) ? S.N * (S.N - 1) / 2 : 0;
-  Lo.enc = caches ? 1 : 0;
+  Lo.enc = caches && S.N <= 40 ? 1 : 0;
   const int state = S.N * S.n_ao + 2 * S.N + 6 * S.N + 12 + 32 + (Lo.enc ? 8 * S.N * S.n_nuc : 0) + Lo.n_pc;
   Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + Lo.n_draw + 4 + S.n_ao + 3 * n +
                  std::max(Lo.n_scr, state);
