@@ -12,8 +12,9 @@
 // silu''(z) z'^2 + silu'(z) z'').
 //
 // Training arithmetic is FP32 with the parameters staged in shared memory
-// (bfloat16-rounded when the spec asks for it); one warp evaluates one
-// pair, lane l owning hidden units l and l + 32.
+// (bfloat16-rounded when the spec asks for it). A block takes 32 pairs at a
+// time; their chains are the 96 rows of small matrix products with W2, which
+// the threads compute in register tiles (below).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -23,6 +24,7 @@
 #include <vector>
 
 #include "lrdmc_internal.h"
+#include "lean64.cuh"
 
 namespace lrdmc {
 
@@ -169,41 +171,68 @@ void nj_build_table(const lrdmc_nj_spec& sp, const float* params, std::vector<do
 // ----------------------------------------------------------------------------
 constexpr int kNjH = LRDMC_NJ_HIDDEN;
 constexpr int kNjMaxF = LRDMC_NJ_MAX_FEAT;
-constexpr int kNjMaxC = LRDMC_NJ_MAX_CH;
-constexpr int kNjWarps = 4;
-static_assert(kNjH == 64, "lanes own hidden units l and l + 32");
+constexpr int kNjThreads = 128;
+constexpr int kNjTile = 32;    // pairs per tile
+constexpr int kNjSuper = 128;  // pairs whose geometry is formed at once, one per thread
+constexpr int kNjLd = kNjH + 4;  // row stride of the chain matrices (floats; 16-byte aligned, staggered over the banks)
+static_assert(kNjH == 64, "16 unit groups of four");
 
-// Shared-memory image of the parameters (float, bf16-rounded if asked):
-// W1T [D][H] (transposed), b1, W2T [H][H] (transposed, forward), W2 [H][H]
-// (row-major, backward), b2, w3, b3; then the pair table and the per-warp
-// chain buffers.
+// Shared memory of a block: the parameters (float, bf16-rounded if asked) as
+// W1T [D][H], b1, W2T [H][H] (transposed), b2, w3, b3; the pair table; of 128
+// pairs the radius, unit vector and channel; of the tile's 32 pairs the
+// features with their radial derivatives; the layer-1 activations A [chain][pair][H].
+// The backward pass adds W2 [H][H], the upstream derivatives, the layer-2
+// derivatives Z [chain][pair][H] and a layer-1 gradient slice per warp.
+//
+// Thread (pg, ug) of a tile owns pairs 4 pg .. 4 pg + 3 and units 4 ug .. 4 ug +
+// 3: per step of a product it reads 12 chain values and 4 weights (16-byte
+// loads, most of them broadcast) for 48 multiply-adds, so the FP32 pipe binds
+// (with one warp per pair a lane read three words for six multiply-adds, and
+// 128 weight gradients per lane spilled).
 struct NjSmem {
-  float* W1T; float* b1; float* W2T; float* W2; float* b2; float* w3; float* b3;
+  float* W1T; float* b1; float* W2T; float* b2; float* w3; float* b3;
   int* pairs;      // [n_pairs]: i | j << 8 | channel << 16 (j = nucleus for e-n)
-  float4* chain;   // [warps][H] per-warp broadcast buffer
+  float4* geo;     // [128] r, e
+  int* ch;         // [128]
+  float4* feat;    // [32][F] f, f', f''
+  float* A;        // [96][kNjLd]
+  float* sum;      // [96] output-layer sums
+  float* W2;       // backward: [H][H]
+  float4* up;      // [128] upstream derivatives of m, m', m''
+  float* Z;        // [96][kNjLd]
+  float* acc1;     // [4][D][H]
 };
 
-__host__ __device__ inline int nj_smem_floats(int D, int n_pairs)
+__host__ __device__ inline int nj_smem_floats(int F, int C, int n_pairs, bool backward)
 {
-  return D * kNjH + kNjH + 2 * kNjH * kNjH + 2 * kNjH + 1 + 3 /*pad*/ + n_pairs + 4 * kNjWarps * kNjH + 4;
+  const int D = F + C, H = kNjH;
+  int n = D * H + H + H * H + 2 * H + 4;
+  n += (n_pairs + 3) & ~3;
+  n += 4 * kNjSuper + kNjSuper + 4 * kNjTile * F + 3 * kNjTile * (kNjLd + 1);
+  if (backward) n += H * H + 4 * kNjSuper + 3 * kNjTile * kNjLd + 4 * D * H;
+  return n;
 }
 
-__device__ inline NjSmem nj_stage(const NjGeom& G, const NjNetDev& N, const float* params, float* sm)
+__device__ inline NjSmem nj_stage(const NjGeom& G, const NjNetDev& N, const float* params, float* sm, bool backward)
 {
   NjSmem m;
-  const int D = N.D, H = kNjH;
+  const int D = N.D, H = kNjH, np = G.n_pairs;
   m.W1T = sm;
   m.b1 = m.W1T + D * H;
   m.W2T = m.b1 + H;
-  m.W2 = m.W2T + H * H;
-  m.b2 = m.W2 + H * H;
+  m.b2 = m.W2T + H * H;
   m.w3 = m.b2 + H;
   m.b3 = m.w3 + H;
   m.pairs = reinterpret_cast<int*>(m.b3 + 4);
-  const int np = G.n_pairs;
-  uintptr_t a = reinterpret_cast<uintptr_t>(m.pairs + np);
-  a = (a + 15) & ~(uintptr_t)15;
-  m.chain = reinterpret_cast<float4*>(a);
+  m.geo = reinterpret_cast<float4*>(m.pairs + ((np + 3) & ~3));
+  m.ch = reinterpret_cast<int*>(m.geo + kNjSuper);
+  m.feat = reinterpret_cast<float4*>(m.ch + kNjSuper);
+  m.A = reinterpret_cast<float*>(m.feat + kNjTile * N.F);
+  m.sum = m.A + 3 * kNjTile * kNjLd;
+  m.W2 = m.sum + 3 * kNjTile;
+  m.up = reinterpret_cast<float4*>(m.W2 + H * H);
+  m.Z = reinterpret_cast<float*>(m.up + kNjSuper);
+  m.acc1 = m.Z + 3 * kNjTile * kNjLd;
   auto rd = [&](int idx) { float v = params[idx]; return N.bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v; };
   const int oW1 = 0, ob1 = H * D, oW2 = ob1 + H, ob2 = oW2 + H * H, ow3 = ob2 + H, ob3 = ow3 + H;
   for (int q = threadIdx.x; q < H * D; q += blockDim.x) {
@@ -213,7 +242,7 @@ __device__ inline NjSmem nj_stage(const NjGeom& G, const NjNetDev& N, const floa
   for (int q = threadIdx.x; q < H * H; q += blockDim.x) {
     const int u = q / H, v = q % H;
     const float w = rd(oW2 + q);
-    m.W2[q] = w;
+    if (backward) m.W2[q] = w;
     m.W2T[v * H + u] = w;
   }
   for (int q = threadIdx.x; q < H; q += blockDim.x) {
@@ -222,6 +251,8 @@ __device__ inline NjSmem nj_stage(const NjGeom& G, const NjNetDev& N, const floa
     m.w3[q] = rd(ow3 + q);
   }
   if (threadIdx.x == 0) m.b3[0] = rd(ob3);
+  if (backward)
+    for (int q = threadIdx.x; q < 4 * D * H; q += blockDim.x) m.acc1[q] = 0.0f;
   // pair table: electron pairs i < j, then electron-nucleus pairs i-major
   const int N_e = G.N, n_ee = N_e * (N_e - 1) / 2;
   for (int q = threadIdx.x; q < np; q += blockDim.x) {
@@ -253,54 +284,19 @@ __device__ __forceinline__ void silu3(float z, float& a, float& d1, float& d2, f
   a = z * sg;
   d1 = sg * (1.0f + z * (1.0f - sg));     // silu'
   d2 = sp * (2.0f + z * u);               // silu''
-  d3 = sp * (u * (3.0f + z * u) - 2.0f * z * sp);  // silu'''
+  d3 = sp * (u * (3.0f + z * u) - 2.0f * z * sp);  // third derivative
 }
 
-// Geometry of pair q of configuration cfg: radius, unit vector (from i to
-// the partner: r_i - r_j or r_i - R_I), electrons and channel.
-struct PairGeo {
-  float r, e[3];
-  int i, j, c, is_en;
-};
-
-__device__ __forceinline__ PairGeo pair_geo(const NjGeom& G, const NjSmem& m, const double* x, size_t cfg, int q)
+// Distance and unit vector of d = a - b (both double): in double-float
+// arithmetic, rounded to single (as the FP64 form to within its rounding;
+// FP64 instructions hold their pipe for 64 cycles each).
+__device__ __forceinline__ float4 unit_vector(const double* a, const double* b)
 {
-  PairGeo p;
-  const int code = m.pairs[q];
-  p.i = code & 0xFF;
-  p.j = (code >> 8) & 0xFF;
-  p.c = code >> 16;
-  p.is_en = p.c >= 2;
-  const double* xi = x + (cfg * G.N + p.i) * 3;
-  double d[3];
-  if (p.is_en) {
-    for (int k = 0; k < 3; ++k) d[k] = xi[k] - G.nuc[p.j][k];
-  } else {
-    const double* xj = x + (cfg * G.N + p.j) * 3;
-    for (int k = 0; k < 3; ++k) d[k] = xi[k] - xj[k];
-  }
-  const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-  p.r = (float)r;
-  for (int k = 0; k < 3; ++k) p.e[k] = (float)(d[k] / r);
-  return p;
-}
-
-// Features and their radial derivatives (radial part only; the channel code
-// is constant).
-__device__ __forceinline__ void features(const NjNetDev& N, float r, float f0[kNjMaxF], float f1[kNjMaxF],
-                                         float f2[kNjMaxF])
-{
-#pragma unroll
-  for (int f = 0; f < kNjMaxF; ++f) {
-    if (f < N.F) {
-      const float l2 = N.ell2[f], r2 = r * r, den = r2 + l2, id = 1.0f / den;
-      f0[f] = r2 * id;
-      f1[f] = 2.0f * r * l2 * id * id;
-      f2[f] = 2.0f * l2 * (l2 - 3.0f * r2) * id * id * id;
-    } else {
-      f0[f] = 0.0f; f1[f] = 0.0f; f2[f] = 0.0f;
-    }
-  }
+  dl d[3];
+  for (int k = 0; k < 3; ++k) d[k] = dl_sub_n(dl_from_double(a[k]), dl_from_double(b[k]));
+  const dl r = dl_norm(dl_sqrt_acc(dl_norm(dl_add(dl_add(dl_sqr(d[0]), dl_sqr(d[1])), dl_sqr(d[2])))));
+  const dl ir = dl_rcp(r);
+  return make_float4(r.hi, dl_norm(dl_mul(d[0], ir)).hi, dl_norm(dl_mul(d[1], ir)).hi, dl_norm(dl_mul(d[2], ir)).hi);
 }
 
 // Cut-off factor s(r/r_c) and its radial derivatives.
@@ -313,45 +309,111 @@ __device__ __forceinline__ void cutoff(float r, float rc, float& s, float& s1, f
   s2 = -60.0f * t * (1.0f - t) * (1.0f - 2.0f * t) / (rc * rc);
 }
 
-// The two layers for the warp's pair; lane l computes units l and l + 32.
-// On return: z1 chains of layer 1 (own units), the layer-1 activations of
-// all units in the warp buffer, the z2 chains of layer 2 (own units).
-struct Fwd {
-  float z[2], z1[2], z2[2];   // layer 1 pre-activation chains
-  float y[2], y1[2], y2[2];   // layer 2 pre-activation chains
-};
+// Features of the tile's pairs and their radial derivatives (radial part
+// only; the channel code is constant).
+__device__ __forceinline__ void tile_features(const NjNetDev& N, const NjSmem& m, int sub)
+{
+  for (int t = threadIdx.x; t < kNjTile * N.F; t += kNjThreads) {
+    const int p = t / N.F, f = t - p * N.F;
+    const float r = m.geo[sub * kNjTile + p].x;
+    const float l2 = N.ell2[f], r2 = r * r, den = r2 + l2, id = 1.0f / den;
+    m.feat[t] = make_float4(r2 * id, 2.0f * r * l2 * id * id, 2.0f * l2 * (l2 - 3.0f * r2) * id * id * id, 0.0f);
+  }
+}
 
-__device__ __forceinline__ void fwd_layers(const NjNetDev& N, const NjSmem& m, float4* buf, int lane, int c,
-                                           const float f0[kNjMaxF], const float f1[kNjMaxF],
-                                           const float f2[kNjMaxF], Fwd& o)
+// c[0..3] += a b over four units
+__device__ __forceinline__ void fma4(float c[4], float a, const float4& b)
+{
+  c[0] = fmaf(a, b.x, c[0]);
+  c[1] = fmaf(a, b.y, c[1]);
+  c[2] = fmaf(a, b.z, c[2]);
+  c[3] = fmaf(a, b.w, c[3]);
+}
+
+// Layer-1 pre-activation chains z[chain][pair][unit] of the thread's tile.
+__device__ __forceinline__ void layer1(const NjNetDev& N, const NjSmem& m, int sub, int pg, int ug, float z[3][4][4])
+{
+  const float4 b = *reinterpret_cast<const float4*>(m.b1 + 4 * ug);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int c = m.ch[sub * kNjTile + 4 * pg + p];
+    const float4 w = *reinterpret_cast<const float4*>(m.W1T + (N.F + c) * kNjH + 4 * ug);
+    z[0][p][0] = b.x + w.x; z[0][p][1] = b.y + w.y; z[0][p][2] = b.z + w.z; z[0][p][3] = b.w + w.w;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) z[1][p][u] = z[2][p][u] = 0.0f;
+  }
+#pragma unroll 1
+  for (int f = 0; f < N.F; ++f) {
+    const float4 w = *reinterpret_cast<const float4*>(m.W1T + f * kNjH + 4 * ug);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const float4 ft = m.feat[(4 * pg + p) * N.F + f];
+      fma4(z[0][p], ft.x, w);
+      fma4(z[1][p], ft.y, w);
+      fma4(z[2][p], ft.z, w);
+    }
+  }
+}
+
+// y[chain][pair][unit] += sum_k X[chain][pair][k] W[k][unit] over the 64 k.
+__device__ __forceinline__ void row_product(const float* X, const float* W, int pg, int ug, float y[3][4][4])
+{
+#pragma unroll 1
+  for (int k = 0; k < kNjH; k += 4) {
+    float4 w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[q] = *reinterpret_cast<const float4*>(W + (k + q) * kNjH + 4 * ug);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const float4 x = *reinterpret_cast<const float4*>(X + (c * kNjTile + 4 * pg + p) * kNjLd + k);
+        fma4(y[c][p], x.x, w[0]);
+        fma4(y[c][p], x.y, w[1]);
+        fma4(y[c][p], x.z, w[2]);
+        fma4(y[c][p], x.w, w[3]);
+      }
+  }
+}
+
+// Activations of the tile's pre-activation chains into A (all three chains).
+__device__ __forceinline__ void activate(float* A, int pg, int ug, float z[3][4][4])
 {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int u = lane + 32 * h;
-    float z = m.b1[u] + m.W1T[(N.F + c) * kNjH + u], z1 = 0.0f, z2 = 0.0f;
+  for (int p = 0; p < 4; ++p) {
+    float v[3][4];
 #pragma unroll
-    for (int f = 0; f < kNjMaxF; ++f) {
-      if (f < N.F) {
-        const float w = m.W1T[f * kNjH + u];
-        z = fmaf(w, f0[f], z); z1 = fmaf(w, f1[f], z1); z2 = fmaf(w, f2[f], z2);
-      }
+    for (int u = 0; u < 4; ++u) {
+      float d1, d2, d3;
+      silu3(z[0][p][u], v[0][u], d1, d2, d3);
+      v[1][u] = d1 * z[1][p][u];
+      v[2][u] = fmaf(d1, z[2][p][u], __fmul_rn(__fmul_rn(d2, z[1][p][u]), z[1][p][u]));
     }
-    o.z[h] = z; o.z1[h] = z1; o.z2[h] = z2;
-    float a, d1, d2, d3;
-    silu3(z, a, d1, d2, d3);
-    buf[u] = make_float4(a, d1 * z1, d2 * z1 * z1 + d1 * z2, 0.0f);
-  }
-  __syncwarp();
-  float y[2] = {m.b2[lane], m.b2[lane + 32]}, y1[2] = {0.0f, 0.0f}, y2[2] = {0.0f, 0.0f};
-#pragma unroll 8
-  for (int v = 0; v < kNjH; ++v) {
-    const float4 a = buf[v];
-    const float w0 = m.W2T[v * kNjH + lane], w1 = m.W2T[v * kNjH + lane + 32];
-    y[0] = fmaf(w0, a.x, y[0]); y1[0] = fmaf(w0, a.y, y1[0]); y2[0] = fmaf(w0, a.z, y2[0]);
-    y[1] = fmaf(w1, a.x, y[1]); y1[1] = fmaf(w1, a.y, y1[1]); y2[1] = fmaf(w1, a.z, y2[1]);
-  }
 #pragma unroll
-  for (int h = 0; h < 2; ++h) { o.y[h] = y[h]; o.y1[h] = y1[h]; o.y2[h] = y2[h]; }
+    for (int c = 0; c < 3; ++c)
+      *reinterpret_cast<float4*>(A + (c * kNjTile + 4 * pg + p) * kNjLd + 4 * ug) =
+          make_float4(v[c][0], v[c][1], v[c][2], v[c][3]);
+  }
+}
+
+// Both layers' pre-activations of the tile: A filled, y the layer-2 chains.
+// Two barriers: the features before, A after.
+__device__ __forceinline__ void tile_forward(const NjNetDev& N, const NjSmem& m, int sub, int pg, int ug,
+                                             float y[3][4][4])
+{
+  tile_features(N, m, sub);
+  __syncthreads();
+  layer1(N, m, sub, pg, ug, y);
+  activate(m.A, pg, ug, y);
+  const float4 b = *reinterpret_cast<const float4*>(m.b2 + 4 * ug);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    y[0][p][0] = b.x; y[0][p][1] = b.y; y[0][p][2] = b.z; y[0][p][3] = b.w;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) y[1][p][u] = y[2][p][u] = 0.0f;
+  }
+  __syncthreads();
+  row_product(m.A, m.W2T, pg, ug, y);
 }
 
 __device__ __forceinline__ float warp_sum_f(float v)
@@ -361,46 +423,77 @@ __device__ __forceinline__ float warp_sum_f(float v)
   return v;
 }
 
+// Geometry of this thread's pair of the super-tile; pairs beyond the total
+// repeat the last one (their results are not used).
+__device__ __forceinline__ void super_geometry(const NjGeom& G, const NjSmem& m, const double* x, long long p,
+                                               size_t& cfg, int& code)
+{
+  cfg = (size_t)(p / G.n_pairs);
+  code = m.pairs[(int)(p - (long long)cfg * G.n_pairs)];
+  const int i = code & 0xFF, j = (code >> 8) & 0xFF, c = code >> 16;
+  const double* xi = x + (cfg * G.N + i) * 3;
+  m.geo[threadIdx.x] = unit_vector(xi, c >= 2 ? G.nuc[j] : x + (cfg * G.N + j) * 3);
+  m.ch[threadIdx.x] = c;
+}
+
 // g, g', g'' of every pair of every configuration.
-__global__ void __launch_bounds__(kNjWarps * 32)
+__global__ void __launch_bounds__(kNjThreads, 2)
 k_nj_pairs_fwd(const __grid_constant__ NjGeom G, const __grid_constant__ NjNetDev N, const float* params, int n,
                const double* x, float* pair_out)
 {
   extern __shared__ float4 nj_smem4[];
-  const NjSmem m = nj_stage(G, N, params, reinterpret_cast<float*>(nj_smem4));
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float4* buf = m.chain + wib * kNjH;
+  const NjSmem m = nj_stage(G, N, params, reinterpret_cast<float*>(nj_smem4), false);
+  const int pg = threadIdx.x >> 4, ug = threadIdx.x & 15;
   const long long total = (long long)n * G.n_pairs;
-  for (long long p = (long long)blockIdx.x * kNjWarps + wib; p < total; p += (long long)gridDim.x * kNjWarps) {
-    const size_t cfg = (size_t)(p / G.n_pairs);
-    const int q = (int)(p % G.n_pairs);
-    const PairGeo pg = pair_geo(G, m, x, cfg, q);
-    float f0[kNjMaxF], f1[kNjMaxF], f2[kNjMaxF];
-    features(N, pg.r, f0, f1, f2);
-    Fwd o;
-    fwd_layers(N, m, buf, lane, pg.c, f0, f1, f2, o);
-    float mv = 0.0f, m1 = 0.0f, m2 = 0.0f;
+  const float b3 = m.b3[0];
+  for (long long base = (long long)blockIdx.x * kNjSuper; base < total; base += (long long)gridDim.x * kNjSuper) {
+    __syncthreads();  // the previous super-tile is done with geo, ch and A
+    size_t cfg;
+    int code;
+    super_geometry(G, m, x, min(base + threadIdx.x, total - 1), cfg, code);
+    __syncthreads();
+#pragma unroll 1
+    for (int sub = 0; sub < kNjSuper / kNjTile && base + sub * kNjTile < total; ++sub) {
+      float y[3][4][4];
+      tile_forward(N, m, sub, pg, ug, y);
+      __syncthreads();  // A is read; it takes the layer-2 activation chains now
+      activate(m.A, pg, ug, y);
+      __syncthreads();
+      // output layer, one row (chain, pair) per thread: p_l = w_l k_l + w_{l+32}
+      // k_{l+32}, summed as the tree l, l ^ 16, l ^ 8, .., l ^ 1
+      if (threadIdx.x < 3 * kNjTile) {
+        const float* k = m.A + threadIdx.x * kNjLd;
+        float v[8][4];
+        // the four residues of l modulo 4, each of its eight l
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float a, d1, d2, d3;
-      silu3(o.y[h], a, d1, d2, d3);
-      const float w = m.w3[lane + 32 * h];
-      mv = fmaf(w, a, mv);
-      m1 = fmaf(w, d1 * o.y1[h], m1);
-      m2 = fmaf(w, d2 * o.y1[h] * o.y1[h] + d1 * o.y2[h], m2);
+        for (int q = 0; q < 8; ++q) {
+          const float4 a = *reinterpret_cast<const float4*>(k + 4 * q), b = *reinterpret_cast<const float4*>(k + 4 * q + 32);
+          const float4 wa = *reinterpret_cast<const float4*>(m.w3 + 4 * q),
+                       wb = *reinterpret_cast<const float4*>(m.w3 + 4 * q + 32);
+          v[q][0] = fmaf(wb.x, b.x, wa.x * a.x);
+          v[q][1] = fmaf(wb.y, b.y, wa.y * a.y);
+          v[q][2] = fmaf(wb.z, b.z, wa.z * a.z);
+          v[q][3] = fmaf(wb.w, b.w, wa.w * a.w);
+        }
+        float t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          t[u] = ((v[0][u] + v[4][u]) + (v[2][u] + v[6][u])) + ((v[1][u] + v[5][u]) + (v[3][u] + v[7][u]));
+        const float mv = (t[0] + t[2]) + (t[1] + t[3]);
+        m.sum[threadIdx.x] = mv;
+      }
+      __syncthreads();
+      const int t = sub * kNjTile + threadIdx.x;
+      if (threadIdx.x < kNjTile && base + t < total) {
+        const float mv = m.sum[threadIdx.x] + b3, m1 = m.sum[kNjTile + threadIdx.x], m2 = m.sum[2 * kNjTile + threadIdx.x];
+        float s, s1, s2;
+        cutoff(m.geo[t].x, N.rcut[m.ch[t]], s, s1, s2);
+        float* out = pair_out + (size_t)(base + t) * 3;
+        out[0] = mv * s;
+        out[1] = fmaf(mv, s1, __fmul_rn(m1, s));
+        out[2] = fmaf(mv, s2, fmaf(2.0f * m1, s1, __fmul_rn(m2, s)));
+      }
     }
-    mv = warp_sum_f(mv) + m.b3[0];
-    m1 = warp_sum_f(m1);
-    m2 = warp_sum_f(m2);
-    if (lane == 0) {
-      float s, s1, s2;
-      cutoff(pg.r, N.rcut[pg.c], s, s1, s2);
-      float* out = pair_out + (size_t)p * 3;
-      out[0] = mv * s;
-      out[1] = m1 * s + mv * s1;
-      out[2] = m2 * s + 2.0f * m1 * s1 + mv * s2;
-    }
-    __syncwarp();
   }
 }
 
@@ -424,21 +517,17 @@ k_nj_assemble(const __grid_constant__ NjGeom G, int n, const double* x, const do
       if (j == i) continue;
       const int a = min(i, j), b = max(i, j);
       const int q = a * N_e - a * (a + 1) / 2 + (b - a - 1);
-      double d[3];
-      for (int k = 0; k < 3; ++k) d[k] = xc[3 * i + k] - xc[3 * j + k];
-      const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      const float g1 = po[3 * q + 1], g2 = po[3 * q + 2], rf = (float)r;
-      for (int k = 0; k < 3; ++k) Gi[k] += g1 * (float)(d[k] / r);
-      Li += g2 + 2.0f * g1 / rf;
+      const float4 e = unit_vector(&xc[3 * i], &xc[3 * j]);
+      const float g1 = po[3 * q + 1], g2 = po[3 * q + 2];
+      Gi[0] += g1 * e.y; Gi[1] += g1 * e.z; Gi[2] += g1 * e.w;
+      Li += g2 + 2.0f * g1 / e.x;
     }
     for (int I = 0; I < G.n_nuc; ++I) {
       const int q = n_ee + i * G.n_nuc + I;
-      double d[3];
-      for (int k = 0; k < 3; ++k) d[k] = xc[3 * i + k] - G.nuc[I][k];
-      const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      const float g1 = po[3 * q + 1], g2 = po[3 * q + 2], rf = (float)r;
-      for (int k = 0; k < 3; ++k) Gi[k] += g1 * (float)(d[k] / r);
-      Li += g2 + 2.0f * g1 / rf;
+      const float4 e = unit_vector(&xc[3 * i], G.nuc[I]);
+      const float g1 = po[3 * q + 1], g2 = po[3 * q + 2];
+      Gi[0] += g1 * e.y; Gi[1] += g1 * e.z; Gi[2] += g1 * e.w;
+      Li += g2 + 2.0f * g1 / e.x;
     }
     const double* a = grad_base + ((size_t)cfg * N_e + i) * 3;
     float dot = 0.0f, gg = 0.0f;
@@ -460,162 +549,235 @@ k_nj_assemble(const __grid_constant__ NjGeom G, int n, const double* x, const do
 
 // Backward: per pair, the upstream derivatives with respect to g, g', g''
 // from d_el and d_j of its configuration, then reverse through the cut-off,
-// the output layer and both activations (the derivative chains included).
-// Every sum runs in a fixed order, so the gradient is the same bits from
-// run to run: each warp accumulates layers 2 and 3 in registers and layer 1
-// in its own shared-memory slice (a lane owns its hidden units), the warps
-// are added in warp order, and each block writes its sums to partials
-// [blockIdx.x][n_params] for k_nj_grad_reduce.
-__global__ void __launch_bounds__(kNjWarps * 32, 2)
+// the output layer and both activations (the derivative chains included):
+// per tile three products, W2 times the layer-1 chains (recomputed), W2^T
+// times the layer-2 derivatives, and the weight gradient, of which a thread
+// keeps 4 x 8 entries in registers over all its block's tiles. Every sum runs
+// in a fixed order, so the gradient is the same bits from run to run; each
+// block writes its sums to partials [blockIdx.x][n_params] for
+// k_nj_grad_reduce.
+__global__ void __launch_bounds__(kNjThreads, 2)
 k_nj_pairs_bwd(const __grid_constant__ NjGeom G, const __grid_constant__ NjNetDev N, const float* params, int n,
                const double* x, const float* qv, const float* d_el, const float* d_j, float* partials)
 {
   extern __shared__ float4 nj_smem4[];
-  const NjSmem m = nj_stage(G, N, params, reinterpret_cast<float*>(nj_smem4));
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  float4* buf = m.chain + wib * kNjH;
-  float4* dbuf = m.chain + (kNjWarps + wib) * kNjH;
-  const int D = N.D;
-  const int H = kNjH, oW1 = 0, ob1 = H * D, oW2 = ob1 + H, ob2 = oW2 + H * H, ow3 = ob2 + H, ob3 = ow3 + H;
-  const int np = ob3 + 1;
-  // block accumulator of the gradient, then one layer-1 slice per warp
-  // (W1 and b1, the first ob1 + H entries of the parameter vector)
-  float* acc = reinterpret_cast<float*>(m.chain + 2 * kNjWarps * kNjH);
-  const int np1 = ob1 + H;
-  float* acc1 = acc + np;
-  float* my1 = acc1 + wib * np1;
-  for (int t = threadIdx.x; t < np; t += blockDim.x) acc[t] = 0.0f;
-  for (int t = threadIdx.x; t < kNjWarps * np1; t += blockDim.x) acc1[t] = 0.0f;
-  __syncthreads();
-  float gW2[2][kNjH];
-  float gb2[2] = {0.0f, 0.0f}, gw3[2] = {0.0f, 0.0f};
-  float gb3 = 0.0f;
+  const NjSmem m = nj_stage(G, N, params, reinterpret_cast<float*>(nj_smem4), true);
+  const int pg = threadIdx.x >> 4, ug = threadIdx.x & 15, lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int D = N.D, F = N.F, H = kNjH;
+  const int oW1 = 0, ob1 = H * D, oW2 = ob1 + H, ob2 = oW2 + H * H, ow3 = ob2 + H, ob3 = ow3 + H, np = ob3 + 1;
+  float gW2[4][8], gb2[4] = {0.0f, 0.0f, 0.0f, 0.0f}, gw3[4] = {0.0f, 0.0f, 0.0f, 0.0f}, gb3 = 0.0f;
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int v = 0; v < kNjH; ++v) gW2[h][v] = 0.0f;
+    for (int b = 0; b < 8; ++b) gW2[a][b] = 0.0f;
+  const float4 w34 = *reinterpret_cast<const float4*>(m.w3 + 4 * ug);
+  const float w3[4] = {w34.x, w34.y, w34.z, w34.w};
+  float* my1 = m.acc1 + wib * D * H;
   const long long total = (long long)n * G.n_pairs;
-  for (long long p = (long long)blockIdx.x * kNjWarps + wib; p < total; p += (long long)gridDim.x * kNjWarps) {
-    const size_t cfg = (size_t)(p / G.n_pairs);
-    const int q = (int)(p % G.n_pairs);
-    const PairGeo pg = pair_geo(G, m, x, cfg, q);
-    // upstream derivatives
-    const float de = d_el[cfg], dj = d_j[cfg];
-    const float* qi = qv + (cfg * G.N + pg.i) * 3;
-    float dg1, dg2;
-    if (pg.is_en) {
-      const float qe = qi[0] * pg.e[0] + qi[1] * pg.e[1] + qi[2] * pg.e[2];
-      dg1 = de * (-qe - 1.0f / pg.r);
-      dg2 = -0.5f * de;
-    } else {
-      const float* qj = qv + (cfg * G.N + pg.j) * 3;
-      const float qe = (qi[0] - qj[0]) * pg.e[0] + (qi[1] - qj[1]) * pg.e[1] + (qi[2] - qj[2]) * pg.e[2];
-      dg1 = de * (-qe - 2.0f / pg.r);
-      dg2 = -de;
-    }
-    float s, s1, s2;
-    cutoff(pg.r, N.rcut[pg.c], s, s1, s2);
-    const float dm = dj * s + dg1 * s1 + dg2 * s2;
-    const float dm1 = dg1 * s + 2.0f * dg2 * s1;
-    const float dm2 = dg2 * s;
-    // forward recomputation
-    float f0[kNjMaxF], f1[kNjMaxF], f2[kNjMaxF];
-    features(N, pg.r, f0, f1, f2);
-    Fwd o;
-    fwd_layers(N, m, buf, lane, pg.c, f0, f1, f2, o);
-    gb3 += dm;  // counted on every lane; lane 0's value is used
-    // output layer and layer-2 activation
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int u = lane + 32 * h;
-      float a, d1, d2, d3;
-      silu3(o.y[h], a, d1, d2, d3);
-      const float k1 = d1 * o.y1[h], k2 = d2 * o.y1[h] * o.y1[h] + d1 * o.y2[h];
-      gw3[h] += dm * a + dm1 * k1 + dm2 * k2;
-      const float w = m.w3[u];
-      const float dh = w * dm, dh1 = w * dm1, dh2 = w * dm2;
-      const float dz = dh * d1 + dh1 * d2 * o.y1[h] + dh2 * (d3 * o.y1[h] * o.y1[h] + d2 * o.y2[h]);
-      const float dz1 = dh1 * d1 + 2.0f * dh2 * d2 * o.y1[h];
-      const float dz2 = dh2 * d1;
-      gb2[h] += dz;
-#pragma unroll
-      for (int v = 0; v < kNjH; ++v) {
-        const float4 av = buf[v];
-        gW2[h][v] = fmaf(dz, av.x, fmaf(dz1, av.y, fmaf(dz2, av.z, gW2[h][v])));
+  for (long long base = (long long)blockIdx.x * kNjSuper; base < total; base += (long long)gridDim.x * kNjSuper) {
+    __syncthreads();
+    {
+      // upstream derivatives of this thread's pair (0 beyond the total)
+      const bool in = base + threadIdx.x < total;
+      size_t cfg;
+      int code;
+      super_geometry(G, m, x, min(base + threadIdx.x, total - 1), cfg, code);
+      const int i = code & 0xFF, j = (code >> 8) & 0xFF, c = code >> 16;
+      const float4 e = m.geo[threadIdx.x];
+      const float de = in ? d_el[cfg] : 0.0f, dj = in ? d_j[cfg] : 0.0f;
+      const float* qi = qv + (cfg * G.N + i) * 3;
+      float dg1, dg2;
+      if (c >= 2) {
+        const float qe = qi[0] * e.y + qi[1] * e.z + qi[2] * e.w;
+        dg1 = de * (-qe - 1.0f / e.x);
+        dg2 = -0.5f * de;
+      } else {
+        const float* qj = qv + (cfg * G.N + j) * 3;
+        const float qe = (qi[0] - qj[0]) * e.y + (qi[1] - qj[1]) * e.z + (qi[2] - qj[2]) * e.w;
+        dg1 = de * (-qe - 2.0f / e.x);
+        dg2 = -de;
       }
-      dbuf[u] = make_float4(dz, dz1, dz2, 0.0f);
-    }
-    __syncwarp();
-    // layer-1 activations: da = W2^T dz (chains), then through silu
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int v = lane + 32 * h;
-      float da = 0.0f, da1 = 0.0f, da2 = 0.0f;
-#pragma unroll 8
-      for (int u = 0; u < kNjH; ++u) {
-        const float4 d = dbuf[u];
-        const float w = m.W2[u * kNjH + v];
-        da = fmaf(w, d.x, da); da1 = fmaf(w, d.y, da1); da2 = fmaf(w, d.z, da2);
-      }
-      float a, d1, d2, d3;
-      silu3(o.z[h], a, d1, d2, d3);
-      const float z1 = o.z1[h], z2 = o.z2[h];
-      const float dz = da * d1 + da1 * d2 * z1 + da2 * (d3 * z1 * z1 + d2 * z2);
-      const float dz1 = da1 * d1 + 2.0f * da2 * d2 * z1;
-      const float dz2 = da2 * d1;
-      // hidden unit v belongs to this lane alone within the warp's slice
-      my1[ob1 + v] += dz;
-      my1[oW1 + v * D + N.F + pg.c] += dz;
-#pragma unroll
-      for (int f = 0; f < kNjMaxF; ++f)
-        if (f < N.F) my1[oW1 + v * D + f] += dz * f0[f] + dz1 * f1[f] + dz2 * f2[f];
-    }
-    __syncwarp();
-  }
-  // block reduction in warp order (a lane owns output units u, so the adds
-  // of one warp touch distinct entries), layer 1 from the warp slices
-  __syncthreads();
-  for (int w = 0; w < kNjWarps; ++w) {
-    if (wib == w) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int u = lane + 32 * h;
-#pragma unroll
-        for (int v = 0; v < kNjH; ++v) acc[oW2 + u * H + v] += gW2[h][v];
-        acc[ob2 + u] += gb2[h];
-        acc[ow3 + u] += gw3[h];
-      }
-      if (lane == 0) acc[ob3] += gb3;
+      float s, s1, s2;
+      cutoff(e.x, N.rcut[c], s, s1, s2);
+      m.up[threadIdx.x] = in ? make_float4(dj * s + dg1 * s1 + dg2 * s2, dg1 * s + 2.0f * dg2 * s1, dg2 * s, 0.0f)
+                             : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     __syncthreads();
+#pragma unroll 1
+    for (int sub = 0; sub < kNjSuper / kNjTile && base + sub * kNjTile < total; ++sub) {
+      float y[3][4][4];
+      tile_forward(N, m, sub, pg, ug, y);
+      // output layer and layer-2 activation; the derivatives of the layer-2
+      // chains into Z
+      float tb2[4] = {0.0f, 0.0f, 0.0f, 0.0f}, tw3[4] = {0.0f, 0.0f, 0.0f, 0.0f}, tb3 = 0.0f;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const float4 d = m.up[sub * kNjTile + 4 * pg + p];
+        if (ug == 0) tb3 += d.x;
+        float v[3][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float y1 = y[1][p][u], y2 = y[2][p][u];
+          float a, d1, d2, d3;
+          silu3(y[0][p][u], a, d1, d2, d3);
+          const float k1 = d1 * y1, k2 = d2 * y1 * y1 + d1 * y2;
+          tw3[u] += d.x * a + d.y * k1 + d.z * k2;
+          const float dh = w3[u] * d.x, dh1 = w3[u] * d.y, dh2 = w3[u] * d.z;
+          v[0][u] = dh * d1 + dh1 * d2 * y1 + dh2 * (d3 * y1 * y1 + d2 * y2);
+          v[1][u] = dh1 * d1 + 2.0f * dh2 * d2 * y1;
+          v[2][u] = dh2 * d1;
+          tb2[u] += v[0][u];
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          *reinterpret_cast<float4*>(m.Z + (c * kNjTile + 4 * pg + p) * kNjLd + 4 * ug) =
+              make_float4(v[c][0], v[c][1], v[c][2], v[c][3]);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        gb2[u] += tb2[u];
+        gw3[u] += tw3[u];
+      }
+      gb3 += tb3;
+      __syncthreads();
+      // weight gradient: units 4 ug .., inputs 8 pg ..; the tile's sum is
+      // formed first (a pair's three chains, which largely cancel, together)
+      {
+        float gt[4][8];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) gt[a][b] = 0.0f;
+#pragma unroll 1
+        for (int p = 0; p < kNjTile; ++p)
+#pragma unroll
+          for (int c = 2; c >= 0; --c) {
+            const int r = c * kNjTile + p;
+            const float4 z = *reinterpret_cast<const float4*>(m.Z + r * kNjLd + 4 * ug);
+            const float4 a0 = *reinterpret_cast<const float4*>(m.A + r * kNjLd + 8 * pg);
+            const float4 a1 = *reinterpret_cast<const float4*>(m.A + r * kNjLd + 8 * pg + 4);
+            fma4(gt[0], z.x, a0); fma4(gt[0] + 4, z.x, a1);
+            fma4(gt[1], z.y, a0); fma4(gt[1] + 4, z.y, a1);
+            fma4(gt[2], z.z, a0); fma4(gt[2] + 4, z.z, a1);
+            fma4(gt[3], z.w, a0); fma4(gt[3] + 4, z.w, a1);
+          }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 8; ++b) gW2[a][b] += gt[a][b];
+      }
+      // derivatives of the layer-1 activations, W2^T dz, then through silu
+      float da[3][4][4];
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) da[c][p][u] = 0.0f;
+      row_product(m.Z, m.W2, pg, ug, da);
+      layer1(N, m, sub, pg, ug, y);
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float z1 = y[1][p][u], z2 = y[2][p][u];
+          float a, d1, d2, d3;
+          silu3(y[0][p][u], a, d1, d2, d3);
+          const float e0 = da[0][p][u], e1 = da[1][p][u], e2 = da[2][p][u];
+          da[0][p][u] = e0 * d1 + e1 * d2 * z1 + e2 * (d3 * z1 * z1 + d2 * z2);
+          da[1][p][u] = e1 * d1 + 2.0f * e2 * d2 * z1;
+          da[2][p][u] = e2 * d1;
+        }
+      // layer-1 gradient: the warp's two pair groups added, then into its slice
+#pragma unroll 1
+      for (int f = 0; f < F; ++f) {
+        float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float4 ft = m.feat[(4 * pg + p) * F + f];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            g[u] += da[0][p][u] * ft.x + da[1][p][u] * ft.y + da[2][p][u] * ft.z;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) g[u] += __shfl_xor_sync(0xffffffffu, g[u], 16);
+        if (lane < 16) {
+          float4* o = reinterpret_cast<float4*>(my1 + f * H + 4 * ug);
+          float4 t = *o;
+          t.x += g[0]; t.y += g[1]; t.z += g[2]; t.w += g[3];
+          *o = t;
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if ((lane >> 4) == h) {
+            float4* o = reinterpret_cast<float4*>(my1 + (F + m.ch[sub * kNjTile + 4 * pg + p]) * H + 4 * ug);
+            float4 t = *o;
+            t.x += da[0][p][0]; t.y += da[0][p][1]; t.z += da[0][p][2]; t.w += da[0][p][3];
+            *o = t;
+          }
+          __syncwarp();
+        }
+      __syncthreads();  // the features and Z are free again
+    }
   }
-  for (int t = threadIdx.x; t < np1; t += blockDim.x) {
-    float a = 0.0f;
-    for (int w = 0; w < kNjWarps; ++w) a += acc1[w * np1 + t];
-    acc[t] = a;
-  }
-  __syncthreads();
+  // block totals: the weight gradient is the threads' own; the others are
+  // added over the pair groups (layers 2 and 3) or warps (layer 1) in order
   float* out = partials + (size_t)blockIdx.x * np;
-  for (int t = threadIdx.x; t < np; t += blockDim.x) out[t] = acc[t];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) out[oW2 + (4 * ug + a) * H + 8 * pg + b] = gW2[a][b];
+  __syncthreads();
+  float* red = m.A;  // [8][2][H], then [8]
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    red[(pg * 2) * H + 4 * ug + u] = gb2[u];
+    red[(pg * 2 + 1) * H + 4 * ug + u] = gw3[u];
+  }
+  if (ug == 0) red[16 * H + pg] = gb3;
+  __syncthreads();
+  for (int t = threadIdx.x; t < H; t += blockDim.x) {
+    float a = 0.0f, b = 0.0f;
+    for (int g = 0; g < 8; ++g) {
+      a += red[(g * 2) * H + t];
+      b += red[(g * 2 + 1) * H + t];
+    }
+    out[ob2 + t] = a;
+    out[ow3 + t] = b;
+    float c1 = 0.0f;
+    for (int f = 0; f < D; ++f) {
+      float w = 0.0f;
+      for (int g = 0; g < 4; ++g) w += m.acc1[(g * D + f) * H + t];
+      out[oW1 + t * D + f] = w;
+      if (f >= F) c1 += w;  // every pair has one channel
+    }
+    out[ob1 + t] = c1;
+  }
+  if (threadIdx.x == 0) {
+    float a = 0.0f;
+    for (int g = 0; g < 8; ++g) a += red[16 * H + g];
+    out[ob3] = a;
+  }
 }
 
-// grad[t] = sum over the backward blocks of partials[b][t], in block order.
+// grad[t] = sum over the backward blocks of partials[b][t], in block order,
+// compensated (the blocks' sums cancel).
 __global__ void k_nj_grad_reduce(const float* partials, int blocks, int np, float* grad)
 {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= np) return;
-  float a = 0.0f;
-  for (int b = 0; b < blocks; ++b) a += partials[(size_t)b * np + t];
-  grad[t] = a;
+  dl a = df_make(0.0f, 0.0f);
+#pragma unroll 8
+  for (int b = 0; b < blocks; ++b) a = dl_add_f(a, partials[(size_t)b * np + t]);
+  grad[t] = a.hi + a.lo;
 }
 
 static int nj_smem_bytes(const NjGeom& G, const NjNetDev& N, bool backward)
 {
-  // staging image and one chain buffer per warp; the backward pass adds a
-  // second chain buffer per warp and the block's gradient accumulator
-  int f = nj_smem_floats(N.D, G.n_pairs);
-  if (backward) f += 4 * kNjWarps * kNjH + nj_n_params(N.F, N.C, kNjH) + kNjWarps * (kNjH * N.D + kNjH);
-  return (int)sizeof(float) * f;
+  return (int)sizeof(float) * nj_smem_floats(N.F, N.C, G.n_pairs, backward);
 }
 
 static int nj_grid(const void* fn, int smem)
@@ -623,7 +785,7 @@ static int nj_grid(const void* fn, int smem)
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kNjWarps * 32, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kNjThreads, smem);
   return sms * (per > 0 ? per : 1);
 }
 
@@ -637,8 +799,8 @@ cudaError_t launch_nj_forward(const NjGeom& G, const NjNetDev& N, const float* p
   if (e != cudaSuccess) return e;
   const long long total = (long long)n * G.n_pairs;
   long long blocks = nj_grid((const void*)k_nj_pairs_fwd, smem);
-  blocks = std::min(blocks, (total + kNjWarps - 1) / kNjWarps);
-  k_nj_pairs_fwd<<<(int)blocks, kNjWarps * 32, smem, st>>>(G, N, params, n, x, pair_out);
+  blocks = std::min(blocks, (total + kNjSuper - 1) / kNjSuper);
+  k_nj_pairs_fwd<<<(int)blocks, kNjThreads, smem, st>>>(G, N, params, n, x, pair_out);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_nj_assemble<<<(n + 3) / 4, 128, 0, st>>>(G, n, x, grad_base, e_base, pair_out, el, j, q);
@@ -665,8 +827,8 @@ cudaError_t launch_nj_backward(const NjGeom& G, const NjNetDev& N, const float* 
                                        smem);
   if (e != cudaSuccess) return e;
   const long long total = (long long)n * G.n_pairs;
-  long long blocks = std::min((long long)max_blocks, (total + kNjWarps - 1) / kNjWarps);
-  k_nj_pairs_bwd<<<(int)blocks, kNjWarps * 32, smem, st>>>(G, N, params, n, x, q, d_el, d_j, partials);
+  long long blocks = std::min((long long)max_blocks, (total + kNjSuper - 1) / kNjSuper);
+  k_nj_pairs_bwd<<<(int)blocks, kNjThreads, smem, st>>>(G, N, params, n, x, q, d_el, d_j, partials);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_nj_grad_reduce<<<(np + 255) / 256, 256, 0, st>>>(partials, (int)blocks, np, grad);
