@@ -32,6 +32,8 @@ struct LShell {
   int kind, l, m_int, ao;      // kind 0 Slater, 1 Gaussian contraction
   int prim, n_prim, same_exp, center;
   float zeta_hi, zeta_lo, m_hi, m_lo;
+  int gt_base, gt_cells, gt_key0;
+  float gt_beta;
 };
 
 static __device__ const __align__(16) float2 g_exp_tab[kExpEntries] = {
@@ -72,6 +74,7 @@ __device__ __forceinline__ void lean_stage(const SysDev& S, double* head)
     const DfShell& d = S.D.sh[q];
     o->kind = sh.kind; o->l = sh.l; o->m_int = sh.m_int; o->ao = sh.ao_offset;
     o->prim = sh.prim_begin; o->n_prim = sh.n_prim; o->same_exp = sh.same_exp; o->center = sh.center;
+    o->gt_base = sh.gt_base; o->gt_cells = sh.gt_cells; o->gt_key0 = sh.gt_key0; o->gt_beta = sh.gt_beta;
     o->zeta_hi = d.zeta.hi; o->zeta_lo = d.zeta.lo; o->m_hi = d.m.hi; o->m_lo = d.m.lo;
     float4* pr = const_cast<float4*>(m.prim) + sh.prim_begin;
 #pragma unroll 1
@@ -493,6 +496,54 @@ __device__ __forceinline__ dl2 nj_value64_2(const SysDev& S, int c, dl2 r)
   return dl2_pack(nj_value64(S, c, a), nj_value64(S, c, b));
 }
 
+// A contracted Gaussian's radial part at two squared distances from its
+// table: cells of 1/256 octave of y = x + beta (beta about one over the
+// largest exponent: uniform cells near the nucleus, relative ones beyond),
+// the degree-7 polynomial of the cell in u = (y - centre)/width, its first
+// four coefficients as double-floats, the others single (their terms stay
+// below 2e-6 of the value while the exponent is below 40); 0 beyond the last
+// cell, where every primitive's exponent is below -87. About 75 instructions
+// for the two distances whatever the contraction length, against about 55
+// per primitive: 64 k cycles of a water walker-move's 116 k went to its 30
+// primitives.
+__device__ __forceinline__ dl2 radial_table2(const LShell& sh, const float4* gt, dl2 x)
+{
+  const dl2 y = dl2_two_sum(x.hi, f2_all(sh.gt_beta));
+  const f2 ylo = f2_add(y.lo, x.lo);
+  float yh[2], ctr[2], iw[2];
+  f2_split(y.hi, yh[0], yh[1]);
+  float4 c[2][3];
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    const unsigned key = __float_as_uint(yh[m]) >> 15;
+    const unsigned cell = key - (unsigned)sh.gt_key0;
+    ctr[m] = __uint_as_float((key << 15) | 0x4000u);
+    iw[m] = __uint_as_float((262u - (key >> 8)) << 23);
+    if (cell < (unsigned)sh.gt_cells) {
+      const float4* p = gt + 3 * (size_t)(sh.gt_base + (int)cell);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) c[m][q] = __ldg(p + q);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) c[m][q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      ctr[m] = yh[m];
+      iw[m] = 0.0f;
+    }
+  }
+  const f2 w = f2_make(iw[0], iw[1]);
+  const dl2 u = dl2_make(f2_mul(f2_sub(y.hi, f2_make(ctr[0], ctr[1])), w), f2_mul(ylo, w));
+#define LRDMC_C(q, f) f2_make(c[0][q].f, c[1][q].f)
+  f2 t = f2_fma(u.hi, LRDMC_C(2, w), LRDMC_C(2, z));
+  t = f2_fma(u.hi, t, LRDMC_C(2, y));
+  t = f2_fma(u.hi, t, LRDMC_C(2, x));
+  dl2 v = dl2_fast_two_sum(LRDMC_C(1, z), f2_fma(u.hi, t, LRDMC_C(1, w)));
+  v = dl2_add(dl2_make(LRDMC_C(1, x), LRDMC_C(1, y)), dl2_mul(u, v));
+  v = dl2_add(dl2_make(LRDMC_C(0, z), LRDMC_C(0, w)), dl2_mul(u, v));
+  v = dl2_add(dl2_make(LRDMC_C(0, x), LRDMC_C(0, y)), dl2_mul(u, v));
+#undef LRDMC_C
+  return v;
+}
+
 // One partner of the e-e sums of the moves +-h e_k: Dh = b^2 (D + h^2), p =
 // 2 b^2 h (y_ik - y_jk)/b; acc receives q (or s q, the general form).
 template <bool NJ>
@@ -511,10 +562,11 @@ __device__ __forceinline__ void ee_partner64(const SysDev& S, dl Dh, dl p, int c
 }
 
 // The two lattice moves +-h e_k of unit u = (electron, grid, axis): rates
-// into Td, ratios into ratio_out (nullable).
+// into Td, ratios into ratio_out (nullable). gt: the radial table, or null
+// (the stateless evaluations, which keep no device memory for a system).
 template <bool NJ, bool NC>
 __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const WarpMem& wm, const Lean& lt, int u,
-                                        df* Td, double* ratio_out)
+                                        df* Td, double* ratio_out, const float4* gt)
 {
   const int G = L.G, i = u / (3 * G), rem = u - i * 3 * G, g = rem / 3, k = rem - 3 * g;
   const int nu = S.n_up;
@@ -566,6 +618,8 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
           if (!sh.same_exp)
             e = dl2_exp(dl2_norm(dl2_mul(dl2_all(df_make(-sh.zeta_hi, -sh.zeta_lo)), r)), S.D.lexp, lt.tab);
           R = sh.m_int == 0 ? e : dl2_mul(slater_power2(sh, r, S, lt), e);
+        } else if (gt && sh.gt_cells) {
+          R = radial_table2(sh, gt, r2);
         } else {
           R = dl2_zero();
 #pragma unroll 1
@@ -873,14 +927,14 @@ __device__ __forceinline__ void total_jastrow64(const SysDev& S, const WarpMem& 
 // One whole evaluation (stateless evaluation, change of lattice).
 template <bool NJ, bool NC>
 __device__ void warp_eval64(const SysDev& S, double* sC, const LatDev& L, const WarpMem& wm, int lane,
-                            double* ratio_out, double& b, double& el)
+                            double* ratio_out, double& b, double& el, const float4* gt)
 {
   const Lean lt = lean_mem(S, sC);
   el = prelude64<NJ, NC>(S, sC, wm, lt, lane, -1);
   const int units = 3 * L.G * S.N;
   df* Td = reinterpret_cast<df*>(wm.T);
 #pragma unroll 1
-  for (int u = lane; u < units; u += 32) moves64<NJ, NC>(S, L, wm, lt, u, Td, ratio_out);
+  for (int u = lane; u < units; u += 32) moves64<NJ, NC>(S, L, wm, lt, u, Td, ratio_out, gt);
   __syncwarp();
   b = df_to_double(rate_scan64(Td, 2 * units, lane, wm.pfx));
 }

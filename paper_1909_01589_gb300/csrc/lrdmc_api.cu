@@ -75,6 +75,9 @@ struct lrdmc_system_s {
   int blocks = 0;  // persistent grid of the interval kernel (0 = occupancy default)
   int helpers = 1;  // tail helpers of the interval kernel (lrdmc_set_tail_helpers)
   uint64_t version = 0;  // bumped whenever kernel arguments change (batches re-capture)
+  // radial table of the Gaussian shells, made with the population
+  float4* gt_tab = nullptr;
+  int gt_dev = -1;
   // neural pair term (lrdmc_set_neural_jastrow)
   double* nj_tab = nullptr;
   df* nj_tab_df = nullptr;
@@ -478,6 +481,7 @@ lrdmc_status lrdmc_create_system(int n_nuc, const double* nuc_xyz, const double*
       }
   S.precision = LRDMC_PRECISION_DF64;
   fill_df_constants(S);
+  plan_radial_table(S);
   // one block holds kWarpsPerBlock walkers in shared memory; without room
   // for the evaluation caches the system runs without them, and a system
   // that does not fit even then is rejected
@@ -617,6 +621,25 @@ lrdmc_status lrdmc_init_walkers(lrdmc_system_t s, int W, const double* x0, uint6
   P.tau = tau;
   P.e_trial = e_trial;
   P.helpers = s->helpers;
+  P.gt = nullptr;
+  if (s->S.gt_total > 0) {
+    // the table on the population's device (without memory for it the
+    // primitives are summed directly)
+    int dev = -1;
+    if (cudaGetDevice(&dev) == cudaSuccess && (!s->gt_tab || dev != s->gt_dev)) {
+      if (s->gt_tab) cudaFree(s->gt_tab);
+      s->gt_tab = nullptr;
+      if (cudaMalloc((void**)&s->gt_tab, sizeof(float4) * 3 * (size_t)s->S.gt_total) != cudaSuccess) {
+        cudaGetLastError();
+        s->gt_tab = nullptr;
+      } else {
+        s->gt_dev = dev;
+        cudaError_t et = launch_radial_table(s->S, s->gt_tab, s->stream);
+        if (et != cudaSuccess) return cuda_fail(s, et, "radial table");
+      }
+    }
+    P.gt = s->gt_tab;
+  }
   // moves, err, counter, kdev, resid, ticket
   cudaError_t e = cudaMemsetAsync(s->ws + p.moves, 0, 6 * 256, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "workspace clear");
@@ -1551,6 +1574,7 @@ void lrdmc_destroy(lrdmc_system_t s)
   if (!s) return;
   if (s->err_host) cudaFreeHost(s->err_host);
   if (s->eval_err) cudaFree(s->eval_err);
+  if (s->gt_tab) cudaFree(s->gt_tab);
   if (s->nj_tab) cudaFree(s->nj_tab);
   if (s->nj_tab_df) cudaFree(s->nj_tab_df);
   if (s->base_err) cudaFree(s->base_err);

@@ -72,6 +72,10 @@ struct ShellDev {
   int m_int;       // Slater power r^m as an integer (>= 0), or -1 for pow()
   int same_exp;    // 1: same centre and Slater exponent as the previous shell
   int prim_begin;  // first primitive among those of all Gaussian shells
+  // the shell's cells in the radial table (gt_cells of them from cell gt_base
+  // on; 0: not tabulated), the key of the first one and the table's offset
+  int gt_base, gt_cells, gt_key0;
+  float gt_beta;
   double m;        // n_eff - 1 - l
   double zeta;
   double alpha[kMaxPrim];
@@ -128,6 +132,7 @@ struct SysDev {
   int n_grp64;
   int grp64_first[kMaxShell + 1];
   int n_prim;       // primitives of all Gaussian shells
+  int gt_total;     // cells of the radial table
   int ee_recip;     // 1: the e-e Pade sum in the reciprocal form (b >= 1/4)
   float ee_sign;    // sign of b (0 for b = 0)
   // the non-zero MO coefficients: bit m of row_mask[mu] and bit mu of
@@ -226,6 +231,7 @@ struct CombPart {
 };
 
 struct PopDev {
+  const float4* gt;  // radial table of the Gaussian shells (null: none), [gt_total][3]
   double* rec_src;
   double* rec_dst;
   int* parent;
@@ -260,6 +266,9 @@ struct PopDev {
 };
 
 void fill_df_constants(SysDev& S);
+// Lays out the radial table (gt_* of the shells), and fills it on the device.
+void plan_radial_table(SysDev& S);
+cudaError_t launch_radial_table(const SysDev& S, float4* tab, cudaStream_t st);
 void fill_lattice_df(LatDev& L);
 
 cudaError_t launch_init(const SysDev& S, const Layout& Lo, const PopDev& P, const double* x0,

@@ -24,6 +24,7 @@
 // parent[s] from the source buffer, so reconfiguration needs no copy pass.
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <cuda_bf16.h>
 
@@ -1163,10 +1164,11 @@ __device__ void warp_eval32(const SysDev& S, double* sC, const LatDev& L, const 
 
 template <int PREC, bool NJ, bool NC>
 __device__ __forceinline__ void warp_eval_any(const SysDev& S, double* sC, const LatDev& L, const WarpMem& wm,
-                                              int lane, double* ratio_out, double& b, double& el)
+                                              int lane, double* ratio_out, double& b, double& el,
+                                              const float4* gt = nullptr)
 {
   if (PREC == LRDMC_PRECISION_DF64) {
-    warp_eval64<NJ, NC>(S, sC, L, wm, lane, ratio_out, b, el);
+    warp_eval64<NJ, NC>(S, sC, L, wm, lane, ratio_out, b, el, gt);
   } else if (PREC == LRDMC_PRECISION_FP32) {
     warp_eval32<NJ>(S, sC, L, wm, lane, ratio_out, b, el);
   } else {
@@ -1309,7 +1311,7 @@ k_eval_all(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
   double* rec = P.rec_src + (size_t)s * Lo.rec;
   double b, el;
   load_record(Lo, rec, wm, lane, b, el);
-  warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, el);
+  warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, el, P.gt);
   if (!isfinite(el) || !isfinite(b)) {
     if (lane == 0) atomicOr(P.err, kErrNonFinite);
   }
@@ -1375,7 +1377,7 @@ __device__ __forceinline__ int team_publish(TeamSlot* t, int lane)
 // A unit is one move, in the double-float mode the two moves along one axis.
 template <class NT, bool NJ, bool NC>
 __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, const WarpMem& wm, const BlockMem& bm,
-                                              const Lean& lt, TeamSlot* t, int units, int lane)
+                                              const Lean& lt, TeamSlot* t, int units, int lane, const float4* gt)
 {
   df* Td = reinterpret_cast<df*>(wm.T);
   // chunks of 16 moves in a team (more helpers take part in a small
@@ -1393,7 +1395,7 @@ __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, 
     }
     if (c0 >= units) break;
     if (lane < cs && c0 + lane < units) {
-      if (sizeof(NT) == sizeof(df)) moves64<NJ, NC>(S, L, wm, lt, c0 + lane, Td, nullptr);
+      if (sizeof(NT) == sizeof(df)) moves64<NJ, NC>(S, L, wm, lt, c0 + lane, Td, nullptr, gt);
       else candidate_m<float, NJ>(S, L, wm, bm, c0 + lane, Td, nullptr);
     }
   }
@@ -1680,7 +1682,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
     {
       const WarpMem twm = warp_mem(Lo, S, sC + Lo.head + target * Lo.smem_warp);
       chunked_moves<NT, NJ, NC>(S, L, twm, bm, lt, (mode == kHelper || nh > 0) ? &g_team[target] : nullptr, units,
-                                lane);
+                                lane, P.gt);
     }
     if (mode == kHelper) {
       if (lane == 0) atomicAdd(&g_team[target].done, 1);
@@ -2261,6 +2263,87 @@ void fill_df_constants(SysDev& S)
     D.inv_fact[k] = split_ld(1.0L / f);
   }
   D.half_pi = split_ld(2.0L * atanl(1.0L));
+}
+
+// The radial table pays from three primitives on (about 75 instructions per
+// pair of distances against 55 per primitive); a shell whose exponents span so
+// much that it would take over kMaxCells cells (0.8 MB) is summed directly.
+constexpr int kMaxCells = 16384;
+static uint32_t cell_key(float y)
+{
+  uint32_t u;
+  memcpy(&u, &y, 4);
+  return u >> 15;
+}
+
+void plan_radial_table(SysDev& S)
+{
+  S.gt_total = 0;
+  for (int q = 0; q < S.n_shell; ++q) {
+    ShellDev& sh = S.sh[q];
+    sh.gt_cells = 0;
+    if (sh.kind != 1 || sh.n_prim < 3) continue;
+    double lo = sh.alpha[0], hi = sh.alpha[0];
+    bool fine = true;
+    for (int p = 0; p < sh.n_prim; ++p) {
+      lo = std::min(lo, sh.alpha[p]);
+      hi = std::max(hi, sh.alpha[p]);
+      fine = fine && std::isfinite(sh.alpha[p]) && std::isfinite(sh.coef[p]);
+    }
+    if (!fine || !(lo > 1e-6) || !(hi < 1e12)) continue;
+    sh.gt_beta = (float)exp2(floor(-log2(hi)));
+    sh.gt_key0 = (int)cell_key(sh.gt_beta);
+    const int n = (int)cell_key((float)(87.0 / lo + sh.gt_beta)) - sh.gt_key0 + 1;
+    if (n > kMaxCells) continue;
+    sh.gt_base = S.gt_total;
+    sh.gt_cells = n;
+    S.gt_total += n;
+  }
+}
+
+// One cell per thread: the Taylor coefficients of sum_p c_p e^(-alpha_p x) at
+// the cell's centre to degree 9 in u, the last two economised onto the lower
+// ones by Chebyshev polynomials (the remainder is 2^-15 of the degree-8 term).
+__global__ void __launch_bounds__(128) k_radial_table(const __grid_constant__ SysDev S, float4* tab)
+{
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= S.gt_total) return;
+  int q = 0;
+  while (S.sh[q].gt_cells == 0 || id < S.sh[q].gt_base || id >= S.sh[q].gt_base + S.sh[q].gt_cells) ++q;
+  const ShellDev& sh = S.sh[q];
+  const unsigned key = (unsigned)(sh.gt_key0 + id - sh.gt_base);
+  const double y0 = __uint_as_float(key << 15), w = (double)__uint_as_float((key + 1) << 15) - y0;
+  const double x = y0 + 0.5 * w - (double)sh.gt_beta;
+  double c[10];
+  for (int j = 0; j < 10; ++j) c[j] = 0.0;
+  for (int p = 0; p < sh.n_prim; ++p) {
+    const double al = sh.alpha[p], z = al * x, r = fma(al, x, -z);
+    double t = sh.coef[p] * exp(-z);
+    t -= t * r;
+    for (int j = 0; j < 10; ++j) {
+      c[j] += t;
+      t *= -al * w / (j + 1);
+    }
+  }
+  c[7] += 0.5625 * c[9];
+  c[5] -= 0.10546875 * c[9];
+  c[3] += 0.00732421875 * c[9];
+  c[1] -= 0.0001373291015625 * c[9];
+  c[6] += 0.5 * c[8];
+  c[4] -= 0.078125 * c[8];
+  c[2] += 0.00390625 * c[8];
+  c[0] -= 0.000030517578125 * c[8];
+  df d[4];
+  for (int j = 0; j < 4; ++j) d[j] = df_from_double(c[j]);
+  tab[3 * (size_t)id] = make_float4(d[0].hi, d[0].lo, d[1].hi, d[1].lo);
+  tab[3 * (size_t)id + 1] = make_float4(d[2].hi, d[2].lo, d[3].hi, d[3].lo);
+  tab[3 * (size_t)id + 2] = make_float4((float)c[4], (float)c[5], (float)c[6], (float)c[7]);
+}
+
+cudaError_t launch_radial_table(const SysDev& S, float4* tab, cudaStream_t st)
+{
+  k_radial_table<<<(S.gt_total + 127) / 128, 128, 0, st>>>(S, tab);
+  return cudaGetLastError();
 }
 
 void fill_lattice_df(LatDev& L)
