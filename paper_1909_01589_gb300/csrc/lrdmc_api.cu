@@ -8,6 +8,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <functional>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -33,7 +35,7 @@ struct NvtxRange {
 // Quadrature of Eq. 7 for one Z (core_quadrature).
 constexpr int kPanels = 240, kPanelNodes = 24;
 struct CoreQuadrature {
-  int Z = 0;
+  std::once_flag made;
   double edge[kPanels + 1];           // panel limits
   std::vector<double> r, w, f;        // nodes, weights, density
   std::vector<double> later;          // largest w f from a panel on
@@ -77,6 +79,7 @@ struct lrdmc_system_s {
   uint64_t version = 0;  // bumped whenever kernel arguments change (batches re-capture)
   // radial table of the Gaussian shells, made with the population
   float4* gt_tab = nullptr;
+  cudaEvent_t gt_ready = nullptr;
   int gt_dev = -1;
   // neural pair term (lrdmc_set_neural_jastrow)
   double* nj_tab = nullptr;
@@ -230,12 +233,11 @@ static void core_quadrature(CoreQuadrature& c, int Z)
     for (int i = 0; i < kPanelNodes; ++i)
       c.later[p] = fmax(c.later[p], c.w[p * kPanelNodes + i] * c.f[p * kPanelNodes + i]);
   }
-  c.Z = Z;
 }
 
 static double n_core(CoreQuadrature& c, int Z, double rc)
 {
-  if (c.Z != Z) core_quadrature(c, Z);
+  std::call_once(c.made, core_quadrature, std::ref(c), Z);
   const bool gauss = rc > 0.0 && isfinite(rc);
   double total = 0.0;
   for (int p = 0; p < kPanels; ++p) {
@@ -568,6 +570,56 @@ static lrdmc_status read_error_word(lrdmc_system_t s)
   return LRDMC_OK;
 }
 
+static void free_radial_table(lrdmc_system_t s)
+{
+  if (s->gt_tab) cudaFree(s->gt_tab);
+  if (s->gt_ready) cudaEventDestroy(s->gt_ready);
+  s->gt_tab = nullptr;
+  s->gt_ready = nullptr;
+}
+
+// The radial table on the population's device and ready in its stream: made
+// once per system and device; a population in another stream waits for it.
+// Null (the primitives are summed directly) without memory for it and while
+// the stream is being captured, when neither an allocation nor a wait on
+// work outside the capture is allowed.
+static cudaError_t radial_table(lrdmc_system_t s, const float4** out)
+{
+  *out = nullptr;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int dev = -1;
+  cudaError_t e = cudaStreamIsCapturing(s->stream, &cap);
+  if (e != cudaSuccess) return e;
+  if (cap != cudaStreamCaptureStatusNone) return cudaSuccess;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (s->gt_tab && dev == s->gt_dev) {
+    *out = s->gt_tab;
+    return cudaStreamWaitEvent(s->stream, s->gt_ready, 0);
+  }
+  free_radial_table(s);
+  // another thread may be capturing: its capture is none of this call's
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  e = cudaMalloc((void**)&s->gt_tab, sizeof(float4) * 3 * (size_t)s->S.gt_total);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    s->gt_tab = nullptr;
+    return cudaSuccess;
+  }
+  s->gt_dev = dev;
+  e = cudaEventCreateWithFlags(&s->gt_ready, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = launch_radial_table(s->S, s->gt_tab, s->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(s->gt_ready, s->stream);
+  if (e != cudaSuccess) {
+    free_radial_table(s);
+    return e;
+  }
+  *out = s->gt_tab;
+  return cudaSuccess;
+}
+
 lrdmc_status lrdmc_init_walkers(lrdmc_system_t s, int W, const double* x0, uint64_t seed, double tau,
                                 double e_trial, int recompute_every, int cap, void* workspace,
                                 size_t ws_bytes, void* stream)
@@ -623,22 +675,8 @@ lrdmc_status lrdmc_init_walkers(lrdmc_system_t s, int W, const double* x0, uint6
   P.helpers = s->helpers;
   P.gt = nullptr;
   if (s->S.gt_total > 0) {
-    // the table on the population's device (without memory for it the
-    // primitives are summed directly)
-    int dev = -1;
-    if (cudaGetDevice(&dev) == cudaSuccess && (!s->gt_tab || dev != s->gt_dev)) {
-      if (s->gt_tab) cudaFree(s->gt_tab);
-      s->gt_tab = nullptr;
-      if (cudaMalloc((void**)&s->gt_tab, sizeof(float4) * 3 * (size_t)s->S.gt_total) != cudaSuccess) {
-        cudaGetLastError();
-        s->gt_tab = nullptr;
-      } else {
-        s->gt_dev = dev;
-        cudaError_t et = launch_radial_table(s->S, s->gt_tab, s->stream);
-        if (et != cudaSuccess) return cuda_fail(s, et, "radial table");
-      }
-    }
-    P.gt = s->gt_tab;
+    cudaError_t et = radial_table(s, &P.gt);
+    if (et != cudaSuccess) return cuda_fail(s, et, "radial table");
   }
   // moves, err, counter, kdev, resid, ticket
   cudaError_t e = cudaMemsetAsync(s->ws + p.moves, 0, 6 * 256, s->stream);
@@ -1574,7 +1612,7 @@ void lrdmc_destroy(lrdmc_system_t s)
   if (!s) return;
   if (s->err_host) cudaFreeHost(s->err_host);
   if (s->eval_err) cudaFree(s->eval_err);
-  if (s->gt_tab) cudaFree(s->gt_tab);
+  free_radial_table(s);
   if (s->nj_tab) cudaFree(s->nj_tab);
   if (s->nj_tab_df) cudaFree(s->nj_tab_df);
   if (s->base_err) cudaFree(s->base_err);

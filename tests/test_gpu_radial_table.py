@@ -71,3 +71,23 @@ def test_tabulated_rates_match_oracle(pkg, kind):
         scale = U.ratio_scale(o, system, lat, x0[w], R, ref["ratio"])
         tol = U.rate_tolerance(lat, ref["w"], scale, w_abs=U.W_ABS)
         assert np.all(np.abs(got["T"][t] - ref["T"]) <= tol), (w, np.max(np.abs(got["T"][t] - ref["T"]) / tol))
+
+
+def test_table_reaches_a_population_of_another_stream(pkg):
+    """A system whose table was made in one stream and that takes a new
+    population in another stream: the same walkers bit for bit."""
+    rng = np.random.default_rng(2)
+    x0 = rng.normal(size=(64, 4, 3))
+
+    def project(g):
+        g.init_walkers(x0, seed=3, tau=0.02, trace_capacity=8)
+        g.step(2, 0.12, pkg.Spacing(pkg.THIS_WORK))
+        return g.walkers()
+
+    want = project(pkg.LrdmcSystem(_system()))
+    g = pkg.LrdmcSystem(_system())
+    for _ in range(2):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            got = project(g)
+        for key in want:
+            assert np.array_equal(np.asarray(got[key]), np.asarray(want[key])), key
