@@ -145,39 +145,11 @@ static __device__ void rotation_matrix(double u1, double u2, double u3, double* 
 // The same rotation from the three uniforms of bits[0..2], with the work
 // spread over the warp: lanes 0-3 evaluate sqrt(1-u1), sqrt(u1),
 // sincospi(2 u2) and sincospi(2 u3), lanes 0-8 then form one entry of R
-// each. FP64 mode: IEEE double (the same operations as rotation_matrix).
-// FP32 mode: single precision. (The double-float mode: rotation64.) All
-// lanes must call it; R (double) goes to shared memory.
-template <int PREC>
-__device__ LRDMC_JUMP_INLINE void rotation_matrix_warp(const uint64_t* bits, double* R, int lane, const SysDev& S)
+// each. IEEE double (the same operations as rotation_matrix), for the FP64
+// mode; the others draw ahead. All lanes must call it; R goes to shared memory.
+__device__ LRDMC_JUMP_INLINE void rotation_matrix_warp(const uint64_t* bits, double* R, int lane)
 {
   double x, y, z, w;
-  if (PREC == LRDMC_PRECISION_FP32) {
-    float a = 0.0f, c = 0.0f;
-    if (lane == 0) a = sqrtf(1.0f - f_u01(bits[0]));
-    else if (lane == 1) a = sqrtf(f_u01(bits[0]));
-    else if (lane == 2) sincospif(2.0f * f_u01(bits[1]), &a, &c);
-    else if (lane == 3) sincospif(2.0f * f_u01(bits[2]), &a, &c);
-    float s1 = __shfl_sync(FULL_MASK, a, 0), s2 = __shfl_sync(FULL_MASK, a, 1);
-    float sa = __shfl_sync(FULL_MASK, a, 2), ca = __shfl_sync(FULL_MASK, c, 2);
-    float sb = __shfl_sync(FULL_MASK, a, 3), cb = __shfl_sync(FULL_MASK, c, 3);
-    float qx = s1 * sa, qy = s1 * ca, qz = s2 * sb, qw = s2 * cb;
-    float v = 0.0f;
-    switch (lane) {
-      case 0: v = 1.0f - 2.0f * (qy * qy + qz * qz); break;
-      case 1: v = 2.0f * (qx * qy - qz * qw); break;
-      case 2: v = 2.0f * (qx * qz + qy * qw); break;
-      case 3: v = 2.0f * (qx * qy + qz * qw); break;
-      case 4: v = 1.0f - 2.0f * (qx * qx + qz * qz); break;
-      case 5: v = 2.0f * (qy * qz - qx * qw); break;
-      case 6: v = 2.0f * (qx * qz - qy * qw); break;
-      case 7: v = 2.0f * (qy * qz + qx * qw); break;
-      case 8: v = 1.0f - 2.0f * (qx * qx + qy * qy); break;
-      default: break;
-    }
-    if (lane < 9) R[lane] = (double)v;
-    return;
-  }
   {
     double a = 0.0, c = 0.0;
     const double u1 = to_u01(bits[0]);
@@ -1561,25 +1533,16 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       const df bdf = st.bdf;
       bool over = st.finish != 0;
       double t = 0.0, logw = st.logw;
-      uint64_t b0[4], b1[4];
       const int it = (int)(st.m % kDrawAhead);
+      const df* draws = reinterpret_cast<const df*>(wm.dr + it * kDrawWords);
       if (!over) {
-        if (kDf) {
-          if (it == 0) draw_ahead64(P.seed, (uint64_t)st.s, k, (uint64_t)st.m, wm.dr, lane, S, lt);
-          const df nl = reinterpret_cast<const df*>(wm.dr + it * kDrawWords)[9];
-          t = b > 0.0 ? df_to_double(dl_mul(nl, dl_norm(dl_rcp(bdf)))) : INFINITY;
-        } else {
-          // both draws of this iteration at once: even lanes compute the
-          // (waiting time, heat bath) block, odd lanes the rotation block
-          uint64_t cb[4] = {(uint64_t)st.s, k, (uint64_t)st.m, (lane & 1) ? kTagRot : kTagTimeHB};
-          philox4x64_10(cb, P.seed, 0ull);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            b0[j] = shfl_u64(cb[j], 0);
-            b1[j] = shfl_u64(cb[j], 1);
-          }
-          t = b > 0.0 ? (double)(-logf(f_u01(b0[0])) / bdf.hi) : INFINITY;
+        if (it == 0) {
+          if (kDf) draw_ahead64(P.seed, (uint64_t)st.s, k, (uint64_t)st.m, wm.dr, lane, S, lt);
+          else draw_ahead32(P.seed, (uint64_t)st.s, k, (uint64_t)st.m, wm.dr, lane);
         }
+        const df nl = draws[9];
+        if (kDf) t = b > 0.0 ? df_to_double(dl_mul(nl, dl_norm(dl_rcp(bdf)))) : INFINITY;
+        else t = b > 0.0 ? (double)(nl.hi / bdf.hi) : INFINITY;
         if (t >= tau_left) {
           logw -= tau_left * (el - P.e_trial);
           over = true;
@@ -1591,10 +1554,10 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
         // heat bath over the cached rates
         if (kDf) {
           pick = heat_bath64(reinterpret_cast<const df*>(wm.T), P_moves, lane, wm.pfx,
-                             dl_norm(dl_mul(reinterpret_cast<const df*>(wm.dr + it * kDrawWords)[10], bdf)));
+                             dl_norm(dl_mul(draws[10], bdf)));
         } else {
           int lastc;
-          warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, f_u01(b0[1]) * bdf.hi, &pick,
+          warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, draws[10].hi * bdf.hi, &pick,
                              &lastc);
           if (pick < 0) pick = lastc;
         }
@@ -1635,11 +1598,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
       }
       if (lane < 3) wm.x[3 * i + lane] = wm.sm[lane];
       __syncwarp();
-      if (kDf) {
-        if (lane < 9) wm.R[lane] = wm.dr[it * kDrawWords + lane];
-      } else {
-        rotation_matrix_warp<PR>(b1, wm.R, lane, S);
-      }
+      if (lane < 9) wm.R[lane] = wm.dr[it * kDrawWords + lane];
       __syncwarp();
       double eln;
       if (kDf) eln = prelude64<NJ, NC>(S, sC, wm, lt, lane, st.fresh ? -1 : i);
@@ -1815,7 +1774,7 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
         }
         if (lane < 3) wm.x[3 * i + lane] = pnew[lane];
         __syncwarp();
-        rotation_matrix_warp<PR>(b1, wm.R, lane, S);
+        rotation_matrix_warp(b1, wm.R, lane);
         __syncwarp();
         warp_eval_any<PR, NJ, NC>(S, sC, L, wm, lane, nullptr, b, el);
         ++jumps;
