@@ -2111,19 +2111,15 @@ __global__ void __launch_bounds__(kCombThreads) k_comb_parents(const PopDev P, c
 }
 #endif  // LRDMC_PART == 0
 
-// Stateless evaluation of configuration c (one warp): inverses from x, then
-// one evaluation of every lattice move and of the local energy. Returns
-// false, with no output written, for a singular Slater matrix. The body of
-// k_evaluate and of k_evaluate_static, which differ only in where they
-// report that.
-template <int PREC>
-__device__ __forceinline__ bool evaluate_config(const SysDev& S, const Layout& Lo, const LatDev& L, const double* sC,
-                                                int c, int lane, int wib, const double* x, const double* rot,
-                                                double* ratio, double* T, double* b_out, double* el_out)
+// The FP64 mode's stateless evaluation of configuration c (one warp):
+// inverses from x, then one evaluation of every lattice move and of the
+// local energy. Returns false, with no output written, for a singular Slater
+// matrix.
+template <bool NJ>
+__device__ __forceinline__ bool evaluate_config64(const SysDev& S, const Layout& Lo, const LatDev& L, const double* sC,
+                                                  int c, int lane, int wib, const double* x, const double* rot,
+                                                  double* ratio, double* T, double* b_out, double* el_out)
 {
-  constexpr int PR = PREC & 3;         // the arithmetic (LRDMC_PRECISION_*)
-  constexpr bool NJ = (PREC & 8) != 0;  // the neural pair term is set
-  constexpr bool NC = (PREC & 4) != 0;  // the layout has no evaluation caches
   WarpMem wm = warp_mem(Lo, S, const_cast<double*>(sC) + Lo.head + wib * Lo.smem_warp);
   for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x[(size_t)c * 3 * Lo.N + j];
   for (int j = lane; j < 9; j += 32) wm.R[j] = rot[(size_t)c * 9 + j];
@@ -2132,11 +2128,9 @@ __device__ __forceinline__ bool evaluate_config(const SysDev& S, const Layout& L
   if (!ok) return false;
   const int P = S.N * 6 * L.G;
   double b, el;
-  warp_eval_any<PR, NJ, NC>(S, const_cast<double*>(sC), L, wm, lane, ratio ? ratio + (size_t)c * P : nullptr, b, el);
+  warp_eval<NJ>(S, sC, L, wm, lane, ratio ? ratio + (size_t)c * P : nullptr, b, el);
   if (T)
-    for (int j = lane; j < P; j += 32)
-      T[(size_t)c * P + j] = (PR != LRDMC_PRECISION_FP64) ? df_to_double(reinterpret_cast<const df*>(wm.T)[j])
-                                                            : wm.T[j];
+    for (int j = lane; j < P; j += 32) T[(size_t)c * P + j] = wm.T[j];
   if (lane == 0) {
     if (b_out) b_out[c] = b;
     if (el_out) el_out[c] = el;
@@ -2144,21 +2138,94 @@ __device__ __forceinline__ bool evaluate_config(const SysDev& S, const Layout& L
   return true;
 }
 
-// Stateless evaluation of given configurations (one warp per configuration).
+// Warps and configurations of an evaluation block, at most.
+constexpr int kMaxEvalWarps = 8, kMaxEvalConfigs = 8;
+
+// The stateless evaluations of a block: r configurations, one warp each for
+// the inverses, the local energy and the Jastrow sums, then every warp of the
+// block takes chunks of all their moves. Bound, like the projection, by the
+// latency of dependent chains: shared memory holds 4 warps' worth of Kr
+// configurations per SM side by side, and a call with fewer configurations
+// than SMs has one each, so the moves (about half of the work) get the warps
+// that have no configuration of their own; and warps that pass through the
+// same code together share its instruction fetches. 16384 Kr: 7.10 to 4.64
+// ms; 37 H2O: 105 to 90 us. report: a singular configuration.
+template <int PREC, class Report>
+__device__ __forceinline__ void evaluate_block(const SysDev& S, const Layout& Lo, const LatDev& L, double* sC, int n,
+                                               int r, const double* x, const double* rot, double* ratio, double* T,
+                                               double* b_out, double* el_out, Report report)
+{
+  constexpr int PR = PREC & 3;         // the arithmetic (LRDMC_PRECISION_*)
+  constexpr bool NJ = (PREC & 8) != 0;  // the neural pair term is set
+  constexpr bool NC = (PREC & 4) != 0;  // the layout has no evaluation caches
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int c = blockIdx.x * r + wib;
+  if constexpr (PR == LRDMC_PRECISION_FP64) {
+    if (wib < r && c < n && !evaluate_config64<NJ>(S, Lo, L, sC, c, lane, wib, x, rot, ratio, T, b_out, el_out) &&
+        lane == 0)
+      report();
+  } else {
+    __shared__ int s_ok[kMaxEvalConfigs];
+    const Lean lt = lean_mem(S, sC);
+    const int P = S.N * 6 * L.G, units = PR == LRDMC_PRECISION_DF64 ? P / 2 : P;
+    double el = 0.0;
+    bool ok = false;
+    if (wib < r) {
+      if (c < n) {
+        const WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
+        for (int j = lane; j < 3 * Lo.N; j += 32) wm.x[j] = x[(size_t)c * 3 * Lo.N + j];
+        for (int j = lane; j < 9; j += 32) wm.R[j] = rot[(size_t)c * 9 + j];
+        __syncwarp();
+        ok = warp_inverses(S, sC, wm.x, wm.A, wm.scr, lane);
+        if (!ok && lane == 0) report();
+        if (ok) {
+          if (PR == LRDMC_PRECISION_DF64) el = prelude64<NJ, NC>(S, sC, wm, lt, lane, -1);
+          else el = prelude32<NJ>(S, sC, wm, lt, lane, -1);
+        }
+      }
+      if (lane == 0) s_ok[wib] = ok;
+    }
+    __syncthreads();
+    // chunks of 32 units, of 16 where whole ones would leave warps idle
+    const int nw = blockDim.x >> 5, cs = r * ((units + 31) / 32) < nw ? 16 : 32, nch = (units + cs - 1) / cs;
+#pragma unroll 1
+    for (int ch = wib; ch < r * nch; ch += nw) {
+      const int q = ch / nch, u = (ch - q * nch) * cs + lane, cq = blockIdx.x * r + q;
+      if (!s_ok[q] || lane >= cs || u >= units) continue;
+      const WarpMem wm = warp_mem(Lo, S, sC + Lo.head + q * Lo.smem_warp);
+      df* Td = reinterpret_cast<df*>(wm.T);
+      double* ro = ratio ? ratio + (size_t)cq * P : nullptr;
+      if (PR == LRDMC_PRECISION_DF64) moves64<NJ, NC>(S, L, wm, lt, u, Td, ro, nullptr);
+      else candidate_m<float, NJ>(S, L, wm, block_mem(S, sC), u, Td, ro);
+    }
+    __syncthreads();
+    if (ok) {
+      const WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
+      const df* Td = reinterpret_cast<const df*>(wm.T);
+      const double b = PR == LRDMC_PRECISION_DF64
+                           ? df_to_double(rate_scan64(Td, P, lane, wm.pfx))
+                           : (double)warp_scan_m<float>(Td, P, lane, 0.0f, nullptr, nullptr);
+      if (T)
+        for (int j = lane; j < P; j += 32) T[(size_t)c * P + j] = df_to_double(Td[j]);
+      if (lane == 0) {
+        if (b_out) b_out[c] = b;
+        if (el_out) el_out[c] = el;
+      }
+    }
+  }
+}
+
+// Stateless evaluation of given configurations.
 template <int PREC>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-k_evaluate(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n,
+__global__ void __launch_bounds__(kMaxEvalWarps * 32, 2)
+k_evaluate(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n, int r,
            const double* x, const double* rot, double* ratio, double* T, double* b_out,
            double* el_out, int* err)
 {
   extern __shared__ __align__(16) double smem[];
   double* sC = smem;
   stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int c = blockIdx.x * kWarpsPerBlock + wib;
-  if (c >= n) return;
-  if (!evaluate_config<PREC>(S, Lo, L, sC, c, lane, wib, x, rot, ratio, T, b_out, el_out) && lane == 0)
-    atomicOr(err, kErrSingular);
+  evaluate_block<PREC>(S, Lo, L, sC, n, r, x, rot, ratio, T, b_out, el_out, [&] { atomicOr(err, kErrSingular); });
 }
 
 // ----------------------------------------------------------------------------
@@ -2494,36 +2561,59 @@ cudaError_t launch_interval_t(const SysDev& S, const Layout& Lo, const LatDev& L
   return cudaLaunchKernelEx(&cfg, k_interval<PREC>, S, Lo, L, P);
 }
 
+// Configurations r and warps of an evaluation block. Four and four where three
+// such blocks fit an SM. A larger system gets as many as let two blocks of
+// eight warps share an SM (one's inverses and local energies run beside the
+// other's moves). Fewer configurations than fill the SMs are spread over
+// them.
+struct EvalShape {
+  int r, warps;
+};
+
+template <int PREC>
+static EvalShape eval_shape(const Layout& Lo, int n)
+{
+  EvalShape e = {kWarpsPerBlock, kWarpsPerBlock};
+  if ((PREC & 3) == LRDMC_PRECISION_FP64) return e;
+  const int sm = 228 * 1024, reserved = 1024 + 64;  // of an SM; the runtime's and the static part of a block
+  if (3 * (Lo.smem_block_bytes + reserved) > sm) {
+    e.warps = kMaxEvalWarps;
+    int r = std::min(kMaxEvalConfigs, (int)((sm / 2 - reserved) / sizeof(double) - Lo.head) / Lo.smem_warp);
+    if (r >= 2) e.r = r;
+  }
+  const int per_sm = std::max(1, (n + sm_count_current() - 1) / sm_count_current());
+  if (per_sm < e.r) e = {per_sm, kMaxEvalWarps};
+  return e;
+}
+
 template <int PREC>
 cudaError_t launch_evaluate_t(const SysDev& S, const Layout& Lo, const LatDev& L, int n, const double* x,
                                      const double* rot, double* ratio, double* T, double* b, double* el, int* err,
                                      cudaStream_t st)
 {
-  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  cudaError_t e = set_smem((const void*)k_evaluate<PREC>, Lo.smem_block_bytes);
+  const EvalShape sh = eval_shape<PREC>(Lo, n);
+  const int blocks = (n + sh.r - 1) / sh.r, smem = interval_smem(Lo, sh.r);
+  // the largest size always: calls of other sizes may run in other threads
+  cudaError_t e = set_smem((const void*)k_evaluate<PREC>, kMaxSmemBlock);
   if (e != cudaSuccess) return e;
-  k_evaluate<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio, T, b, el,
-                                                                            err);
+  k_evaluate<PREC><<<blocks, sh.warps * 32, smem, st>>>(S, Lo, L, n, sh.r, x, rot, ratio, T, b, el, err);
   return cudaGetLastError();
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-k_evaluate_static(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n,
+__global__ void __launch_bounds__(kMaxEvalWarps * 32, 2)
+k_evaluate_static(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, int n, int r,
                   const double* x, const double* rot, double* ratio, double* T, double* b_out,
                   double* el_out, int* scratch)
 {
   extern __shared__ __align__(16) double smem[];
   double* sC = smem;
   stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int c = blockIdx.x * kWarpsPerBlock + wib;
-  if (c >= n) return;
   // word 64 + c: status of configuration c; word 0: OR of all statuses
-  if (!evaluate_config<PREC>(S, Lo, L, sC, c, lane, wib, x, rot, ratio, T, b_out, el_out) && lane == 0) {
-    scratch[64 + c] = kErrSingular;
+  evaluate_block<PREC>(S, Lo, L, sC, n, r, x, rot, ratio, T, b_out, el_out, [&] {
+    scratch[64 + blockIdx.x * r + (threadIdx.x >> 5)] = kErrSingular;
     atomicOr(&scratch[0], kErrSingular);
-  }
+  });
 }
 
 template <int PREC>
@@ -2531,12 +2621,13 @@ cudaError_t launch_evaluate_static_t(const SysDev& S, const Layout& Lo, const La
                                      const double* rot, double* ratio, double* T, double* b, double* el,
                                      int* scratch, cudaStream_t st)
 {
-  const int blocks = (n + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  cudaError_t e = set_smem((const void*)k_evaluate_static<PREC>, Lo.smem_block_bytes);
+  const EvalShape sh = eval_shape<PREC>(Lo, n);
+  const int blocks = (n + sh.r - 1) / sh.r, smem = interval_smem(Lo, sh.r);
+  // the largest size always: calls of other sizes may run in other threads
+  cudaError_t e = set_smem((const void*)k_evaluate_static<PREC>, kMaxSmemBlock);
   if (e != cudaSuccess) return e;
   if (blocks > 0)
-    k_evaluate_static<PREC><<<blocks, kWarpsPerBlock * 32, Lo.smem_block_bytes, st>>>(S, Lo, L, n, x, rot, ratio, T,
-                                                                                     b, el, scratch);
+    k_evaluate_static<PREC><<<blocks, sh.warps * 32, smem, st>>>(S, Lo, L, n, sh.r, x, rot, ratio, T, b, el, scratch);
   return cudaGetLastError();
 }
 
