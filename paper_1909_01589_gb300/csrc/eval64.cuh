@@ -442,7 +442,7 @@ __device__ __forceinline__ double prelude64(const SysDev& S, const double* sC, c
       const int i = q / S.n_nuc, I = q - i * S.n_nuc;
       dl d[3], D;
       en_geometry(S, wm, i, I, d, D);
-      df* e = &wm.enc[8 * q];
+      df* e = &wm.enc[kEncWords * q];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         e[k] = d[k];
@@ -586,7 +586,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
         en_geometry(S, wm, i, I, d, D);
         hp = dl_mul(h, axis_dot(wm, k, d));
       } else {
-        const df* e = &wm.enc[8 * (i * S.n_nuc + I)];
+        const df* e = &wm.enc[kEncWords * (i * S.n_nuc + I)];
 #pragma unroll
         for (int q = 0; q < 3; ++q) d[q] = e[q];
         D = e[3];

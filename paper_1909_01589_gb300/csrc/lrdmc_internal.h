@@ -24,6 +24,9 @@ constexpr int kMaxItersPerInterval = 1 << 20;
 // once, and the doubles each takes (rotation, waiting time, heat bath).
 constexpr int kDrawAhead = 16;
 constexpr int kDrawWords = 11;
+// An electron and nucleus in the evaluation's cache: d, D, d on the axes (an
+// eighth word would cost Kr one of its eight warps per SM).
+constexpr int kEncWords = 7;
 
 // Error bits of the device error word.
 constexpr int kErrSingular = 1;

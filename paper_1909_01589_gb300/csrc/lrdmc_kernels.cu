@@ -468,7 +468,7 @@ struct WarpMem {
   df* y;        // [N][3]      double-float mode: positions on the rotated axes, scaled
   df* Rd;       // [12]
   df* pfx;      // [32]        double-float mode: running sums of the rates
-  df* enc;      // [N][n_nuc][8] electron-nucleus cache: d, |d|^2, e_k . d
+  df* enc;      // [N][n_nuc][7] electron-nucleus cache: d, |d|^2, e_k . d
   df* pc;       // [n_pc] squared distances of the electron pairs, scaled
   double* scr;
   int n_pc;     // pairs in the cache (0: no cache)
@@ -497,7 +497,7 @@ __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, d
   m.Rd = m.y + 3 * Lo.N;
   m.pfx = m.Rd + 12;
   m.enc = m.pfx + 32;
-  m.pc = m.enc + (Lo.enc ? 8 * Lo.N * S.n_nuc : 0);
+  m.pc = m.enc + (Lo.enc ? kEncWords * Lo.N * S.n_nuc : 0);
   m.n_pc = Lo.n_pc;
   return m;
 }
@@ -1352,12 +1352,10 @@ __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, 
                                               const Lean& lt, TeamSlot* t, int units, int lane, const float4* gt)
 {
   df* Td = reinterpret_cast<df*>(wm.T);
-  // chunks of 16 moves in a team (more helpers take part in a small
-  // system's moves; measured 3 % faster than 32 on the bench workload)
-#ifndef LRDMC_TEAM_CHUNK
-#define LRDMC_TEAM_CHUNK 16
-#endif
-  const int cs = t ? LRDMC_TEAM_CHUNK : 32;
+  // in a team chunks of 16 where whole ones would not go round: 3 % faster
+  // than 32 for Ne (60 units); 32 for Kr (216), 40.5 ms to 39.3 for 4096
+  // walkers, since a half chunk costs as many issue slots as a whole one
+  const int cs = t && units <= 32 * ((ld_vol(&t->pub) & 15) + 1) ? 16 : 32;
 #pragma unroll 1
   for (int c0 = 0;; c0 += 32) {
     if (t) {
@@ -2404,12 +2402,12 @@ Layout make_layout(const SysDev& S, bool caches)
   Lo.n_scr = n * n + S.N * S.n_ao + n + (n + 1) / 2;         // inverses: basis values, matrix, pivot column, order
   Lo.n_scr = std::max(Lo.n_scr, S.n_ao + 3 * n + n * n);     // Sherman-Morrison (FP64 or FP32 mode)
   // The caches of the double-float evaluation (omitted when caches is false):
-  // the electron-nucleus cache (8 df per electron and nucleus), and one
+  // the electron-nucleus cache (7 df per electron and nucleus), and one
   // squared distance per electron pair; up to 40 electrons (beyond, they
   // would cost warps per SM)
   Lo.n_pc = (caches && S.N <= 40) ? S.N * (S.N - 1) / 2 : 0;
   Lo.enc = caches && S.N <= 40 ? 1 : 0;
-  const int state = S.N * S.n_ao + 2 * S.N + 6 * S.N + 12 + 32 + (Lo.enc ? 8 * S.N * S.n_nuc : 0) + Lo.n_pc;
+  const int state = S.N * S.n_ao + 2 * S.N + 6 * S.N + 12 + 32 + (Lo.enc ? kEncWords * S.N * S.n_nuc : 0) + Lo.n_pc;
   Lo.smem_warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + Lo.P_max + Lo.n_draw + 4 + S.n_ao + 3 * n +
                  std::max(Lo.n_scr, state);
   Lo.smem_warp = (Lo.smem_warp + 1) & ~1;
