@@ -34,6 +34,7 @@
 
 #include "lrdmc_internal.h"
 #include "mixed_arith.cuh"
+#include "lean64.cuh"
 
 // This file is compiled several times, so that the kernel variants build in
 // parallel: part 0 holds the kernels without variants and every host entry,
@@ -290,61 +291,69 @@ __device__ __forceinline__ int solid(int l, const double d[3], double S[5], doub
   return 5;
 }
 
-// Sum_mu v[mu] chi_mu(p): the determinant ratio when v is the projected
-// inverse column of the moving electron.
-static __device__ double ao_dot(const SysDev& S, const double* v, double px, double py, double pz)
+// A float's value as a double, in integer operations (a conversion holds the
+// FP64 pipe for 64 cycles); a zero or a denormal becomes about 1e-38.
+__device__ __forceinline__ double widen(float f)
 {
-  double acc = 0.0;
-  int prev_c = -1;
-  double d[3] = {0, 0, 0}, r = 0.0, e = 0.0;
-  for (int q = 0; q < S.n_shell; ++q) {
-    const ShellDev& sh = S.sh[q];
-    if (sh.center != prev_c) {
-      prev_c = sh.center;
-      d[0] = px - S.nuc[prev_c][0];
-      d[1] = py - S.nuc[prev_c][1];
-      d[2] = pz - S.nuc[prev_c][2];
-      r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    }
-    if (sh.kind == 0 && !sh.same_exp) e = exp(-sh.zeta * r);
-    double R, R1, R2, Sv[5], gS[5][3];
-    radial(sh, r, e, R, R1, R2, false);
-    int nf = solid(sh.l, d, Sv, gS, false);
-    double part = 0.0;
-    for (int f = 0; f < nf; ++f) part += v[sh.ao_offset + f] * Sv[f];
-    acc += part * R;
-  }
-  return acc;
+  const unsigned u = __float_as_uint(f);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
 
-// Sum_mu v[mu] chi_mu, grad chi_mu, lap chi_mu at p.
-static __device__ void ao_dot_der(const SysDev& S, const double* v, const double* p, double& val,
-                           double g[3], double& lap)
+// sqrt(x) in three operations of the FP64 pipe, which takes 64 cycles for
+// each, against about nine: Karp and Markstein's iteration (ACM TOMS 23
+// (1997)) in double-float on the FP32 pipe (to 2^-45), the last step in
+// double. Outside [2^-95, 2^80] (and for zero, NaN) CUDA's.
+__device__ __forceinline__ double sqrt64(double x)
 {
-  val = 0.0; g[0] = g[1] = g[2] = 0.0; lap = 0.0;
+  const unsigned h = (unsigned)__double2hiint(x);
+  if (h - 0x3a000000u >= 0x0af00000u) return sqrt(x);
+  const df a = dl_from_double(x);
+  const float y = rsqrt_ftz(a.hi), s = __fmul_rn(a.hi, y), hy = __fmul_rn(0.5f, y);
+  const float ds = __fmul_rn(__fadd_rn(__fmaf_rn(-s, s, a.hi), a.lo), hy);
+  const double g = widen(s) + widen(ds);
+  return fma(fma(-g, g, x), widen(hy), g);
+}
+
+// Shells [q0, q1) of the basis at d = p - R_centre of electron position p:
+// v . chi, and with der its gradient and Laplacian, added to the sums.
+template <bool DER>
+__device__ __forceinline__ void ao_dot(const SysDev& S, const double* v, const double* p, int q0, int q1, double& val,
+                                       double g[3], double& lap)
+{
   int prev_c = -1;
   double d[3] = {0, 0, 0}, r = 0.0, e = 0.0;
-  for (int q = 0; q < S.n_shell; ++q) {
+#pragma unroll 1
+  for (int q = q0; q < q1; ++q) {
     const ShellDev& sh = S.sh[q];
     if (sh.center != prev_c) {
       prev_c = sh.center;
-      d[0] = p[0] - S.nuc[prev_c][0];
-      d[1] = p[1] - S.nuc[prev_c][1];
-      d[2] = p[2] - S.nuc[prev_c][2];
-      r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    }
-    if (sh.kind == 0 && !sh.same_exp) e = exp(-sh.zeta * r);
-    double R, R1, R2, Sv[5], gS[5][3];
-    radial(sh, r, e, R, R1, R2, true);
-    int nf = solid(sh.l, d, Sv, gS, true);
-    double radlap = R2 + 2.0 * (sh.l + 1) * R1;
-    for (int f = 0; f < nf; ++f) {
-      double c = v[sh.ao_offset + f];
-      val += c * Sv[f] * R;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) g[k] += c * (R * gS[f][k] + Sv[f] * R1 * d[k]);
-      lap += c * Sv[f] * radlap;
+      for (int k = 0; k < 3; ++k) d[k] = p[k] - S.nuc[prev_c][k];
+      r = sqrt64(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
     }
+    if (sh.kind == 0 && (q == q0 || !sh.same_exp)) e = exp(-sh.zeta * r);
+    double R, R1, R2, Sv[5], gS[5][3];
+    radial(sh, r, e, R, R1, R2, DER);
+    const int nf = solid(sh.l, d, Sv, gS, DER);
+    if (!DER) {
+      double part = 0.0;
+      for (int f = 0; f < nf; ++f) part += v[sh.ao_offset + f] * Sv[f];
+      val += part * R;
+      continue;
+    }
+    // with P = sum_f v_f S_f: grad = R grad P + (R'/r) P d
+    double P = 0.0;
+    for (int f = 0; f < nf; ++f) {
+      const double c = v[sh.ao_offset + f], cR = c * R;
+      P += c * Sv[f];
+      if (sh.l > 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) g[k] += cR * gS[f][k];
+    }
+    const double W = P * R1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) g[k] += W * d[k];
+    lap += P * (R2 + 2.0 * (sh.l + 1) * R1);
   }
 }
 
@@ -353,7 +362,7 @@ static __device__ void shell_values(const SysDev& S, int q, const double* p, dou
 {
   const ShellDev& sh = S.sh[q];
   const double d[3] = {p[0] - S.nuc[sh.center][0], p[1] - S.nuc[sh.center][1], p[2] - S.nuc[sh.center][2]};
-  const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+  const double r = sqrt64(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
   const double e = sh.kind == 0 ? exp(-sh.zeta * r) : 0.0;
   double R, R1, R2, Sv[5], gS[5][3];
   radial(sh, r, e, R, R1, R2, false);
@@ -405,45 +414,6 @@ __device__ __forceinline__ void nj_value3(const SysDev& S, int c, double r, doub
   const double d2 = 2.0 * c2 + t * (6.0 * c3 + t * (12.0 * c4 + t * 20.0 * c5));
   g1 = d1 * iw;
   g2 = d2 * iw * iw;
-}
-
-// sum_{j != i} u_ee(|p - r_j|) + sum_I u_en(|p - R_I|).
-template <bool NJ>
-__device__ double jastrow_terms(const SysDev& S, const double* sx, int i, double px, double py,
-                                double pz)
-{
-  double acc = 0.0;
-  const int si = spin_of(S, i);
-  for (int j = 0; j < S.N; ++j) {
-    if (j == i) continue;
-    double dx = px - sx[3 * j], dy = py - sx[3 * j + 1], dz = pz - sx[3 * j + 2];
-    double r = sqrt(dx * dx + dy * dy + dz * dz);
-    double c = (spin_of(S, j) == si) ? S.c_par : S.c_anti;
-    acc += c * r / (1.0 + S.b_ee * r);
-    if (NJ) acc += nj_value(S, nj_ch_ee(S, i, j), r);
-  }
-  for (int I = 0; I < S.n_nuc; ++I) {
-    double dx = px - S.nuc[I][0], dy = py - S.nuc[I][1], dz = pz - S.nuc[I][2];
-    double r = sqrt(dx * dx + dy * dy + dz * dz);
-    acc -= S.en_b1[I] * r / (1.0 + S.en_b2 * r);
-    if (NJ) acc += nj_value(S, 2 + S.nj_species[I], r);
-  }
-  return acc;
-}
-
-// p at a point: nearest heavy nucleus, Eq. 3 (Gaussian) or Eq. 2 (Pade).
-__device__ __forceinline__ double p_weight(const SysDev& S, const LatDev& L, double px, double py,
-                                           double pz)
-{
-  double best = INFINITY;
-  for (int I = 0; I < S.n_nuc; ++I) {
-    if (!S.heavy[I]) continue;
-    double dx = px - S.nuc[I][0], dy = py - S.nuc[I][1], dz = pz - S.nuc[I][2];
-    double d2 = dx * dx + dy * dy + dz * dz;
-    best = fmin(best, d2);
-  }
-  if (L.pkind == 0) return exp(-best * L.p_coef);
-  return 1.0 / (1.0 + L.p_coef * best);
 }
 
 // ----------------------------------------------------------------------------
@@ -683,104 +653,239 @@ static __device__ LRDMC_COLD bool warp_inverses(const SysDev& S, const double* s
 // (Eq. 1 lattice, fixed-node rates) and of its continuous local energy.
 // On return sT holds T_c, b and el are warp-uniform. ratio_out (global,
 // nullable) receives psi_G(x')/psi_G(x) for every move.
+//
+// Bound by the FP64 pipe: an instruction holds it for 64 cycles whatever its
+// lane count. So the local energy is dealt to all lanes (el_L parts per
+// electron, combined by shuffles), a lane evaluates the two moves +-h e_k
+// from D + h^2 +- 2 h (y_ik - y_jk) as the double-float evaluation does
+// (eval64.cuh), square roots take three operations of that pipe, and the e-e
+// Pade sum is one running fraction, c r/(1 + b r) = c/b - (c/b)/(1 + b r),
+// whose constant cancels (three operations per partner instead of nine; for b
+// below 1/4, where that form would lose digits, term by term). Ne, 1021
+// walkers, 4 intervals: 10.34 ms to 7.37.
 // ----------------------------------------------------------------------------
+// den's power of two out of num/den (exact)
+__device__ __forceinline__ void pow2_rescale64(double& num, double& den)
+{
+  const int e = (__double2hiint(den) >> 20) & 0x7ff;
+  const double s = __hiloint2double((2046 - min(e, 2045)) << 20, 0);
+  num *= s;
+  den *= s;
+}
+
 template <bool NJ>
 __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, const WarpMem& wm,
                           int lane, double* ratio_out, double& b, double& el, double* grad_out = nullptr,
                           bool moves = true)
 {
-  const int N = S.N, nao = S.n_ao, nu = S.n_up;
+  const int N = S.N, nao = S.n_ao, nu = S.n_up, E = S.el_E, Lp = S.el_L;
   const BlockMem bm = block_mem(S, const_cast<double*>(sC));
+  double* see_i = wm.Ssum;                               // [N] e-e sums: of c q, or c r q (below b = 1/4)
+  double* sen_i = reinterpret_cast<double*>(wm.Sn);      // [N] e-n sums and the neural terms
+  double* y = reinterpret_cast<double*>(wm.y);           // [N][3] positions on the rotated axes
+  const bool recip = S.ee_recip != 0;
   // projected inverse columns: v[i][mu] = sum_m C[mu][m] Ainv_sigma[m][l_i]
+#pragma unroll 1
   for (int idx = lane; idx < N * nao; idx += 32) {
     int i = idx / nao, mu = idx % nao;
     int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
     const double* A = spin ? wm.A + nu * nu : wm.A;
     wm.v[idx] = project_ao(S, bm, A, mu, l, n);
   }
-  __syncwarp();
-  // local energy: lanes over electrons
-  double part = 0.0;
-  for (int i = lane; i < N; i += 32) {
-    const double* ri = &wm.x[3 * i];
-    double val, gD[3], lD;
-    ao_dot_der(S, &wm.v[i * nao], ri, val, gD, lD);
-    double gJ[3] = {0.0, 0.0, 0.0}, lJ = 0.0, Ssum = 0.0, V = 0.0;
-    const int si = spin_of(S, i);
-    for (int j = 0; j < N; ++j) {
-      if (j == i) continue;
-      double d0 = ri[0] - wm.x[3 * j], d1 = ri[1] - wm.x[3 * j + 1], d2 = ri[2] - wm.x[3 * j + 2];
-      double r = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-      double c = (spin_of(S, j) == si) ? S.c_par : S.c_anti;
-      double inv = 1.0 / (1.0 + S.b_ee * r);
-      double u1 = c * inv * inv;
-      double u2 = -2.0 * S.b_ee * c * inv * inv * inv;
-      double ir = 1.0 / r;
-      Ssum += c * r * inv;
-      if (NJ) {
-        double g, g1, g2;
-        nj_value3(S, nj_ch_ee(S, i, j), r, g, g1, g2);
-        u1 += g1; u2 += g2; Ssum += g;
-      }
-      gJ[0] += u1 * d0 * ir; gJ[1] += u1 * d1 * ir; gJ[2] += u1 * d2 * ir;
-      lJ += u2 + 2.0 * u1 * ir;
-      if (j > i && S.ee_on) V += ir;
-    }
-    for (int I = 0; I < S.n_nuc; ++I) {
-      double d0 = ri[0] - S.nuc[I][0], d1 = ri[1] - S.nuc[I][1], d2 = ri[2] - S.nuc[I][2];
-      double r = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-      double b1 = S.en_b1[I];
-      double inv = 1.0 / (1.0 + S.en_b2 * r);
-      double u1 = -b1 * inv * inv;
-      double u2 = 2.0 * S.en_b2 * b1 * inv * inv * inv;
-      double ir = 1.0 / r;
-      Ssum -= b1 * r * inv;
-      if (NJ) {
-        double g, g1, g2;
-        nj_value3(S, 2 + S.nj_species[I], r, g, g1, g2);
-        u1 += g1; u2 += g2; Ssum += g;
-      }
-      gJ[0] += u1 * d0 * ir; gJ[1] += u1 * d1 * ir; gJ[2] += u1 * d2 * ir;
-      lJ += u2 + 2.0 * u1 * ir;
-      V -= S.Z[I] * ir;
-    }
-    wm.Ssum[i] = Ssum;
-    if (grad_out)
-      for (int k = 0; k < 3; ++k) grad_out[3 * i + k] = gD[k] + gJ[k];
-    double lap = lD + 2.0 * (gD[0] * gJ[0] + gD[1] * gJ[1] + gD[2] * gJ[2]) + lJ +
-                 gJ[0] * gJ[0] + gJ[1] * gJ[1] + gJ[2] * gJ[2];
-    part += -0.5 * lap + V;
+#pragma unroll 1
+  for (int j = lane; moves && j < 3 * N; j += 32) {
+    const int i = j / 3, k = j - 3 * i;
+    y[j] = wm.R[k] * wm.x[3 * i] + wm.R[3 + k] * wm.x[3 * i + 1] + wm.R[6 + k] * wm.x[3 * i + 2];
   }
-  el = warp_sum(part) + S.V_nn;
+  __syncwarp();
+  // local energy: E electrons at a time, Lp lanes (parts) each
+  double total = 0.0;
+  const int part = lane / E;
+#pragma unroll 1
+  for (int i0 = 0; i0 < N; i0 += E) {
+    const int i = i0 + lane - part * E;
+    const bool act = part < Lp && i < N;
+    double gD[3] = {0.0, 0.0, 0.0}, gJ[3] = {0.0, 0.0, 0.0}, see = 0.0, sen = 0.0;
+    if (act) {
+      const double* ri = &wm.x[3 * i];
+      double val = 0.0, lap = 0.0, V = 0.0;
+#pragma unroll 1
+      for (int gi = part; gi < S.n_grp64; gi += Lp)
+        ao_dot<true>(S, &wm.v[i * nao], ri, S.grp64_first[gi], S.grp64_first[gi + 1], val, gD, lap);
+      const int si = spin_of(S, i);
+#pragma unroll 1
+      for (int t = part; t < N - 1; t += Lp) {
+        const int j = t < i ? t : t + 1;
+        const double d0 = ri[0] - wm.x[3 * j], d1 = ri[1] - wm.x[3 * j + 1], d2 = ri[2] - wm.x[3 * j + 2];
+        const double r = sqrt64(d0 * d0 + d1 * d1 + d2 * d2);
+        const double c = (spin_of(S, j) == si) ? S.c_par : S.c_anti;
+        // 1/(1 + b r) and 1/r from one division
+        const double u = fma(S.b_ee, r, 1.0), w = 1.0 / (r * u), inv = w * r, ir = w * u;
+        const double cq = c * inv;
+        see += recip ? cq : cq * r;
+        double u1 = cq * inv, u2 = -2.0 * S.b_ee * u1 * inv;
+        if (NJ) {
+          double g, g1, g2;
+          nj_value3(S, nj_ch_ee(S, i, j), r, g, g1, g2);
+          u1 += g1; u2 += g2; sen += g;
+        }
+        const double a = u1 * ir;
+        gJ[0] += a * d0; gJ[1] += a * d1; gJ[2] += a * d2;
+        lap += u2 + 2.0 * a;
+        if (j > i && S.ee_on) V += ir;
+      }
+#pragma unroll 1
+      for (int I = part; I < S.n_nuc; I += Lp) {
+        const double d0 = ri[0] - S.nuc[I][0], d1 = ri[1] - S.nuc[I][1], d2 = ri[2] - S.nuc[I][2];
+        const double r = sqrt64(d0 * d0 + d1 * d1 + d2 * d2);
+        const double b1 = S.en_b1[I], ir = 1.0 / r;
+        double u1 = 0.0, u2 = 0.0;
+        if (b1 != 0.0) {
+          const double inv = 1.0 / (1.0 + S.en_b2 * r);
+          u1 = -b1 * inv * inv;
+          u2 = -2.0 * S.en_b2 * u1 * inv;
+          sen -= b1 * r * inv;
+        }
+        if (NJ) {
+          double g, g1, g2;
+          nj_value3(S, 2 + S.nj_species[I], r, g, g1, g2);
+          u1 += g1; u2 += g2; sen += g;
+        }
+        const double a = u1 * ir;
+        gJ[0] += a * d0; gJ[1] += a * d1; gJ[2] += a * d2;
+        lap += u2 + 2.0 * a;
+        V -= S.Z[I] * ir;
+      }
+      total += V - 0.5 * lap;
+    }
+    // combine the parts of each electron (lane part * E + i)
+    if (Lp > 1) {
+#pragma unroll 1
+      for (int o = S.el_top; o > 0; o >>= 1) {
+        const bool take = part < o && part + o < Lp;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          double t = __shfl_down_sync(FULL_MASK, gD[k], o * E);
+          if (take) gD[k] += t;
+          t = __shfl_down_sync(FULL_MASK, gJ[k], o * E);
+          if (take) gJ[k] += t;
+        }
+        double t = __shfl_down_sync(FULL_MASK, see, o * E);
+        if (take) see += t;
+        t = __shfl_down_sync(FULL_MASK, sen, o * E);
+        if (take) sen += t;
+      }
+    }
+    if (part == 0 && act) {
+      see_i[i] = see;
+      sen_i[i] = sen;
+      double quad = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        quad += gJ[k] * (gJ[k] + 2.0 * gD[k]);
+        if (grad_out) grad_out[3 * i + k] = gD[k] + gJ[k];
+      }
+      total -= 0.5 * quad;
+    }
+  }
+  el = warp_sum(total) + S.V_nn;
   __syncwarp();
   if (!moves) {
     b = 0.0;
     return;
   }
-  // the P lattice moves: lanes over candidates
-  const int G = L.G, per_e = 6 * G, P = N * per_e;
-  for (int c = lane; c < P; c += 32) {
-    int i = c / per_e, rem = c - i * per_e, g = rem / 6, k = (rem % 6) >> 1;
-    double sign = (c & 1) ? -1.0 : 1.0;
-    double h = g ? L.ap : L.a;
-    double ex = wm.R[k], ey = wm.R[3 + k], ez = wm.R[6 + k];
+  // the moves: lanes over (electron, grid, axis), both directions each
+  const int G = L.G, units = 3 * G * N;
+#pragma unroll 1
+  for (int u = lane; u < units; u += 32) {
+    const int i = u / (3 * G), rem = u - i * 3 * G, g = rem / 3, k = rem - 3 * g;
+    const double h = g ? L.ap : L.a, h2 = h * h;
     const double* ri = &wm.x[3 * i];
-    double px = ri[0] + sign * h * ex, py = ri[1] + sign * h * ey, pz = ri[2] + sign * h * ez;
-    double rdet = ao_dot(S, &wm.v[i * nao], px, py, pz);
-    double dJ = jastrow_terms<NJ>(S, wm.x, i, px, py, pz) - wm.Ssum[i];
-    double rho = rdet * exp(dJ);
-    double w = 1.0;
-    if (G == 2) {
-      double hh = 0.5 * h;
-      double pm = p_weight(S, L, ri[0] + sign * hh * ex, ri[1] + sign * hh * ey, ri[2] + sign * hh * ez);
-      w = g ? 1.0 - pm : pm;
+    const double he[3] = {h * wm.R[k], h * wm.R[3 + k], h * wm.R[6 + k]};
+    double rdet[2], jn[2] = {0.0, 0.0}, mid[2] = {INFINITY, INFINITY};
+#pragma unroll 1
+    for (int m = 0; m < 2; ++m) {
+      const double p[3] = {m ? ri[0] - he[0] : ri[0] + he[0], m ? ri[1] - he[1] : ri[1] + he[1],
+                           m ? ri[2] - he[2] : ri[2] + he[2]};
+      double none[3], lap, acc = 0.0, jm = 0.0;
+      ao_dot<false>(S, &wm.v[i * nao], p, 0, S.n_shell, acc, none, lap);
+      if (m) rdet[1] = acc;
+      else rdet[0] = acc;
+#pragma unroll 1
+      for (int I = 0; I < S.n_nuc; ++I) {
+        if (!NJ && S.en_b1[I] == 0.0) continue;
+        const double d0 = p[0] - S.nuc[I][0], d1 = p[1] - S.nuc[I][1], d2 = p[2] - S.nuc[I][2];
+        const double r = sqrt64(d0 * d0 + d1 * d1 + d2 * d2);
+        if (S.en_b1[I] != 0.0) jm -= S.en_b1[I] * r / (1.0 + S.en_b2 * r);
+        if (NJ) jm += nj_value(S, 2 + S.nj_species[I], r);
+      }
+      if (m) jn[1] = jm;
+      else jn[0] = jm;
     }
-    double T = rho > 0.0 ? w * (g ? L.inv2ap2 : L.inv2a2) * rho : 0.0;
-    wm.T[c] = T;
-    if (ratio_out) ratio_out[c] = rho;
+    if (G == 2) {
+      // |d +- h e/2|^2 of the nearest heavy nucleus
+#pragma unroll 1
+      for (int I = 0; I < S.n_nuc; ++I) {
+        if (!S.heavy[I]) continue;
+        const double d0 = ri[0] - S.nuc[I][0], d1 = ri[1] - S.nuc[I][1], d2 = ri[2] - S.nuc[I][2];
+        const double q = d0 * d0 + d1 * d1 + d2 * d2 + 0.25 * h2, w = d0 * he[0] + d1 * he[1] + d2 * he[2];
+        mid[0] = fmin(mid[0], q + w);
+        mid[1] = fmin(mid[1], q - w);
+      }
+    }
+    double jee[2] = {0.0, 0.0};
+    const double hh = 2.0 * h, yi = y[3 * i + k];
+    const int si = spin_of(S, i);
+#pragma unroll 1
+    for (int sp = 0; sp < 2; ++sp) {
+      const int j0 = sp ? nu : 0, j1 = sp ? N : nu;
+      const double c = sp == si ? S.c_par : S.c_anti;
+      double num[2] = {0.0, 0.0}, den[2] = {1.0, 1.0};
+#pragma unroll 1
+      for (int j = j0; j < j1; ++j) {
+        if (j == i) continue;
+        const double d0 = ri[0] - wm.x[3 * j], d1 = ri[1] - wm.x[3 * j + 1], d2 = ri[2] - wm.x[3 * j + 2];
+        const double D = fma(d0, d0, fma(d1, d1, fma(d2, d2, h2))), p = hh * (yi - y[3 * j + k]);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          double t = m ? D - p : D + p;
+          if (t < 0.0) t = 0.0;  // a rounding residue
+          const double r = sqrt64(t), q = fma(S.b_ee, r, 1.0);
+          if (recip) {
+            num[m] = fma(num[m], q, den[m]);
+            den[m] *= q;
+          } else {
+            num[m] += r / q;
+          }
+          if (NJ) jn[m] += nj_value(S, nj_ch_ee(S, i, j), r);
+        }
+        if (recip && ((j - j0) & 15) == 15) {
+          pow2_rescale64(num[0], den[0]);
+          pow2_rescale64(num[1], den[1]);
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 2; ++m) jee[m] += c * (recip ? num[m] / den[m] : num[m]);
+    }
+    const int c0 = (i * G + g) * 6 + 2 * k;
+    const double fac = recip ? -1.0 / S.b_ee : 1.0, inv2 = g ? L.inv2ap2 : L.inv2a2;
+#pragma unroll 1
+    for (int m = 0; m < 2; ++m) {
+      const double dJ = fac * ((m ? jee[1] : jee[0]) - see_i[i]) + ((m ? jn[1] : jn[0]) - sen_i[i]);
+      const double rho = (m ? rdet[1] : rdet[0]) * exp(dJ);
+      double w = 1.0;
+      if (G == 2) {
+        const double q = L.p_coef * (m ? mid[1] : mid[0]);
+        const double pm = L.pkind == 0 ? exp(-q) : 1.0 / (1.0 + q);
+        w = g ? 1.0 - pm : pm;
+      }
+      const double T = rho > 0.0 ? w * inv2 * rho : 0.0;
+      wm.T[c0 + m] = T;
+      if (ratio_out) ratio_out[c0 + m] = rho;
+    }
   }
   __syncwarp();
-  b = warp_scan(wm.T, P, lane, 0.0, nullptr, nullptr);
+  b = warp_scan(wm.T, 6 * G * N, lane, 0.0, nullptr, nullptr);
 }
 
 // ----------------------------------------------------------------------------
