@@ -20,8 +20,8 @@ constexpr int kMaxMO = LRDMC_MAX_SPIN;
 constexpr int kMaxNjCh = LRDMC_NJ_MAX_CH;
 constexpr int kWarpsPerBlock = 4;
 constexpr int kMaxItersPerInterval = 1 << 20;
-// Iterations whose random numbers a warp of the double-float mode draws at
-// once, and the doubles each takes (rotation, waiting time, heat bath).
+// Iterations whose random numbers a warp of the double-float or mixed mode
+// draws at once, and the doubles each takes (rotation, waiting time, heat bath).
 constexpr int kDrawAhead = 16;
 constexpr int kDrawWords = 11;
 // An electron and nucleus in the evaluation's cache: d, D, d on the axes (an
@@ -122,15 +122,13 @@ struct SysDev {
   double b_ee, c_par, c_anti, en_b2;
   double V_nn;
   ShellDev sh[kMaxShell];
-  // units of consecutive shells that the parts of an electron's local
-  // energy deal out (unit g is shells [grp_first[g], grp_first[g + 1])):
+  // the parts of an electron's local energy: el_E electrons at a time with
+  // el_L lanes each (el_top: the largest power of two below el_L) deal out
+  // units of consecutive shells, unit g the shells [grp64_first[g],
+  // grp64_first[g + 1]):
   // every shell alone when there are no more shells than parts (each then
   // forms its own exponential), else groups sharing one Slater exponential
   // (a shell with same_exp joins the group of the shell before it)
-  int n_grp;
-  int grp_first[kMaxShell + 1];
-  // the same for the double-float mode, which takes el_E electrons at a time
-  // with el_L lanes each (el_top: the largest power of two below el_L)
   int el_E, el_L, el_top;
   int n_grp64;
   int grp64_first[kMaxShell + 1];

@@ -54,7 +54,6 @@ namespace lrdmc {
 // interval loop (tuning switches; the default inlines everything):
 //   LRDMC_NOINLINE_COLD  the Gauss-Jordan recompute (every few intervals)
 //   LRDMC_NOINLINE_JUMP  the Sherman-Morrison update and the new rotation
-//   LRDMC_NOINLINE_EL    the local-energy parts of an evaluation
 #ifdef LRDMC_NOINLINE_COLD
 #define LRDMC_COLD __noinline__
 #else
@@ -66,11 +65,6 @@ namespace lrdmc {
 #else
 #define LRDMC_JUMP
 #define LRDMC_JUMP_INLINE __forceinline__
-#endif
-#ifdef LRDMC_NOINLINE_EL
-#define LRDMC_EL __noinline__
-#else
-#define LRDMC_EL
 #endif
 
 // ----------------------------------------------------------------------------
@@ -424,7 +418,7 @@ struct WarpMem {
   double* A;    // inverse up [nu][nu] then down [nd][nd]
   double* R;    // [9]
   double* T;    // [P_max]
-  double* dr;   // [kDrawAhead][kDrawWords] draws made ahead (double-float mode)
+  double* dr;   // [kDrawAhead][kDrawWords] draws made ahead (double-float and mixed modes)
   double* sm;   // [4 + n_ao + 3 nu] Sherman-Morrison scratch of the double-float mode
   // the evaluation's state; scr is scratch over the same storage (the
   // inverse and the other modes' Sherman-Morrison updates, which run while
@@ -1131,15 +1125,6 @@ __device__ __forceinline__ NT p_weight_m(const SysDev& S, const LatDev& L, const
   }
   if (L.pkind == 0) return A::exp(A::neg(A::mul(best, A::c(L.p_coef_df))), S.D.exp.K, bm.tab);
   return A::rcp(A::add_f(A::mul(A::c(L.p_coef_df), best), 1.0f));
-}
-
-template <class NT>
-__device__ __forceinline__ NT warp_sum_m(NT v)
-{
-  typedef Ar<NT> A;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = A::add(v, A::shfl_xor(v, o));
-  return v;
 }
 
 // Chunked inclusive scan of the rates (as warp_scan) in NT.
