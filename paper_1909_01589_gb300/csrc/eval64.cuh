@@ -302,7 +302,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
         const int j = t < i ? t : t + 1;
         dl dd[3], D;
         D = pair_d2(S, wm, i, j, dd);
-        const dl s = dl_norm(dl_sqrt_acc(D)), is = dl_norm(dl_rcp(s));
+        const dl s = dl_norm(dl_sqrt_acc(D)), is = dl_inv_distance(D, s);
         const dl c = spin_of(S, j) == si ? S.D.c_par : S.D.c_anti;
         dl q, qs;
         if (recip) {
@@ -342,7 +342,7 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
         dl dd[3], D;
         en_geometry(S, wm, i, I, dd, D);
         const dl rr = dl_norm(dl_sqrt_acc(D));
-        const dl is = dl_norm(dl_rcp(rr));
+        const dl is = dl_inv_distance(D, rr);
         const dl b1 = S.D.en_b1[I], b2 = S.D.en_b2;
         const dl q = dl_norm(dl_rcp(dl_norm(dl_add_f(dl_mul(b2, rr), 1.0f))));
         const dl bq2 = dl_mul_n(b1, dl_norm(dl_sqr(q)));
