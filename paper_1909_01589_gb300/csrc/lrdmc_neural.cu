@@ -289,13 +289,14 @@ __device__ __forceinline__ void silu3(float z, float& a, float& d1, float& d2, f
 
 // Distance and unit vector of d = a - b (both double): in double-float
 // arithmetic, rounded to single (as the FP64 form to within its rounding;
-// FP64 instructions hold their pipe for 64 cycles each).
+// FP64 instructions hold their pipe for 64 cycles each); not a number where
+// the two coincide.
 __device__ __forceinline__ float4 unit_vector(const double* a, const double* b)
 {
   dl d[3];
   for (int k = 0; k < 3; ++k) d[k] = dl_sub_n(dl_from_double(a[k]), dl_from_double(b[k]));
-  const dl r = dl_norm(dl_sqrt_acc(dl_norm(dl_add(dl_add(dl_sqr(d[0]), dl_sqr(d[1])), dl_sqr(d[2])))));
-  const dl ir = dl_rcp(r);
+  const dl r2 = dl_norm(dl_add(dl_add(dl_sqr(d[0]), dl_sqr(d[1])), dl_sqr(d[2])));
+  const dl r = dl_norm(dl_sqrt_acc(r2)), ir = dl_inv_distance(r2, r);
   return make_float4(r.hi, dl_norm(dl_mul(d[0], ir)).hi, dl_norm(dl_mul(d[1], ir)).hi, dl_norm(dl_mul(d[2], ir)).hi);
 }
 

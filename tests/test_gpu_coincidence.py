@@ -71,3 +71,24 @@ def test_local_energy_is_not_finite(pkg, prec, name, where):
         g.step(1, 0.1, sp)
         g.energy_trace()
     assert e.value.status == pkg.ERR_NONFINITE
+
+
+@pytest.mark.parametrize("where", ["nucleus", "pair"])
+def test_training_terms_are_not_finite(pkg, where):
+    """The neural term's own gradient has no direction there: E_L is not a
+    number even with base terms that the caller gives as finite."""
+    from oracle import neural as onn
+    from paper_1909_01589_gb300 import neural
+
+    system = S.make_system("Ne")
+    spec = S.default_neural_spec(system)
+    params = S.neural_init(spec, 4, out_scale=0.5)
+    x = _positions(system, where)
+    grad, e = np.zeros((4, system.N, 3)), np.full(4, -128.0)
+    el, j = neural.NeuralJastrowTerms.apply(torch.tensor(params, device="cuda"), pkg.LrdmcSystem(system), spec,
+                                            torch.tensor(x, device="cuda"), torch.tensor(grad, device="cuda"),
+                                            torch.tensor(e, device="cuda"), False)
+    ref, refj = onn.energy_terms(params, spec, x, system.n_up, system.nuc_xyz, grad, e, bf16=False)
+    assert torch.equal(torch.isfinite(el).cpu(), torch.isfinite(ref))
+    assert list(torch.isfinite(ref)) == [True, False, True, True]
+    assert torch.isfinite(j).all() and torch.isfinite(refj).all()
