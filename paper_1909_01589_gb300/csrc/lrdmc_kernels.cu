@@ -713,8 +713,9 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
         const double d0 = ri[0] - wm.x[3 * j], d1 = ri[1] - wm.x[3 * j + 1], d2 = ri[2] - wm.x[3 * j + 2];
         const double r = sqrt64(d0 * d0 + d1 * d1 + d2 * d2);
         const double c = (spin_of(S, j) == si) ? S.c_par : S.c_anti;
-        // 1/(1 + b r) and 1/r from one division
-        const double u = fma(S.b_ee, r, 1.0), w = 1.0 / (r * u), inv = w * r, ir = w * u;
+        // 1/(1 + b r) and 1/r from one division (a pair on one point: 1 and
+        // infinity, so that its Jastrow sum, and with it the moves, stay finite)
+        const double u = fma(S.b_ee, r, 1.0), w = 1.0 / (r * u), inv = __double2hiint(r) ? w * r : 1.0, ir = w * u;
         const double cq = c * inv;
         see += recip ? cq : cq * r;
         double u1 = cq * inv, u2 = -2.0 * S.b_ee * u1 * inv;

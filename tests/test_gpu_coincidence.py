@@ -42,7 +42,7 @@ def _system(pkg, system, prec):
 
 @pytest.mark.parametrize("where", ["nucleus", "pair"])
 @pytest.mark.parametrize("name", ["He", "Ne", "H2O"])
-@pytest.mark.parametrize("prec", ["df64", "fp32"])
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
 def test_local_energy_is_not_finite(pkg, prec, name, where):
     import oracle
 
