@@ -14,12 +14,13 @@
 //     table read, and their two chains interleave;
 //   * distances come from one cached D = |r_i - r_j|^2 per pair and the
 //     positions on the rotated axes y = R^T r: |r_i +- h e_k - r_j|^2 = D +
-//     h^2 +- 2h (y_ik - y_jk). Lengths of the e-e part are scaled by b, so
-//     that the square root is b r itself;
+//     h^2 +- 2h (y_ik - y_jk). Lengths of the e-e part are scaled by b in
+//     the form below, so that the square root is b r itself;
 //   * the e-e Pade sum needs one reciprocal per partner: c r/(1 + b r) =
 //     c/b - (c/b)/(1 + b r), whose constant cancels in the Jastrow
-//     difference (for |b| below 1/4 or b <= 0, where that form would lose
-//     digits or divide by zero, the product form c r q);
+//     difference (for b below 1/4, where that form would lose digits or
+//     divide by zero, and above 2^20, where its lengths could leave the float
+//     range, the product form c r q);
 //   * after a jump only what moved is formed again: the projected columns of
 //     one spin, one electron's position and its N - 1 distances.
 #pragma once
@@ -173,7 +174,7 @@ __device__ __forceinline__ dl axis_dot(const WarpMem& wm, int k, const dl d[3])
   return dl_add_n(dl_add(dl_mul(wm.Rd[k], d[0]), dl_mul(wm.Rd[3 + k], d[1])), dl_mul(wm.Rd[6 + k], d[2]));
 }
 
-// b^2 |r_i - r_j|^2 from the positions (b: the scale of the e-e part)
+// b^2 |r_i - r_j|^2 from the positions (b: the scale of the e-e part, ee_scale)
 __device__ __forceinline__ dl pair_d2(const SysDev& S, const WarpMem& wm, int i, int j, dl d[3])
 {
 #pragma unroll
@@ -292,9 +293,9 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
           }
           lap = dl_add(lap, dl_mul(P, dl_add_n(R2, dl_mul_f(R1, 2.0f * (sh.l + 1)))));
         }
-      // e-e pairs, the N - 1 partners dealt to the parts. With s = b r,
-      // q = 1/(1 + s): u'/r = c q^2 b / s, u'' + 2 u'/r = 2 b c q^2 (1/s - q)
-      // (b: the scale; sb its sign or 0 in the general form)
+      // e-e pairs, the N - 1 partners dealt to the parts. With s = b r (r in
+      // the general form), q = 1/(1 + b r): u'/r = c q^2 / r, u'' + 2 u'/r =
+      // 2 c q^2 (1/r - b q)
       dl lap2 = zero, pot = zero, snj = zero;
       const int si = spin_of(S, i);
 #pragma unroll 1
@@ -310,9 +311,8 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
           qs = q;
           see = dl_add(see, dl_mul(c, q));
         } else {
-          const dl sb = dl_mul_f(s, S.ee_sign);
-          q = dl_rcp(dl_norm(dl_add_f(sb, 1.0f)));
-          qs = dl_mul_f(q, S.ee_sign);
+          q = dl_rcp(dl_norm(dl_add_f(dl_mul(S.D.b_ee, s), 1.0f)));
+          qs = dl_mul(S.D.b_ee, q);
           see = dl_add(see, dl_mul(c, dl_mul(s, q)));
         }
         const dl cq2 = dl_mul_n(c, dl_norm(dl_sqr(q)));
@@ -545,7 +545,7 @@ __device__ __forceinline__ dl2 radial_table2(const LShell& sh, const float4* gt,
 }
 
 // One partner of the e-e sums of the moves +-h e_k: Dh = b^2 (D + h^2), p =
-// 2 b^2 h (y_ik - y_jk)/b; acc receives q (or s q, the general form).
+// 2 b^2 h (y_ik - y_jk)/b, b the scale; acc receives q (r q in the general form).
 template <bool NJ>
 __device__ __forceinline__ void ee_partner64(const SysDev& S, dl Dh, dl p, int ch, dl2& acc, dl2& nj)
 {
@@ -554,8 +554,7 @@ __device__ __forceinline__ void ee_partner64(const SysDev& S, dl Dh, dl p, int c
     // q <= 1 <= acc: the sum starts from one
     acc = dl2_add_big(acc, dl2_rcp(dl2_one_plus(s)));
   } else {
-    const dl2 sg = dl2_make(f2_mul(s.hi, f2_all(S.ee_sign)), f2_mul(s.lo, f2_all(S.ee_sign)));
-    const dl2 q = dl2_rcp(dl2_norm(dl2_add_f(sg, f2_all(1.0f))));
+    const dl2 q = dl2_rcp(dl2_norm(dl2_add_f(dl2_mul(dl2_all(S.D.b_ee), s), f2_all(1.0f))));
     acc = dl2_add(acc, dl2_mul(s, q));
   }
   if (NJ) nj = dl2_add(nj, nj_value64_2(S, ch, dl2_mul(s, dl2_all(S.D.ee_iscale))));

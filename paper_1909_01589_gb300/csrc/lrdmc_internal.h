@@ -102,9 +102,9 @@ struct DfSys {
   df inv_fact[18];  // 1/k!, k = 0..17 (series of sin and cos)
   df half_pi;
   LeanExp lexp;
-  // e-e part of the double-float evaluation: its lengths are scaled by
-  // ee_scale = |b| (1 for b = 0); ee_factor turns the sums it compares into
-  // the Jastrow exponent (-1/b in the reciprocal form, 1/scale in the other)
+  // e-e part of the double-float evaluation: in the reciprocal form its
+  // lengths are scaled by ee_scale = b (1 in the general form); ee_factor turns
+  // the sums it compares into the Jastrow exponent (-1/b, or 1)
   df ee_scale, ee_scale2, ee_iscale, ee_factor;
 };
 
@@ -134,8 +134,7 @@ struct SysDev {
   int grp64_first[kMaxShell + 1];
   int n_prim;       // primitives of all Gaussian shells
   int gt_total;     // cells of the radial table
-  int ee_recip;     // 1: the e-e Pade sum in the reciprocal form (b >= 1/4)
-  float ee_sign;    // sign of b (0 for b = 0)
+  int ee_recip;     // 1: the e-e Pade sum in the reciprocal form (1/4 <= b <= 2^20)
   // the non-zero MO coefficients: bit m of row_mask[mu] and bit mu of
   // col_mask[m] for C[mu][m] != 0 (an atom's orbitals mix basis functions of
   // one symmetry only)

@@ -2349,14 +2349,15 @@ void fill_df_constants(SysDev& S)
     }
   }
   // e-e part: the reciprocal form needs b away from zero (its terms c/b q
-  // would lose log2(c/b) bits) and positive (1 + b r > 0)
-  const double bs = S.b_ee != 0.0 ? fabs(S.b_ee) : 1.0;
-  S.ee_recip = S.b_ee >= 0.25 ? 1 : 0;
-  S.ee_sign = S.b_ee > 0.0 ? 1.0f : (S.b_ee < 0.0 ? -1.0f : 0.0f);
+  // would lose log2(c/b) bits) and positive (1 + b r > 0), and b^2 r^2 and the
+  // FP64 mode's products of up to 31 (1 + b r) within range; the general form
+  // takes lengths as they are
+  S.ee_recip = S.b_ee >= 0.25 && S.b_ee <= 0x1p20 ? 1 : 0;
+  const double bs = S.ee_recip ? S.b_ee : 1.0;
   D.ee_scale = split_ld(bs);
   D.ee_scale2 = split_ld((long double)bs * bs);
   D.ee_iscale = split_ld(1.0L / bs);
-  D.ee_factor = split_ld((S.ee_recip ? -1.0L : 1.0L) / bs);
+  D.ee_factor = split_ld(S.ee_recip ? -1.0L / bs : 1.0L);
   // Tang's table: 2^(j/64) and ln2/64, from long double arithmetic
   const long double ln2 = logl(2.0L);
   df c = split_ld(ln2 / kExpEntries);
