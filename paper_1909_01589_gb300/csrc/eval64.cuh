@@ -512,6 +512,10 @@ __device__ __forceinline__ dl2 radial_table2(const LShell& sh, const float4* gt,
   const f2 ylo = f2_add(y.lo, x.lo);
   float yh[2], ctr[2], iw[2];
   f2_split(y.hi, yh[0], yh[1]);
+  // x may be a rounding residue below zero: the first cell begins at beta
+#pragma unroll
+  for (int m = 0; m < 2; ++m) yh[m] = fmax_nan(yh[m], sh.gt_beta);
+  const f2 yhi = f2_make(yh[0], yh[1]);
   float4 c[2][3];
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
@@ -531,7 +535,7 @@ __device__ __forceinline__ dl2 radial_table2(const LShell& sh, const float4* gt,
     }
   }
   const f2 w = f2_make(iw[0], iw[1]);
-  const dl2 u = dl2_make(f2_mul(f2_sub(y.hi, f2_make(ctr[0], ctr[1])), w), f2_mul(ylo, w));
+  const dl2 u = dl2_make(f2_mul(f2_sub(yhi, f2_make(ctr[0], ctr[1])), w), f2_mul(ylo, w));
 #define LRDMC_C(q, f) f2_make(c[0][q].f, c[1][q].f)
   f2 t = f2_fma(u.hi, LRDMC_C(2, w), LRDMC_C(2, z));
   t = f2_fma(u.hi, t, LRDMC_C(2, y));
