@@ -650,13 +650,15 @@ static __device__ LRDMC_COLD bool warp_inverses(const SysDev& S, const double* s
 //
 // Bound by the FP64 pipe: an instruction holds it for 64 cycles whatever its
 // lane count. So the local energy is dealt to all lanes (el_L parts per
-// electron, combined by shuffles), a lane evaluates the two moves +-h e_k
-// from D + h^2 +- 2 h (y_ik - y_jk) as the double-float evaluation does
-// (eval64.cuh), square roots take three operations of that pipe, and the e-e
-// Pade sum is one running fraction, c r/(1 + b r) = c/b - (c/b)/(1 + b r),
-// whose constant cancels (three operations per partner instead of nine; for b
-// below 1/4, where that form would lose digits, term by term). Ne, 1021
-// walkers, 4 intervals: 10.34 ms to 7.37.
+// electron, combined by shuffles), a lane evaluates the two moves +-h e_k,
+// square roots take three operations of that pipe, and the e-e Pade sum is one
+// running fraction, c r/(1 + b r) = c/b - (c/b)/(1 + b r), whose constant
+// cancels (three operations per partner instead of nine; for b below 1/4,
+// where that form would lose digits, and above 2^20 term by term). Distances
+// come from the differences of positions: D + h^2 +- 2 h (y_ik - y_jk), as in
+// eval64.cuh, is as fast to 1 % (Ne, 1021 walkers, 4 intervals: 7.45 ms
+// against 7.54, 10.34 before this form), but its absolute error of 2^-53 h^2
+// costs a move that lands close to the partner the digits this mode stands for.
 // ----------------------------------------------------------------------------
 // den's power of two out of num/den (exact)
 __device__ __forceinline__ void pow2_rescale64(double& num, double& den)
@@ -676,7 +678,6 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
   const BlockMem bm = block_mem(S, const_cast<double*>(sC));
   double* see_i = wm.Ssum;                               // [N] e-e sums: of c q, or c r q (below b = 1/4)
   double* sen_i = reinterpret_cast<double*>(wm.Sn);      // [N] e-n sums and the neural terms
-  double* y = reinterpret_cast<double*>(wm.y);           // [N][3] positions on the rotated axes
   const bool recip = S.ee_recip != 0;
   // projected inverse columns: v[i][mu] = sum_m C[mu][m] Ainv_sigma[m][l_i]
 #pragma unroll 1
@@ -685,11 +686,6 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
     int spin = i < nu ? 0 : 1, l = i < nu ? i : i - nu, n = spin ? S.n_dn : nu;
     const double* A = spin ? wm.A + nu * nu : wm.A;
     wm.v[idx] = project_ao(S, bm, A, mu, l, n);
-  }
-#pragma unroll 1
-  for (int j = lane; moves && j < 3 * N; j += 32) {
-    const int i = j / 3, k = j - 3 * i;
-    y[j] = wm.R[k] * wm.x[3 * i] + wm.R[3 + k] * wm.x[3 * i + 1] + wm.R[6 + k] * wm.x[3 * i + 2];
   }
   __syncwarp();
   // local energy: E electrons at a time, Lp lanes (parts) each
@@ -829,7 +825,6 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
       }
     }
     double jee[2] = {0.0, 0.0};
-    const double hh = 2.0 * h, yi = y[3 * i + k];
     const int si = spin_of(S, i);
 #pragma unroll 1
     for (int sp = 0; sp < 2; ++sp) {
@@ -840,12 +835,12 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
       for (int j = j0; j < j1; ++j) {
         if (j == i) continue;
         const double d0 = ri[0] - wm.x[3 * j], d1 = ri[1] - wm.x[3 * j + 1], d2 = ri[2] - wm.x[3 * j + 2];
-        const double D = fma(d0, d0, fma(d1, d1, fma(d2, d2, h2))), p = hh * (yi - y[3 * j + k]);
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-          double t = m ? D - p : D + p;
-          if (t < 0.0) t = 0.0;  // a rounding residue
-          const double r = sqrt64(t), q = fma(S.b_ee, r, 1.0);
+          // from the differences: D + h^2 +- 2 h p loses a move that lands close to the partner
+          const double w0 = m ? d0 - he[0] : d0 + he[0], w1 = m ? d1 - he[1] : d1 + he[1],
+                       w2 = m ? d2 - he[2] : d2 + he[2];
+          const double r = sqrt64(fma(w0, w0, fma(w1, w1, w2 * w2))), q = fma(S.b_ee, r, 1.0);
           if (recip) {
             num[m] = fma(num[m], q, den[m]);
             den[m] *= q;
