@@ -23,6 +23,12 @@
 //     range, the product form c r q);
 //   * after a jump only what moved is formed again: the projected columns of
 //     one spin, one electron's position and its N - 1 distances.
+// Near a node the projected columns are large and the basis sums cancel, so
+// the radial parts and their sums are renormalised at every step (1 to 3 % of
+// a projection's time): error of the ratios against 64 bits, in the 2-norm
+// over 8 samples of 150 configurations (Kr 30; geometric mean), He 5.8e-15, Ne
+// 8e-14, H2O 1.7e-13, Ar 1.3e-13, Kr 1.6e-13, where products and sums left
+// unnormalised gave 7.9e-15, 1.3e-13, 2.6e-13, 1.8e-13 and 2.3e-13.
 #pragma once
 #include "lean64.cuh"
 
@@ -166,7 +172,7 @@ __device__ __forceinline__ void en_geometry(const SysDev& S, const WarpMem& wm, 
 {
 #pragma unroll
   for (int k = 0; k < 3; ++k) d[k] = dl_sub_n(wm.xd[3 * i + k], S.D.nuc[I][k]);
-  D = dl_norm(dl_add(dl_add(dl_sqr(d[0]), dl_sqr(d[1])), dl_sqr(d[2])));
+  D = dl_add_n(dl_add_n(dl_norm(dl_sqr(d[0])), dl_norm(dl_sqr(d[1]))), dl_norm(dl_sqr(d[2])));
 }
 
 __device__ __forceinline__ dl axis_dot(const WarpMem& wm, int k, const dl d[3])
@@ -258,16 +264,17 @@ __device__ __forceinline__ double local_energy64(const SysDev& S, const WarpMem&
             for (int p = 0; p < sh.n_prim; ++p) {
               const float4 pr = lt.prim[sh.prim + p];
               const dl al = dl_at(pr, 0);
-              const dl g = dl_mul_n(dl_at(pr, 1), dl_exp(dl_neg(dl_norm(dl_mul(al, r2))), S.D.lexp, lt.tab));
+              // R'/r = -2 sum a g, R'' = 4 sum a g (a r^2 - 1/2)
+              const dl t = dl_norm(dl_mul(al, r2));
+              const dl g = dl_mul_n(dl_at(pr, 1), dl_norm(dl_exp(dl_neg(t), S.D.lexp, lt.tab)));
               const dl ag = dl_mul_n(al, g);
-              A0 = dl_add(A0, g);
-              A1 = dl_add(A1, ag);
-              A2 = dl_add(A2, dl_mul(al, ag));
+              A0 = dl_add_n(A0, g);
+              A1 = dl_add_n(A1, ag);
+              A2 = dl_add_n(A2, dl_mul_n(dl_norm(dl_add_f(t, -0.5f)), ag));
             }
-            R = dl_norm(A0);
-            A1 = dl_norm(A1);
+            R = A0;
             R1 = dl_scale(A1, -2.0f);
-            R2 = dl_add_n(dl_scale(dl_mul(dl_norm(A2), r2), 4.0f), R1);
+            R2 = dl_scale(A2, 4.0f);
           }
           dl P, g[3];
           if (sh.l == 0) {
@@ -629,7 +636,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
           for (int p = 0; p < sh.n_prim; ++p) {
             const float4 pr = lt.prim[sh.prim + p];
             const dl2 al = dl2_all(df_make(-pr.x, -pr.y)), co = dl2_all(df_make(pr.z, pr.w));
-            R = dl2_add(R, dl2_mul(co, dl2_exp(dl2_norm(dl2_mul(al, r2)), S.D.lexp, lt.tab)));
+            R = dl2_add_n(R, dl2_mul_n(co, dl2_norm(dl2_exp(dl2_norm(dl2_mul(al, r2)), S.D.lexp, lt.tab))));
           }
         }
         dl2 P;
@@ -643,7 +650,7 @@ __device__ __forceinline__ void moves64(const SysDev& S, const LatDev& L, const 
           for (int t = 0; t < 3; ++t) dm[t] = dl2_add_n(dl2_all(d[t]), dl2_pm(he[t]));
           P = solid2_dot2(&v[sh.ao], dm);
         }
-        rdet = dl2_add(rdet, dl2_mul(P, R));
+        rdet = dl2_add_n(rdet, dl2_mul(P, dl2_norm(R)));
       }
     }
   }
