@@ -595,22 +595,34 @@ def tc_leg(args, pkg, torch, seed):
     return out
 
 
+# the sources of the interval kernel, in the order they are hashed
+KERNEL_SOURCES = ("lrdmc_kernels.cu", "eval64.cuh", "lean64.cuh", "df64.cuh", "mixed_arith.cuh", "exp_table.inc",
+                  "lrdmc_internal.h")
+
+
+def _kernel_hash():
+    """SHA-256 over every source that makes up the interval kernel."""
+    import hashlib
+
+    h = hashlib.sha256()
+    for name in KERNEL_SOURCES:
+        with open(os.path.join(ROOT, "paper_1909_01589_gb300", "csrc", name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()
+
+
 def _read_profile(precision):
     """The ncu record of k_interval in this arithmetic on the bench workload
     (profiles/k_interval_<precision>_ne4096_traffic.json: dram bytes per
-    launch and pipe activities), if the kernel source has not changed since
+    launch and pipe activities), if no source of the kernel has changed since
     it was taken; else None."""
     path = os.path.join(ROOT, "profiles", f"k_interval_{precision}_ne4096_traffic.json")
     try:
-        d = json.load(open(path))
+        with open(path) as f:
+            d = json.load(f)
+        return d if d.get("kernel_sha256") == _kernel_hash() else None
     except (OSError, ValueError):
         return None
-    import hashlib
-
-    src = open(os.path.join(ROOT, "paper_1909_01589_gb300", "csrc", "lrdmc_kernels.cu"), "rb").read()
-    if hashlib.sha256(src).hexdigest() != d.get("kernel_sha256"):
-        return None
-    return d
 
 
 def roofline(system, G, precision, leg):
