@@ -596,7 +596,7 @@ def tc_leg(args, pkg, torch, seed):
 
 
 # the sources of the interval kernel, in the order they are hashed
-KERNEL_SOURCES = ("lrdmc_kernels.cu", "eval64.cuh", "lean64.cuh", "df64.cuh", "mixed_arith.cuh", "exp_table.inc",
+KERNEL_SOURCES = ("lrdmc_kernels.cu", "eval64.cuh", "lean64.cuh", "df64.cuh", "exp_table.inc",
                   "lrdmc_internal.h")
 
 

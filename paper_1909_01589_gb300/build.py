@@ -37,8 +37,8 @@ def _inputs():
 
 def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> str:
     """Compile liblrdmc.so (liblrdmc_bounds.so with bounds=True) unless it is
-    newer than every source. Extra nvcc flags (tuning macros such as
-    -DLRDMC_DF_OUTLINE) come from the environment variable LRDMC_NVCC_FLAGS."""
+    newer than every source. Extra nvcc flags come from the environment
+    variable LRDMC_NVCC_FLAGS."""
     lib = LIB_BOUNDS if bounds else LIB
     if not force and os.path.exists(lib):
         newest = max(os.path.getmtime(f) for f in _inputs())

@@ -196,7 +196,7 @@ __device__ __forceinline__ dl nj_value64(const SysDev& S, int c, dl r)
   const float rf = r.hi;
   if (!(rf < S.nj_rcut_f[c])) return df_make(0.0f, 0.0f);
   df E[8];
-  nj_load(nj_cell_m<df>(S, c, rf), E);
+  nj_load(nj_cell_m(S, c, rf), E);
   const dl t = dl_mul(dl_sub_n(r, E[0]), E[1]);
   const float hi = fmaf(fmaf(E[7].hi, t.hi, E[6].hi), t.hi, E[5].hi);
   dl v = dl_add(E[4], dl_mul_f(t, hi));
@@ -204,9 +204,25 @@ __device__ __forceinline__ dl nj_value64(const SysDev& S, int c, dl r)
   return dl_add_n(dl_mul(v, t), E[2]);
 }
 
-__device__ __forceinline__ void nj_value3_64(const SysDev& S, int c, dl r, dl& g, dl& g1, dl& g2)
+__device__ __forceinline__ void nj_value3_64(const SysDev& S, int c, dl r0, dl& g, dl& g1, dl& g2)
 {
-  nj_value3_m<df>(S, c, dl_norm(r), g, g1, g2);
+  g = g1 = g2 = df_make(0.0f, 0.0f);
+  const df r = dl_norm(r0);
+  if (!(r.hi < S.nj_rcut_f[c])) return;
+  df E[8];
+  nj_load(nj_cell_m(S, c, r.hi), E);
+  const df iw = E[1], t = df_mul(df_sub(r, E[0]), iw);
+  df v = E[7], d1 = df_mul_f(E[7], 5.0f), d2 = df_mul_f(E[7], 20.0f);
+#pragma unroll
+  for (int q = 6; q >= 2; --q) v = df_add(df_mul(v, t), E[q]);
+  g = v;
+#pragma unroll
+  for (int q = 6; q >= 4; --q) d1 = df_add(df_mul(d1, t), df_mul_f(E[q], (float)(q - 2)));
+  d1 = df_add(df_mul(d1, t), E[3]);
+#pragma unroll
+  for (int q = 6; q >= 4; --q) d2 = df_add(df_mul(d2, t), df_mul_f(E[q], (float)((q - 2) * (q - 3))));
+  g1 = df_mul(d1, iw);
+  g2 = df_mul(d2, df_sqr(iw));
 }
 
 // ----------------------------------------------------------------------------

@@ -98,7 +98,6 @@ struct DfSys {
   df en_b1[kMaxNuc];
   df b_ee, c_par, c_anti, en_b2;
   DfShell sh[kMaxShell];
-  ExpTable exp;
   df inv_fact[18];  // 1/k!, k = 0..17 (series of sin and cos)
   df half_pi;
   LeanExp lexp;
@@ -192,13 +191,9 @@ int accept_smem_bytes(const SysDev& S, bool caches);
 // Entries of the double-float exponential's table.
 constexpr int kExpBits = 10;
 constexpr int kExpEntries = 1 << kExpBits;
-// A block's shared tables: the MO coefficients in the three arithmetics, the
-// 64-entry table, the coefficients' masks; then the double-float ones.
-__host__ __device__ inline int mask_offset(const SysDev& S)
-{
-  const int nc = S.n_ao * S.n_mo;
-  return (2 * nc + (nc + 1) / 2 + 64 + 1) & ~1;
-}
+// A block's shared tables: the MO coefficients, their masks, then the
+// double-float ones.
+__host__ __device__ inline int mask_offset(const SysDev& S) { return 2 * ((S.n_ao * S.n_mo + 1) / 2); }
 __host__ __device__ inline int lean_offset(const SysDev& S)
 {
   return (mask_offset(S) + S.n_mo + (S.n_ao + 1) / 2 + 1) & ~1;

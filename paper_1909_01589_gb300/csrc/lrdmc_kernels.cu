@@ -33,7 +33,6 @@
 #include <mutex>
 
 #include "lrdmc_internal.h"
-#include "mixed_arith.cuh"
 #include "lean64.cuh"
 
 // This file is compiled several times, so that the kernel variants build in
@@ -50,23 +49,6 @@ namespace lrdmc {
 // ----------------------------------------------------------------------------
 // Counter-based random numbers: Philox4x64-10 (Salmon, Moraes, Dror, Shaw,
 // SC'11), key (seed, 0), counter (slot, interval, iteration, tag).
-// Inlining of the large, once-per-jump or rarely executed parts of the
-// interval loop (tuning switches; the default inlines everything):
-//   LRDMC_NOINLINE_COLD  the Gauss-Jordan recompute (every few intervals)
-//   LRDMC_NOINLINE_JUMP  the Sherman-Morrison update and the new rotation
-#ifdef LRDMC_NOINLINE_COLD
-#define LRDMC_COLD __noinline__
-#else
-#define LRDMC_COLD
-#endif
-#ifdef LRDMC_NOINLINE_JUMP
-#define LRDMC_JUMP __noinline__
-#define LRDMC_JUMP_INLINE __noinline__
-#else
-#define LRDMC_JUMP
-#define LRDMC_JUMP_INLINE __forceinline__
-#endif
-
 // ----------------------------------------------------------------------------
 __device__ __forceinline__ void philox4x64_10(uint64_t c[4], uint64_t k0, uint64_t k1)
 {
@@ -142,7 +124,7 @@ static __device__ void rotation_matrix(double u1, double u2, double u3, double* 
 // sincospi(2 u2) and sincospi(2 u3), lanes 0-8 then form one entry of R
 // each. IEEE double (the same operations as rotation_matrix), for the FP64
 // mode; the others draw ahead. All lanes must call it; R goes to shared memory.
-__device__ LRDMC_JUMP_INLINE void rotation_matrix_warp(const uint64_t* bits, double* R, int lane)
+__device__ __forceinline__ void rotation_matrix_warp(const uint64_t* bits, double* R, int lane)
 {
   double x, y, z, w;
   {
@@ -466,13 +448,9 @@ __device__ __forceinline__ WarpMem warp_mem(const Layout& Lo, const SysDev& S, d
   return m;
 }
 
-// Block-shared tables: MO coefficients (double, then double-float and float
-// copies), the 2^(j/64) table, the masks of the non-zero coefficients.
+// Block-shared tables: the MO coefficients and the masks of the non-zero ones.
 struct BlockMem {
   double* C;
-  df* Cd;
-  float* Cf;
-  float2* tab;
   unsigned long long* col;  // [n_mo] non-zero rows of a column of C
   unsigned* row;            // [n_ao] non-zero columns of a row
 };
@@ -480,11 +458,7 @@ struct BlockMem {
 __device__ __forceinline__ BlockMem block_mem(const SysDev& S, double* smem)
 {
   BlockMem b;
-  const int nc = S.n_ao * S.n_mo;
   b.C = smem;
-  b.Cd = reinterpret_cast<df*>(smem + nc);
-  b.Cf = reinterpret_cast<float*>(smem + 2 * nc);
-  b.tab = reinterpret_cast<float2*>(smem + 2 * nc + (nc + 1) / 2);
   b.col = reinterpret_cast<unsigned long long*>(smem + mask_offset(S));
   b.row = reinterpret_cast<unsigned*>(smem + mask_offset(S) + S.n_mo);
   return b;
@@ -532,7 +506,7 @@ __device__ __forceinline__ double orbital_value(const SysDev& S, const BlockMem&
 // produced where its pivot columns vanish, with the same operations). Pivots
 // are compared as integers, off that pipe.
 // ----------------------------------------------------------------------------
-static __device__ LRDMC_COLD bool warp_inverses(const SysDev& S, const double* sC, const double* sx, double* Ainv0,
+static __device__ bool warp_inverses(const SysDev& S, const double* sC, const double* sx, double* Ainv0,
                                                 double* scr, int lane, double* resid = nullptr)
 {
   const BlockMem bm = block_mem(S, const_cast<double*>(sC));
@@ -879,70 +853,57 @@ __device__ void warp_eval(const SysDev& S, const double* sC, const LatDev& L, co
 }
 
 // ----------------------------------------------------------------------------
-// The evaluation on the FP32 pipe, templated on the number type NT:
-//   NT = df    double-float (LRDMC_PRECISION_DF64), accurate to FP64 parity;
-//   NT = float single precision (LRDMC_PRECISION_FP32), the mixed mode.
-// Inputs are converted once per evaluation (positions, rotation, projected
-// inverse columns) and kept as double-floats in shared memory (the FP32 mode
-// reads their high parts); every lattice move and the local energy are
-// computed in NT; rates stay in NT (stored as double-floats), the local
-// energy is converted to double.
+// The lattice moves of the mixed mode (LRDMC_PRECISION_FP32) in single
+// precision. They read the leading floats of the evaluation's double-float
+// state in shared memory (positions, rotation, projected inverse columns,
+// Jastrow sums); rates are stored as double-floats with a zero low part.
 // ----------------------------------------------------------------------------
-template <class NT>
-__device__ __forceinline__ NT dot3(NT a0, NT a1, NT a2)
+__device__ __forceinline__ float dot3(float a0, float a1, float a2)
 {
-  typedef Ar<NT> A;
-  return A::add_fast(A::add_fast(A::sqr(a0), A::sqr(a1)), A::sqr(a2));
+  return a0 * a0 + a1 * a1 + a2 * a2;
 }
 
 // Slater radial part r^m e^(-zeta r) (e given) or a Gaussian contraction.
-template <class NT>
-__device__ __forceinline__ NT radial_value_m(const SysDev& S, const ShellDev& sh, const DfShell& dsh, NT r, NT r2,
-                                             NT e, const BlockMem& bm)
+__device__ __forceinline__ float radial_value_m(const ShellDev& sh, const DfShell& dsh, float r, float r2, float e)
 {
-  typedef Ar<NT> A;
   if (sh.kind == 0) {
     if (sh.m_int >= 0) {
-      NT pw = A::one();
-      for (int j = 0; j < sh.m_int; ++j) pw = A::mul(pw, r);
-      return A::mul(pw, e);
+      float pw = 1.0f;
+      for (int j = 0; j < sh.m_int; ++j) pw = pw * r;
+      return pw * e;
     }
-    NT lr = A::log(r, S.D.exp.K, bm.tab);
-    return A::mul(A::exp(A::mul(A::c(dsh.m), lr), S.D.exp.K, bm.tab), e);
+    float lr = logf(r);
+    return expf(dsh.m.hi * lr) * e;
   }
-  NT acc = A::zero();
+  float acc = 0.0f;
   for (int p = 0; p < sh.n_prim; ++p)
-    acc = A::add(acc, A::mul(A::c(dsh.coef[p]),
-                             A::exp(A::neg(A::mul(A::c(dsh.alpha[p]), r2)), S.D.exp.K, bm.tab)));
+    acc = acc + dsh.coef[p].hi * expf(-(dsh.alpha[p].hi * r2));
   return acc;
 }
 
-template <class NT>
-__device__ __forceinline__ int solid_m(int l, const NT d[3], NT Sv[5])
+__device__ __forceinline__ int solid_m(int l, const float d[3], float Sv[5])
 {
-  typedef Ar<NT> A;
   if (l == 0) {
-    Sv[0] = A::one();
+    Sv[0] = 1.0f;
     return 1;
   }
   if (l == 1) {
     Sv[0] = d[0]; Sv[1] = d[1]; Sv[2] = d[2];
     return 3;
   }
-  NT xx = A::sqr(d[0]), yy = A::sqr(d[1]), zz = A::sqr(d[2]);
-  Sv[0] = A::mul(d[0], d[1]);
-  Sv[1] = A::mul(d[1], d[2]);
-  Sv[2] = A::mul(d[2], d[0]);
-  Sv[3] = A::sub(xx, yy);
-  Sv[4] = A::sub(A::add(zz, zz), A::add(xx, yy));
+  float xx = d[0] * d[0], yy = d[1] * d[1], zz = d[2] * d[2];
+  Sv[0] = d[0] * d[1];
+  Sv[1] = d[1] * d[2];
+  Sv[2] = d[2] * d[0];
+  Sv[3] = xx - yy;
+  Sv[4] = zz + zz - (xx + yy);
   return 5;
 }
 
 // Per nucleus I (one distance each): the determinant ratio
 // sum_mu v[mu] chi_mu(p) over the shells centred on I, and the e-n Jastrow
 // -sum_I b1_I r/(1 + b2 r).
-// The neural pair term in NT arithmetic (same table, double-float copy).
-template <class NT>
+// The neural pair term (the double-float copy of the table): the cell at r.
 __device__ __forceinline__ const df* nj_cell_m(const SysDev& S, int c, float rf)
 {
   int k = (int)(sqrtf(rf) * S.nj_scale_f[c]);
@@ -961,102 +922,57 @@ __device__ __forceinline__ void nj_load(const df* e, df E[8])
   }
 }
 
-template <class NT>
-__device__ __forceinline__ NT nj_value_m(const SysDev& S, int c, NT r)
+__device__ __forceinline__ float nj_value_m(const SysDev& S, int c, float r)
 {
-  typedef Ar<NT> A;
-  const float rf = A::approx(r);
-  if (!(rf < S.nj_rcut_f[c])) return A::zero();
+  if (!(r < S.nj_rcut_f[c])) return 0.0f;
   df E[8];
-  nj_load(nj_cell_m<NT>(S, c, rf), E);
-  const NT t = A::mul(A::sub(r, A::c(E[0])), A::c(E[1]));
-  if (sizeof(NT) == sizeof(df)) {
-    // the cubic to quintic terms are below 1e-5 of the value on these narrow
-    // cells (c_q ~ w^q g^(q)/q!), so single precision carries them to well
-    // below the double-float rounding of the sum; the low orders in NT
-    const float tf = A::approx(t);
-    const float hi = fmaf(fmaf(E[7].hi, tf, E[6].hi), tf, E[5].hi);
-    NT v = A::add(A::c(E[4]), A::mul_f(t, hi));
-    v = A::add(A::mul(v, t), A::c(E[3]));
-    return A::add(A::mul(v, t), A::c(E[2]));
-  }
-  NT v = A::c(E[7]);
+  nj_load(nj_cell_m(S, c, r), E);
+  const float t = (r - E[0].hi) * E[1].hi;
+  float v = E[7].hi;
 #pragma unroll
-  for (int q = 6; q >= 2; --q) v = A::add(A::mul(v, t), A::c(E[q]));
+  for (int q = 6; q >= 2; --q) v = v * t + E[q].hi;
   return v;
-}
-
-template <class NT>
-__device__ __forceinline__ void nj_value3_m(const SysDev& S, int c, NT r, NT& g, NT& g1, NT& g2)
-{
-  typedef Ar<NT> A;
-  g = A::zero(); g1 = A::zero(); g2 = A::zero();
-  const float rf = A::approx(r);
-  if (!(rf < S.nj_rcut_f[c])) return;
-  df E[8];
-  nj_load(nj_cell_m<NT>(S, c, rf), E);
-  const NT iw = A::c(E[1]);
-  const NT t = A::mul(A::sub(r, A::c(E[0])), iw);
-  const NT c1 = A::c(E[3]), c2 = A::c(E[4]), c3 = A::c(E[5]), c4 = A::c(E[6]), c5 = A::c(E[7]);
-  NT v = c5, d1 = A::mul_f(c5, 5.0f), d2 = A::mul_f(c5, 20.0f);
-  v = A::add(A::mul(v, t), c4);
-  v = A::add(A::mul(v, t), c3);
-  v = A::add(A::mul(v, t), c2);
-  v = A::add(A::mul(v, t), c1);
-  g = A::add(A::mul(v, t), A::c(E[2]));
-  d1 = A::add(A::mul(d1, t), A::mul_f(c4, 4.0f));
-  d1 = A::add(A::mul(d1, t), A::mul_f(c3, 3.0f));
-  d1 = A::add(A::mul(d1, t), A::mul_f(c2, 2.0f));
-  d1 = A::add(A::mul(d1, t), c1);
-  d2 = A::add(A::mul(d2, t), A::mul_f(c4, 12.0f));
-  d2 = A::add(A::mul(d2, t), A::mul_f(c3, 6.0f));
-  d2 = A::add(A::mul(d2, t), A::mul_f(c2, 2.0f));
-  g1 = A::mul(d1, iw);
-  g2 = A::mul(d2, A::sqr(iw));
 }
 
 // One nucleus's part of a lattice move: the e-n Jastrow terms (Pade and,
 // when set, neural) into jen and the basis functions centred on it,
 // contracted with the projected inverse column v, into rdet. d = r' - R_I,
 // r2 = |d|^2.
-template <class NT, bool NJ>
-__device__ __forceinline__ void nucleus_term_m(const SysDev& S, const df* v, int I, const NT d[3], NT r2,
-                                               const BlockMem& bm, NT& rdet, NT& jen)
+template <bool NJ>
+__device__ __forceinline__ void nucleus_term_m(const SysDev& S, const df* v, int I, const float d[3], float r2,
+                                               float& rdet, float& jen)
 {
-  typedef Ar<NT> A;
-  NT r = A::sqrt(r2);
+  float r = sqrtf(r2);
   if (S.en_b1[I] != 0.0)
-    jen = A::sub(jen, A::div(A::mul(A::c(S.D.en_b1[I]), r), A::add_f(A::mul(A::c(S.D.en_b2), r), 1.0f)));
-  if (NJ) jen = A::add(jen, nj_value_m<NT>(S, 2 + S.nj_species[I], r));
-  NT e = A::zero();
+    jen = jen - S.D.en_b1[I].hi * r / (S.D.en_b2.hi * r + 1.0f);
+  if (NJ) jen = jen + nj_value_m(S, 2 + S.nj_species[I], r);
+  float e = 0.0f;
   for (int q = S.nuc_shell_begin[I]; q < S.nuc_shell_begin[I + 1]; ++q) {
     const ShellDev& sh = S.sh[q];
     const DfShell& dsh = S.D.sh[q];
-    if (sh.kind == 0 && !sh.same_exp) e = A::exp(A::neg(A::mul(A::c(dsh.zeta), r)), S.D.exp.K, bm.tab);
-    NT Rv = radial_value_m<NT>(S, sh, dsh, r, r2, e, bm);
-    NT part;
+    if (sh.kind == 0 && !sh.same_exp) e = expf(-(dsh.zeta.hi * r));
+    float Rv = radial_value_m(sh, dsh, r, r2, e);
+    float part;
     if (sh.l == 0) {
-      part = A::c(v[sh.ao_offset]);
+      part = v[sh.ao_offset].hi;
     } else {
-      NT Sv[5];
-      int nf = solid_m<NT>(sh.l, d, Sv);
-      part = A::zero();
-      for (int f = 0; f < nf; ++f) part = A::add(part, A::mul(A::c(v[sh.ao_offset + f]), Sv[f]));
+      float Sv[5];
+      int nf = solid_m(sh.l, d, Sv);
+      part = 0.0f;
+      for (int f = 0; f < nf; ++f) part = part + v[sh.ao_offset + f].hi * Sv[f];
     }
-    rdet = A::add(rdet, A::mul(part, Rv));
+    rdet = rdet + part * Rv;
   }
 }
 
-template <class NT, bool NJ>
-__device__ void nucleus_terms_m(const SysDev& S, const df* v, const NT p[3], const BlockMem& bm, NT& rdet, NT& jen)
+template <bool NJ>
+__device__ void nucleus_terms_m(const SysDev& S, const df* v, const float p[3], float& rdet, float& jen)
 {
-  typedef Ar<NT> A;
-  rdet = A::zero();
-  jen = A::zero();
+  rdet = 0.0f;
+  jen = 0.0f;
   for (int I = 0; I < S.n_nuc; ++I) {
-    NT d[3] = {A::sub_fast(p[0], A::c(S.D.nuc[I][0])), A::sub_fast(p[1], A::c(S.D.nuc[I][1])),
-               A::sub_fast(p[2], A::c(S.D.nuc[I][2]))};
-    nucleus_term_m<NT, NJ>(S, v, I, d, dot3<NT>(d[0], d[1], d[2]), bm, rdet, jen);
+    const float d[3] = {p[0] - S.D.nuc[I][0].hi, p[1] - S.D.nuc[I][1].hi, p[2] - S.D.nuc[I][2].hi};
+    nucleus_term_m<NJ>(S, v, I, d, dot3(d[0], d[1], d[2]), rdet, jen);
   }
 }
 
@@ -1069,84 +985,65 @@ __device__ __forceinline__ void pow2_rescale(float& num, float& den)
   den *= s;
 }
 
-__device__ __forceinline__ void pow2_rescale(df& num, df& den)
-{
-  const float s = __int_as_float((254 - ((__float_as_int(den.hi) >> 23) & 0xff)) << 23);
-  num.hi *= s;
-  num.lo *= s;
-  den.hi *= s;
-  den.lo *= s;
-}
-
 // sum_{j != i} u_ee(|p - r_j|): the Pade terms c r/(1 + b r) (all of one
 // sign) are summed as one running fraction num/den, so one division serves
 // all partners. Every 16 partners pow2_rescale brings den back into [1, 2):
 // the product of the (1 + b r) would otherwise leave the float exponent
-// range (about 3.4e38) that double-floats and floats share, as 47 partners
-// a few bohr away do; 16 factors fit while their geometric mean stays
-// below 200.
-template <class NT, bool NJ>
-__device__ NT jastrow_ee_m(const SysDev& S, const df* xd, int i, const NT p[3])
+// range (about 3.4e38), as 47 partners a few bohr away do; 16 factors fit
+// while their geometric mean stays below 200.
+template <bool NJ>
+__device__ float jastrow_ee_m(const SysDev& S, const df* xd, int i, const float p[3])
 {
-  typedef Ar<NT> A;
-  NT num = A::zero(), den = A::one(), nn = A::zero();
+  float num = 0.0f, den = 1.0f, nn = 0.0f;
   const int si = spin_of(S, i);
-  const NT b = A::c(S.D.b_ee), cp = A::c(S.D.c_par), ca = A::c(S.D.c_anti);
+  const float b = S.D.b_ee.hi, cp = S.D.c_par.hi, ca = S.D.c_anti.hi;
   for (int j = 0; j < S.N; ++j) {
     if (j == i) continue;
-    NT d0 = A::sub_fast(p[0], A::c(xd[3 * j])), d1 = A::sub_fast(p[1], A::c(xd[3 * j + 1])),
-       d2 = A::sub_fast(p[2], A::c(xd[3 * j + 2]));
-    NT r = A::sqrt(dot3<NT>(d0, d1, d2));
-    NT c = (spin_of(S, j) == si) ? cp : ca;
-    NT dj = A::add_f(A::mul(b, r), 1.0f);
-    num = A::add_fast(A::mul(num, dj), A::mul(A::mul(c, r), den));
-    den = A::mul(den, dj);
-    if (NJ) nn = A::add(nn, nj_value_m<NT>(S, nj_ch_ee(S, i, j), r));
+    const float r = sqrtf(dot3(p[0] - xd[3 * j].hi, p[1] - xd[3 * j + 1].hi, p[2] - xd[3 * j + 2].hi));
+    const float c = (spin_of(S, j) == si) ? cp : ca;
+    const float dj = b * r + 1.0f;
+    num = num * dj + c * r * den;
+    den = den * dj;
+    if (NJ) nn = nn + nj_value_m(S, nj_ch_ee(S, i, j), r);
     if ((j & 15) == 15) pow2_rescale(num, den);
   }
-  return A::add(A::div(num, den), nn);
+  return num / den + nn;
 }
 
-template <class NT>
-__device__ __forceinline__ NT p_weight_m(const SysDev& S, const LatDev& L, const NT m[3], const BlockMem& bm)
+__device__ __forceinline__ float p_weight_m(const SysDev& S, const LatDev& L, const float m[3])
 {
-  typedef Ar<NT> A;
-  NT best = A::inf();
+  float best = INFINITY;
   for (int I = 0; I < S.n_nuc; ++I) {
     if (!S.heavy[I]) continue;
-    NT d0 = A::sub_fast(m[0], A::c(S.D.nuc[I][0])), d1 = A::sub_fast(m[1], A::c(S.D.nuc[I][1])),
-       d2 = A::sub_fast(m[2], A::c(S.D.nuc[I][2]));
-    NT d2s = dot3<NT>(d0, d1, d2);
-    if (A::lt(d2s, best)) best = d2s;
+    const float d2s = dot3(m[0] - S.D.nuc[I][0].hi, m[1] - S.D.nuc[I][1].hi, m[2] - S.D.nuc[I][2].hi);
+    if (d2s < best) best = d2s;
   }
-  if (L.pkind == 0) return A::exp(A::neg(A::mul(best, A::c(L.p_coef_df))), S.D.exp.K, bm.tab);
-  return A::rcp(A::add_f(A::mul(A::c(L.p_coef_df), best), 1.0f));
+  if (L.pkind == 0) return expf(-(best * L.p_coef_df.hi));
+  return 1.0f / (L.p_coef_df.hi * best + 1.0f);
 }
 
-// Chunked inclusive scan of the rates (as warp_scan) in NT.
-template <class NT>
-__device__ NT warp_scan_m(const df* T, int P, int lane, NT target, int* pick, int* last)
+// Chunked inclusive scan of the rates (as warp_scan) in single precision.
+static __device__ float warp_scan_m(const df* T, int P, int lane, float target, int* pick, int* last)
 {
-  typedef Ar<NT> A;
-  NT carry = A::zero();
+  float carry = 0.0f;
   int p = -1, lp = -1;
   for (int base = 0; base < P; base += 32) {
     int c = base + lane;
-    NT t = (c < P) ? A::c(T[c]) : A::zero();
-    NT v = t;
+    float t = (c < P) ? T[c].hi : 0.0f;
+    float v = t;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      NT y = A::shfl_up(v, o);
-      if (lane >= o) v = A::add(v, y);
+      float y = __shfl_up_sync(FULL_MASK, v, o);
+      if (lane >= o) v = v + y;
     }
-    NT C = A::add(carry, v);
+    float C = carry + v;
     if (pick) {
-      unsigned hit = __ballot_sync(FULL_MASK, (c < P) && A::lt(target, C));
+      unsigned hit = __ballot_sync(FULL_MASK, (c < P) && target < C);
       if (p < 0 && hit) p = base + __ffs(hit) - 1;
-      unsigned pos = __ballot_sync(FULL_MASK, (c < P) && A::positive(t));
+      unsigned pos = __ballot_sync(FULL_MASK, (c < P) && t > 0.0f);
       if (pos) lp = base + 31 - __clz(pos);
     }
-    carry = A::shfl(C, 31);
+    carry = __shfl_sync(FULL_MASK, C, 31);
   }
   if (pick) { *pick = p; *last = lp; }
   return carry;
@@ -1157,37 +1054,35 @@ __device__ NT warp_scan_m(const df* T, int P, int lane, NT target, int* pick, in
 // midpoint on the double grid, the rate T_c into Td[c]. Reads the
 // evaluation's shared-memory state (projected inverse columns, positions,
 // rotation and the Jastrow sums Sd of its local-energy pass).
-template <class NT, bool NJ>
-__device__ __forceinline__ void candidate_m(const SysDev& S, const LatDev& L, const WarpMem& wm, const BlockMem& bm,
-                                            int c, df* Td, double* ratio_out)
+template <bool NJ>
+__device__ __forceinline__ void candidate_m(const SysDev& S, const LatDev& L, const WarpMem& wm, int c, df* Td,
+                                            double* ratio_out)
 {
-  typedef Ar<NT> A;
   const int nao = S.n_ao;
   const int G = L.G, per_e = 6 * G;
   {
     const int i = c / per_e, rem = c - i * per_e, g = rem / 6, k = (rem % 6) >> 1;
-    NT h = g ? A::c(L.ap_df) : A::c(L.a_df);
-    if (c & 1) h = A::neg(h);
-    const NT e0 = A::c(wm.Rd[k]), e1 = A::c(wm.Rd[3 + k]), e2 = A::c(wm.Rd[6 + k]);
-    NT rdet, jen, jee, pm = A::one();
-    const NT ri[3] = {A::c(wm.xd[3 * i]), A::c(wm.xd[3 * i + 1]), A::c(wm.xd[3 * i + 2])};
-    const NT p[3] = {A::add(ri[0], A::mul(h, e0)), A::add(ri[1], A::mul(h, e1)), A::add(ri[2], A::mul(h, e2))};
-    nucleus_terms_m<NT, NJ>(S, &wm.vd[i * nao], p, bm, rdet, jen);
-    jee = jastrow_ee_m<NT, NJ>(S, wm.xd, i, p);
+    float h = g ? L.ap_df.hi : L.a_df.hi;
+    if (c & 1) h = -h;
+    const float e0 = wm.Rd[k].hi, e1 = wm.Rd[3 + k].hi, e2 = wm.Rd[6 + k].hi;
+    float rdet, jen, jee, pm = 1.0f;
+    const float ri[3] = {wm.xd[3 * i].hi, wm.xd[3 * i + 1].hi, wm.xd[3 * i + 2].hi};
+    const float p[3] = {ri[0] + h * e0, ri[1] + h * e1, ri[2] + h * e2};
+    nucleus_terms_m<NJ>(S, &wm.vd[i * nao], p, rdet, jen);
+    jee = jastrow_ee_m<NJ>(S, wm.xd, i, p);
     if (G == 2) {
-      const NT hh = A::half(h);
-      const NT mid[3] = {A::add(ri[0], A::mul(hh, e0)), A::add(ri[1], A::mul(hh, e1)),
-                         A::add(ri[2], A::mul(hh, e2))};
-      pm = p_weight_m<NT>(S, L, mid, bm);
+      const float hh = 0.5f * h;
+      const float mid[3] = {ri[0] + hh * e0, ri[1] + hh * e1, ri[2] + hh * e2};
+      pm = p_weight_m(S, L, mid);
     }
-    NT dJ = A::sub(A::add(jee, jen), A::c(wm.Sd[i]));
-    NT rho = A::mul(rdet, A::exp(dJ, S.D.exp.K, bm.tab));
-    NT w = A::one();
-    if (G == 2) w = g ? A::add_f(A::neg(pm), 1.0f) : pm;
-    NT T = A::zero();
-    if (A::positive(rho)) T = A::mul(A::mul(w, g ? A::c(L.inv2ap2_df) : A::c(L.inv2a2_df)), rho);
-    Td[c] = A::store(T);
-    if (ratio_out) ratio_out[c] = A::to_double(rho);
+    float dJ = jee + jen - wm.Sd[i].hi;
+    float rho = rdet * expf(dJ);
+    float w = 1.0f;
+    if (G == 2) w = g ? -pm + 1.0f : pm;
+    float T = 0.0f;
+    if (rho > 0.0f) T = w * (g ? L.inv2ap2_df.hi : L.inv2a2_df.hi) * rho;
+    Td[c] = df_make(T, 0.0f);
+    if (ratio_out) ratio_out[c] = (double)rho;
   }
 }
 
@@ -1211,13 +1106,12 @@ template <bool NJ>
 __device__ void warp_eval32(const SysDev& S, double* sC, const LatDev& L, const WarpMem& wm, int lane,
                             double* ratio_out, double& b, double& el)
 {
-  const BlockMem bm = block_mem(S, sC);
   el = prelude32<NJ>(S, sC, wm, lean_mem(S, sC), lane, -1);
   const int P = 6 * L.G * S.N;
   df* Td = reinterpret_cast<df*>(wm.T);  // rates stored as double-floats
-  for (int c = lane; c < P; c += 32) candidate_m<float, NJ>(S, L, wm, bm, c, Td, ratio_out);
+  for (int c = lane; c < P; c += 32) candidate_m<NJ>(S, L, wm, c, Td, ratio_out);
   __syncwarp();
-  b = (double)warp_scan_m<float>(Td, P, lane, 0.0f, nullptr, nullptr);
+  b = (double)warp_scan_m(Td, P, lane, 0.0f, nullptr, nullptr);
 }
 
 template <int PREC, bool NJ, bool NC>
@@ -1240,7 +1134,7 @@ __device__ __forceinline__ void warp_eval_any(const SysDev& S, double* sC, const
 // Ainv[m][n] -= Ainv[m][l] (y_n - delta_nl) / ratio.
 // ----------------------------------------------------------------------------
 // The FP64 mode's update.
-static __device__ LRDMC_JUMP bool warp_sm_update(const SysDev& S, const double* sC, const WarpMem& wm, int i,
+static __device__ bool warp_sm_update(const SysDev& S, const double* sC, const WarpMem& wm, int i,
                                                  const double* p, int lane)
 {
   const int nu = S.n_up;
@@ -1310,12 +1204,7 @@ __device__ __forceinline__ void stage_coefficients(const SysDev& S, double* sC)
 {
   if (LEAN) lean_stage(S, sC);
   BlockMem bm = block_mem(S, sC);
-  for (int j = threadIdx.x; j < S.n_ao * S.n_mo; j += blockDim.x) {
-    sC[j] = S.C[j];
-    bm.Cd[j] = df_from_double(S.C[j]);
-    bm.Cf[j] = (float)S.C[j];
-  }
-  for (int j = threadIdx.x; j < 64; j += blockDim.x) bm.tab[j] = S.D.exp.t[j];
+  for (int j = threadIdx.x; j < S.n_ao * S.n_mo; j += blockDim.x) sC[j] = S.C[j];
   for (int j = threadIdx.x; j < S.n_mo; j += blockDim.x) bm.col[j] = S.col_mask[j];
   for (int j = threadIdx.x; j < S.n_ao; j += blockDim.x) bm.row[j] = S.row_mask[j];
   __syncthreads();
@@ -1433,9 +1322,9 @@ __device__ __forceinline__ int team_publish(TeamSlot* t, int lane)
 // The moves of an evaluation in chunks of 32: alone (t == nullptr) in
 // order, or taken in turn from t->next by the owner and its helpers.
 // A unit is one move, in the double-float mode the two moves along one axis.
-template <class NT, bool NJ, bool NC>
-__device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, const WarpMem& wm, const BlockMem& bm,
-                                              const Lean& lt, TeamSlot* t, int units, int lane, const float4* gt)
+template <bool DF, bool NJ, bool NC>
+__device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, const WarpMem& wm, const Lean& lt,
+                                              TeamSlot* t, int units, int lane, const float4* gt)
 {
   df* Td = reinterpret_cast<df*>(wm.T);
   // in a team chunks of 16 where whole ones would not go round: 3 % faster
@@ -1451,8 +1340,8 @@ __device__ __forceinline__ void chunked_moves(const SysDev& S, const LatDev& L, 
     }
     if (c0 >= units) break;
     if (lane < cs && c0 + lane < units) {
-      if (sizeof(NT) == sizeof(df)) moves64<NJ, NC>(S, L, wm, lt, c0 + lane, Td, nullptr, gt);
-      else candidate_m<float, NJ>(S, L, wm, bm, c0 + lane, Td, nullptr);
+      if (DF) moves64<NJ, NC>(S, L, wm, lt, c0 + lane, Td, nullptr, gt);
+      else candidate_m<NJ>(S, L, wm, c0 + lane, Td, nullptr);
     }
   }
   if (t) __threadfence_block();
@@ -1555,14 +1444,13 @@ static __shared__ WarpState g_ws[kMaxIntervalWarps];
 // each warp is an owner while it runs a walker (the same steps, draws and
 // arithmetic as the loop of the FP64 mode below), then a helper of the
 // warps of its block that still run one.
-template <class NT, int PR, bool NJ, bool NC>
+template <int PR, bool NJ, bool NC>
 __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo, const LatDev& L, const PopDev& P,
                                               double* sC, uint64_t k, bool recompute, int lane, int wib)
 {
   const int P_moves = S.N * 6 * L.G;
   constexpr bool kDf = PR == LRDMC_PRECISION_DF64;
   const int units = kDf ? P_moves / 2 : P_moves;
-  const BlockMem bm = block_mem(S, sC);
   const Lean lt = lean_mem(S, sC);
   TeamSlot* mine = &g_team[wib];
   WarpState& st = g_ws[wib];
@@ -1641,7 +1529,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
                              dl_norm(dl_mul(draws[10], bdf)));
         } else {
           int lastc;
-          warp_scan_m<float>(reinterpret_cast<const df*>(wm.T), P_moves, lane, draws[10].hi * bdf.hi, &pick,
+          warp_scan_m(reinterpret_cast<const df*>(wm.T), P_moves, lane, draws[10].hi * bdf.hi, &pick,
                              &lastc);
           if (pick < 0) pick = lastc;
         }
@@ -1724,8 +1612,8 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
     // code for the owner alone, the owner with helpers, and the helpers
     {
       const WarpMem twm = warp_mem(Lo, S, sC + Lo.head + target * Lo.smem_warp);
-      chunked_moves<NT, NJ, NC>(S, L, twm, bm, lt, (mode == kHelper || nh > 0) ? &g_team[target] : nullptr, units,
-                                lane, P.gt);
+      chunked_moves<kDf, NJ, NC>(S, L, twm, lt, (mode == kHelper || nh > 0) ? &g_team[target] : nullptr, units, lane,
+                                 P.gt);
     }
     if (mode == kHelper) {
       if (lane == 0) atomicAdd(&g_team[target].done, 1);
@@ -1737,7 +1625,7 @@ __device__ __forceinline__ void interval_team(const SysDev& S, const Layout& Lo,
     const df* Td = reinterpret_cast<const df*>(own.T);
     df bnew;
     if (kDf) bnew = rate_scan64(Td, P_moves, lane, own.pfx);
-    else bnew = df_make(warp_scan_m<float>(Td, P_moves, lane, 0.0f, nullptr, nullptr), 0.0f);
+    else bnew = df_make(warp_scan_m(Td, P_moves, lane, 0.0f, nullptr, nullptr), 0.0f);
     const double b = df_to_double(bnew);
     if (lane == 0) {
       st.bdf = bnew;
@@ -1790,8 +1678,8 @@ k_interval(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L, co
   }
   stage_coefficients<(PREC & 3) != LRDMC_PRECISION_FP64>(S, sC);  // ends with __syncthreads
   if constexpr (PR != LRDMC_PRECISION_FP64) {
-    if (PR == LRDMC_PRECISION_DF64) interval_team<df, PR, NJ, NC>(S, Lo, L, P, sC, k, recompute, lane, wib);
-    else interval_team<float, PR, NJ, true>(S, Lo, L, P, sC, k, recompute, lane, wib);
+    if (PR == LRDMC_PRECISION_DF64) interval_team<PR, NJ, NC>(S, Lo, L, P, sC, k, recompute, lane, wib);
+    else interval_team<PR, NJ, true>(S, Lo, L, P, sC, k, recompute, lane, wib);
   } else {
     // the FP64 mode: every warp alone
     WarpMem wm = warp_mem(Lo, S, sC + Lo.head + wib * Lo.smem_warp);
@@ -2280,7 +2168,7 @@ __device__ __forceinline__ void evaluate_block(const SysDev& S, const Layout& Lo
       df* Td = reinterpret_cast<df*>(wm.T);
       double* ro = ratio ? ratio + (size_t)cq * P : nullptr;
       if (PR == LRDMC_PRECISION_DF64) moves64<NJ, NC>(S, L, wm, lt, u, Td, ro, nullptr);
-      else candidate_m<float, NJ>(S, L, wm, block_mem(S, sC), u, Td, ro);
+      else candidate_m<NJ>(S, L, wm, u, Td, ro);
     }
     __syncthreads();
     if (ok) {
@@ -2288,7 +2176,7 @@ __device__ __forceinline__ void evaluate_block(const SysDev& S, const Layout& Lo
       const df* Td = reinterpret_cast<const df*>(wm.T);
       const double b = PR == LRDMC_PRECISION_DF64
                            ? df_to_double(rate_scan64(Td, P, lane, wm.pfx))
-                           : (double)warp_scan_m<float>(Td, P, lane, 0.0f, nullptr, nullptr);
+                           : (double)warp_scan_m(Td, P, lane, 0.0f, nullptr, nullptr);
       if (T)
         for (int j = lane; j < P; j += 32) T[(size_t)c * P + j] = df_to_double(Td[j]);
       if (lane == 0) {
@@ -2353,21 +2241,12 @@ void fill_df_constants(SysDev& S)
   D.ee_scale2 = split_ld((long double)bs * bs);
   D.ee_iscale = split_ld(1.0L / bs);
   D.ee_factor = split_ld(S.ee_recip ? -1.0L / bs : 1.0L);
-  // Tang's table: 2^(j/64) and ln2/64, from long double arithmetic
+  // from long double arithmetic
   const long double ln2 = logl(2.0L);
-  df c = split_ld(ln2 / kExpEntries);
+  const df c = split_ld(ln2 / kExpEntries);
   D.lexp.c_hi = c.hi;
   D.lexp.c_lo = c.lo;
   D.lexp.inv = (float)(kExpEntries / ln2);
-  c = split_ld(ln2 / 64.0L);
-  D.exp.K.ln2_64_hi = c.hi;
-  D.exp.K.ln2_64_lo = c.lo;
-  D.exp.K.inv_ln2_64 = (float)(64.0L / ln2);
-  D.exp.K.pad = 0.0f;
-  for (int j = 0; j < 64; ++j) {
-    df t = split_ld(exp2l((long double)j / 64.0L));
-    D.exp.t[j] = make_float2(t.hi, t.lo);
-  }
   long double f = 1.0L;
   for (int k = 0; k < 18; ++k) {
     if (k > 0) f *= (long double)k;
@@ -2510,7 +2389,9 @@ int accept_smem_bytes(const SysDev& S, bool caches)
   int warp = 3 * S.N + S.n_up * S.n_up + S.n_dn * S.n_dn + 12 + 12 * S.N + S.N * S.n_ao + S.N + (3 * S.N + 12) + scr;
   if (caches) warp += (S.N <= 24 ? S.N * (S.N - 1) / 2 * (S.N <= 12 ? 8 : 4) : 0) + 8 * S.N * S.n_nuc;
   warp = (warp + 1) & ~1;
-  return (int)sizeof(double) * (mask_offset(S) + kWarpsPerBlock * warp);
+  // the head stands for coefficients in three arithmetics and a 64-entry table
+  const int nc = S.n_ao * S.n_mo, head = (2 * nc + (nc + 1) / 2 + 64 + 1) & ~1;
+  return (int)sizeof(double) * (head + kWarpsPerBlock * warp);
 }
 #endif  // LRDMC_PART == 0
 
@@ -3017,25 +2898,23 @@ struct TcRowWriter {
 // Basis values chi_mu(p) of every AO (FP32, in AO order) into the row
 // writer, and the electron-nucleus Jastrow terms into jen.
 template <bool NJ>
-__device__ __forceinline__ void tc_basis_row(const SysDev& S, const float p[3], const BlockMem& bm, TcRowWriter& w,
-                                             float& jen)
+__device__ __forceinline__ void tc_basis_row(const SysDev& S, const float p[3], TcRowWriter& w, float& jen)
 {
-  typedef Ar<float> A;
   jen = 0.0f;
   for (int I = 0; I < S.n_nuc; ++I) {
     const float d[3] = {p[0] - S.D.nuc[I][0].hi, p[1] - S.D.nuc[I][1].hi, p[2] - S.D.nuc[I][2].hi};
     const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
     const float r = sqrtf(r2);
     if (S.en_b1[I] != 0.0) jen -= S.D.en_b1[I].hi * r / (S.D.en_b2.hi * r + 1.0f);
-    if (NJ) jen += nj_value_m<float>(S, 2 + S.nj_species[I], r);
+    if (NJ) jen += nj_value_m(S, 2 + S.nj_species[I], r);
     float e = 0.0f;
     for (int q = S.nuc_shell_begin[I]; q < S.nuc_shell_begin[I + 1]; ++q) {
       const ShellDev& sh = S.sh[q];
       const DfShell& dsh = S.D.sh[q];
       if (sh.kind == 0 && !sh.same_exp) e = expf(-dsh.zeta.hi * r);
-      const float Rv = radial_value_m<float>(S, sh, dsh, r, r2, e, bm);
+      const float Rv = radial_value_m(sh, dsh, r, r2, e);
       float Sv[5];
-      const int nf = solid_m<float>(sh.l, d, Sv);
+      const int nf = solid_m(sh.l, d, Sv);
       w.k = sh.ao_offset;
       for (int f = 0; f < nf; ++f) w.put(Sv[f] * Rv);
     }
@@ -3049,7 +2928,6 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
               int tile_off)
 {
   constexpr bool NJ = (PREC & 8) != 0;
-  typedef Ar<float> A;
   extern __shared__ __align__(16) double smem[];
   __shared__ __align__(8) uint64_t s_mbar;
   __shared__ uint32_t s_tmem;
@@ -3063,7 +2941,6 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
   char* Bh = Al + tileA;
   char* Bl = Bh + tileB;
   stage_coefficients<true>(S, sC);
-  const BlockMem bm = block_mem(S, sC);
   // B = C^T (orbital m, AO k), split into bfloat16 high and low parts
   for (int idx = tid; idx < kTcN * Kp; idx += blockDim.x) {
     const int m = idx / Kp, k = idx - m * Kp;
@@ -3129,12 +3006,12 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
       const float ri[3] = {wm.xd[3 * i].hi, wm.xd[3 * i + 1].hi, wm.xd[3 * i + 2].hi};
       const float p[3] = {ri[0] + h * e0, ri[1] + h * e1, ri[2] + h * e2};
       float jen;
-      tc_basis_row<NJ>(S, p, bm, w, jen);
-      jsum = jastrow_ee_m<float, NJ>(S, wm.xd, i, p) + jen;
+      tc_basis_row<NJ>(S, p, w, jen);
+      jsum = jastrow_ee_m<NJ>(S, wm.xd, i, p) + jen;
       if (G == 2) {
         const float hh = 0.5f * h;
         const float mid[3] = {ri[0] + hh * e0, ri[1] + hh * e1, ri[2] + hh * e2};
-        pm = p_weight_m<float>(S, L, mid, bm);
+        pm = p_weight_m(S, L, mid);
       }
     }
     w.finish();
@@ -3172,7 +3049,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
       if (G == 2) wgt = g ? 1.0f - pm : pm;
       float Tc = 0.0f;
       if (rho > 0.0f) Tc = wgt * (g ? L.inv2ap2_df.hi : L.inv2a2_df.hi) * rho;
-      Td[cand] = A::store(Tc);
+      Td[cand] = df_make(Tc, 0.0f);
       if (ratio) ratio[(size_t)c * P + cand] = (double)rho;
     }
     tc_fence_before();
@@ -3188,7 +3065,7 @@ k_evaluate_tc(const __grid_constant__ SysDev S, const Layout Lo, const LatDev L,
     __syncthreads();
   } else if (ok) {
     __syncwarp();
-    const float btot = warp_scan_m<float>(Td, P, lane, 0.0f, nullptr, nullptr);
+    const float btot = warp_scan_m(Td, P, lane, 0.0f, nullptr, nullptr);
     b = (double)btot;
     if (T)
       for (int j = lane; j < P; j += 32) T[(size_t)c * P + j] = (double)Td[j].hi;
