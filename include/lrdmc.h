@@ -126,9 +126,9 @@ typedef struct {
  * shared memory of one block of four walkers (positions, inverse Slater
  * matrices, rates, projected inverse columns and scratch, which grow as
  * N^2 and N n_ao) must fit in 227 KB. A system whose block fits only
- * without the double-float evaluation caches is laid out without them
- * (same results, slower double-float evaluation): e.g. 48 electrons on 8
- * centres with 42 AOs. 64 electrons with 62 AOs do not fit at all; such
+ * without the double-float evaluation caches, or of more than 40 electrons,
+ * is laid out without them (same results): e.g. 48 electrons on 8 centres
+ * with 42 AOs. 64 electrons with 62 AOs do not fit at all; such
  * systems fail with LRDMC_ERR_ARG and a message giving the size. So do
  * non-finite coordinates, Jastrow parameters or MO coefficients, a charge
  * that is not positive, and two nuclei at one point. No GPU work. */
@@ -158,9 +158,18 @@ LRDMC_API lrdmc_status lrdmc_workspace_bytes(lrdmc_system_t sys, int n_walkers, 
  * interval, e_trial the energy shift of the log-weights, recompute_every the
  * number of intervals between full recomputations of the inverse Slater
  * matrices (0 = never). stream is a cudaStream_t (NULL = default stream).
+ * Besides the workspace, a system with contracted Gaussian shells of three or
+ * more primitives holds a table of their radial parts in device memory of its
+ * own (48 bytes a cell, at most 16384 cells or 0.8 MB per shell, usually 0.2 to
+ * 0.3 MB), made by the first call on a device and freed by lrdmc_destroy. A
+ * call whose stream is being captured, or that finds no memory for the table,
+ * starts the population without it: the same results to rounding, with the
+ * primitives summed, until the next lrdmc_init_walkers.
  * Fails with LRDMC_ERR_SINGULAR if a start configuration has a singular
  * Slater matrix: two electrons of one spin on the same point, or a zero or
- * non-finite pivot in the elimination. */
+ * non-finite pivot in the elimination. An electron on a nucleus or on one of
+ * the other spin is accepted here; its local energy is not finite, which the
+ * first lrdmc_sync after a step reports as LRDMC_ERR_NONFINITE. */
 LRDMC_API lrdmc_status lrdmc_init_walkers(lrdmc_system_t sys, int n_walkers, const double* x0,
                                 uint64_t seed, double tau, double e_trial, int recompute_every,
                                 int trace_capacity, void* workspace, size_t workspace_bytes,
